@@ -86,6 +86,86 @@ __device__ __forceinline__ ds fma(ds x, ds y, ds z) {
   return ds_fast_two_sum(s, __fadd_rn(t, __fadd_rn(e, z.lo)));
 }
 
+// ---- operations of the generated integral code (os_generated.cuh), for double, float and ds
+//
+//   dot2(a, b, c, d)           a b + c d
+//   dot2_add<m>(a, b, c, d, x) a b + c d + m x, m = 1, 2, 3
+//   acc_add / acc_mac          running sums M += x, M += a b;  acc_get reads one
+//
+// In ds the products of a dot product stay unnormalised (p + e, 4 operations
+// each), the leading parts are added error-free and everything small is
+// collected before the one renormalisation: 19 operations for dot2 and 27 for
+// dot2_add<1>, against 22 and 33 for the same sum made of fma and operator+,
+// with fewer roundings.  A running sum keeps (hi, lo) unnormalised, lo
+// collecting the errors (8 operations for acc_add, 12 for acc_mac).
+
+template <class T>
+__device__ __forceinline__ T dot2(T a, T b, T c, T d) {
+  return fma(a, b, c * d);
+}
+template <int m, class T>
+__device__ __forceinline__ T dot2_add(T a, T b, T c, T d, T x) {
+  const T v = fma(a, b, c * d);
+  return m == 1 ? v + x : fma(T(m), x, v);
+}
+template <class T>
+__device__ __forceinline__ void acc_add(T& s, T x) {
+  s += x;
+}
+template <class T>
+__device__ __forceinline__ void acc_mac(T& s, T a, T b) {
+  s = fma(a, b, s);
+}
+template <class T>
+__device__ __forceinline__ T acc_get(T s) {
+  return s;
+}
+
+// x y = p + e without renormalisation
+__device__ __forceinline__ ds ds_mul_raw(ds x, ds y) {
+  const float p = __fmul_rn(x.hi, y.hi);
+  float e = __fmaf_rn(x.hi, y.hi, -p);
+  e = __fmaf_rn(x.hi, y.lo, e);
+  e = __fmaf_rn(x.lo, y.hi, e);
+  return ds_make(p, e);
+}
+
+// a + b = s + e exactly
+__device__ __forceinline__ ds ds_two_sum(float a, float b) {
+  const float s = __fadd_rn(a, b);
+  const float bb = __fsub_rn(s, a);
+  return ds_make(s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb)));
+}
+
+__device__ __forceinline__ ds dot2(ds a, ds b, ds c, ds d) {
+  const ds p = ds_mul_raw(a, b), q = ds_mul_raw(c, d);
+  const ds s = ds_two_sum(p.hi, q.hi);
+  return ds_fast_two_sum(s.hi, __fadd_rn(s.lo, __fadd_rn(p.lo, q.lo)));
+}
+
+template <int m>
+__device__ __forceinline__ ds dot2_add(ds a, ds b, ds c, ds d, ds x) {
+  if (m == 2) x = ds_make(2.0f * x.hi, 2.0f * x.lo);
+  if (m == 3) x = x * 3.0f;
+  const ds p = ds_mul_raw(a, b), q = ds_mul_raw(c, d);
+  const ds s = ds_two_sum(p.hi, q.hi);
+  const ds t = ds_two_sum(s.hi, x.hi);
+  return ds_fast_two_sum(t.hi, __fadd_rn(__fadd_rn(t.lo, s.lo), __fadd_rn(__fadd_rn(p.lo, q.lo), x.lo)));
+}
+
+__device__ __forceinline__ void acc_add(ds& s, ds x) {
+  const ds t = ds_two_sum(s.hi, x.hi);
+  s = ds_make(t.hi, __fadd_rn(s.lo, __fadd_rn(t.lo, x.lo)));
+}
+
+__device__ __forceinline__ void acc_mac(ds& s, ds a, ds b) {
+  const ds p = ds_mul_raw(a, b);
+  const ds t = ds_two_sum(s.hi, p.hi);
+  s = ds_make(t.hi, __fadd_rn(s.lo, __fadd_rn(t.lo, p.lo)));
+}
+
+__device__ __forceinline__ ds acc_get(ds s) { return ds_fast_two_sum(s.hi, s.lo); }
+
 // 1 / sqrt(t) for t > 0: the FP32 estimate refined by one Newton step in ds
 // (the relative error squares: ~1e-14).
 __device__ __forceinline__ ds ds_rsqrt(ds t) {

@@ -351,14 +351,17 @@ int build_setup_one(const snk_basis* basis, const snk_grid* grid, const snk_opti
           p.Px = (al * A[0] + be * B[0]) / z;
           p.Py = (al * A[1] + be * B[1]) / z;
           p.Pz = (al * A[2] + be * B[2]) / z;
-          p.PAx = p.Px - A[0];
-          p.PAy = p.Py - A[1];
-          p.PAz = p.Pz - A[2];
           p.pref = 2.0 * kPi / z * std::exp(-al * be / z * ab2) * s->d[k] * s->d[m];
           p.pref_far = p.pref * 0.5 * std::sqrt(kPi);
-          p.k1 = 0.5 / z;
-          p.k2 = 1.0 / z;
-          p.k3 = 1.5 / z;
+          const double sg = be / z, kp = 0.5 / z;
+          p.c10 = sg;
+          p.c20 = sg * sg;
+          p.c30 = sg * sg * sg;
+          p.c40 = (sg * sg) * (sg * sg);
+          p.c01 = kp;
+          p.c11 = sg * kp;
+          p.c21 = sg * sg * kp;
+          p.c02 = kp * kp;
           s->prims.push_back(p);
         }
       }

@@ -2,7 +2,7 @@
 // of a batch's pair list V_j and every grid point r_i of the batch,
 //
 //   Theta^n_0 = pref * F_n(zeta |P - r_i|^2)              (App. A, seed)
-//   VRR over the primitive pairs, Theta^0 contracted      (App. A, Eq. vrr)
+//   the primitive pairs contracted into scalars, one VRR   (App. A, Eq. vrr)
 //   HRR to the target block Xi_ab                          (App. A, Eq. hrr)
 //   G_{i a} += Xi_ab F_{i b},  G_{i b} += Xi_ab^T F_{i a}  (Eq. gmat, a != b)
 //
@@ -20,7 +20,15 @@
 // GB300 issues FP64 at 2 DFMA per SM per clock (1/64 of FP32), so the kernel
 // is FP64-pipe bound by construction: table lookups, index arithmetic, F loads
 // and the G atomics (L2 reductions, ~600 G/s) all hide under the DFMA stream,
-// and the generated VRR/HRR minimise the FP64 instruction count.  The mixed
+// and what counts is the number of FP64 instructions.  The primitive pairs are
+// therefore contracted before the recursion (gen_os.py): a dd primitive pair
+// costs 29 operations after its Boys functions instead of 180, and the
+// recursion's 313 run once per contracted pair.  Measured with 9 primitive
+// pairs per shell pair, against the recursion per primitive pair: FP64, 24
+// atoms and 72,000 points, 260 -> 172 ms a build (dd 33 -> 15, dp 65 -> 34, pp
+// 40 -> 27, ps 57 -> 48, ss 20); double-FP32, 96 atoms and 768,000 points, 491
+// -> 333 ms (dp 143 -> 74, dd 160 -> 122).  The FP32 tier keeps the recursion
+// per primitive pair: its rounding is what the tier's error consists of.  The mixed
 // form adds an FP32 kernel for its low-estimate pairs and a double-FP32 one
 // (ds_arith.cuh) for the rest; all three take the number of densities sharing
 // each 3c-CP block as a template parameter.
@@ -84,22 +92,26 @@ __device__ __forceinline__ void boys_seeds(double T, double pref, double pref_fa
   }
 }
 
-// Contracted Xi_ab (no component factors) of one pair at the point (cx, cy, cz).
+// Contracted Xi_ab (no component factors) of one pair at the point (cx, cy, cz);
+// A is the centre of shell a.
 template <int LA, int LB>
-__device__ __forceinline__ void pair_xi(const PairHdr& h, const PrimPair* __restrict__ prims, const double* tab,
-                                        double cx, double cy, double cz, double* xi) {
+__device__ __forceinline__ void pair_xi(const PairHdr& h, const PrimPair* __restrict__ prims,
+                                        const double* __restrict__ A, const double* tab, double cx, double cy,
+                                        double cz, double* xi) {
   using C = OsClass<LA, LB>;
-  double acc[C::NACC];
+  double M[C::NM];
 #pragma unroll
-  for (int k = 0; k < C::NACC; ++k) acc[k] = 0.0;
+  for (int k = 0; k < C::NM; ++k) M[k] = 0.0;
   for (int q = 0; q < h.pp_n; ++q) {
     const PrimPair pp = prims[h.pp_off + q];
     const double PCx = pp.Px - cx, PCy = pp.Py - cy, PCz = pp.Pz - cz;
     const double T = pp.zeta * fma(PCx, PCx, fma(PCy, PCy, PCz * PCz));
     double S[C::L + 1];
     boys_seeds<C::L>(T, pp.pref, pp.pref_far, tab, S);
-    C::vrr(S, pp.PAx, pp.PAy, pp.PAz, PCx, PCy, PCz, pp.k1, pp.k2, pp.k3, acc);
+    C::prim(S, OsCoef<double>{pp.c10, pp.c20, pp.c30, pp.c40, pp.c01, pp.c11, pp.c21, pp.c02}, M);
   }
+  double acc[C::NACC];
+  C::build(M, -h.ABx, -h.ABy, -h.ABz, cx - A[0], cy - A[1], cz - A[2], acc);
   C::hrr(acc, h.ABx, h.ABy, h.ABz, xi);
 }
 
@@ -158,7 +170,7 @@ __global__ void __launch_bounds__(kIntThreads) integral_kernel(IntegralArgs a) {
 #pragma unroll
         for (int v = 0; v < NB; ++v) fb[d][v] = F[d * dstr + (colb + v) * ldq];
       double xi[NA * NB];
-      pair_xi<LA, LB>(h, a.prims, s_tab, cx, cy, cz, xi);
+      pair_xi<LA, LB>(h, a.prims, a.shell_xyz + 3 * h.sa, s_tab, cx, cy, cz, xi);
 #pragma unroll
       for (int d = 0; d < ND; ++d)
 #pragma unroll
@@ -620,26 +632,30 @@ __device__ __forceinline__ void boys_seeds_ds(ds T, ds pref, ds pref_far, const 
 }
 
 // Contracted Xi_ab of one pair at the point c in ds arithmetic; the primitive
-// pair data are the host-split (hi, lo) copies of PrimPair (12 pairs each).
+// pair data are the host-split (hi, lo) copies of PrimPair; A is the centre of
+// shell a.
 template <int LA, int LB>
 __device__ __forceinline__ void pair_xi_ds(const PairHdr& h, const float2* __restrict__ prims,
-                                           const float2* __restrict__ ab, const float2* tab, ds cx, ds cy, ds cz,
-                                           ds* xi) {
+                                           const float2* __restrict__ ab, const float2* __restrict__ A,
+                                           const float2* tab, ds cx, ds cy, ds cz, ds* xi) {
   using C = OsClass<LA, LB>;
-  ds acc[C::NACC];
+  ds M[C::NM];
 #pragma unroll
-  for (int k = 0; k < C::NACC; ++k) acc[k] = ds_make(0.f, 0.f);
+  for (int k = 0; k < C::NM; ++k) M[k] = ds_make(0.f, 0.f);
   for (int q = 0; q < h.pp_n; ++q) {
-    const float2* pp = prims + (size_t)(h.pp_off + q) * 12;
+    const float2* pp = prims + (size_t)(h.pp_off + q) * kPrimWords;
     const ds zeta = ds_ld(pp);
     const ds PCx = ds_ld(pp + 1) - cx, PCy = ds_ld(pp + 2) - cy, PCz = ds_ld(pp + 3) - cz;
     const ds T = zeta * fma(PCx, PCx, fma(PCy, PCy, PCz * PCz));
     ds S[C::L + 1];
-    boys_seeds_ds<C::L>(T, ds_ld(pp + 7), ds_ld(pp + 8), tab, S);
-    C::vrr(S, ds_ld(pp + 4), ds_ld(pp + 5), ds_ld(pp + 6), PCx, PCy, PCz, ds_ld(pp + 9), ds_ld(pp + 10),
-           ds_ld(pp + 11), acc);
+    boys_seeds_ds<C::L>(T, ds_ld(pp + 4), ds_ld(pp + 5), tab, S);
+    C::prim(S, OsCoef<ds>{ds_ld(pp + 6), ds_ld(pp + 7), ds_ld(pp + 8), ds_ld(pp + 9), ds_ld(pp + 10), ds_ld(pp + 11),
+                          ds_ld(pp + 12), ds_ld(pp + 13)}, M);
   }
-  C::hrr(acc, ds_ld(ab), ds_ld(ab + 1), ds_ld(ab + 2), xi);
+  const ds ABx = ds_ld(ab), ABy = ds_ld(ab + 1), ABz = ds_ld(ab + 2);
+  ds acc[C::NACC];
+  C::build(M, -ABx, -ABy, -ABz, cx - ds_ld(A), cy - ds_ld(A + 1), cz - ds_ld(A + 2), acc);
+  C::hrr(acc, ABx, ABy, ABz, xi);
 }
 
 // The FP64 lists of the mixed form in ds arithmetic: same tiles, tickets,
@@ -700,13 +716,13 @@ __global__ void __launch_bounds__(kIntThreads) integral_kernel_ds(IntegralArgs a
 #pragma unroll
         for (int v = 0; v < NB; ++v) fb[d][v] = ds_from(F[d * dstr + (colb + v) * ldq]);
       ds xi[NA * NB];
-      pair_xi_ds<LA, LB>(h, a.prims_ds, a.pair_ab + 4 * (size_t)p, s_tab2, cx, cy, cz, xi);
+      pair_xi_ds<LA, LB>(h, a.prims_ds, a.pair_ab + 4 * (size_t)p, a.pair_a + 4 * (size_t)p, s_tab2, cx, cy, cz, xi);
 #pragma unroll
       for (int d = 0; d < ND; ++d)
 #pragma unroll
         for (int u = 0; u < NA; ++u)
 #pragma unroll
-          for (int v = 0; v < NB; ++v) ga[d][u] = fma(xi[u * NB + v], fb[d][v], ga[d][u]);
+          for (int v = 0; v < NB; ++v) acc_mac(ga[d][u], xi[u * NB + v], fb[d][v]);
       if (h.sa != h.sb) {
 #pragma unroll
         for (int d = 0; d < ND; ++d)
@@ -714,7 +730,7 @@ __global__ void __launch_bounds__(kIntThreads) integral_kernel_ds(IntegralArgs a
           for (int v = 0; v < NB; ++v) {
             ds g = ds_make(0.f, 0.f);
 #pragma unroll
-            for (int u = 0; u < NA; ++u) g = fma(xi[u * NB + v], fa[d][u], g);
+            for (int u = 0; u < NA; ++u) acc_mac(g, xi[u * NB + v], fa[d][u]);
             atomicAdd(G + d * dstr + (colb + v) * ldq, ds_to(g));
           }
       }
@@ -775,7 +791,7 @@ __global__ void __launch_bounds__(kIntThreads) label_kernel(IntegralArgs a, cons
         for (int u = 0; u < NA; ++u) fa[u] = F[(cola + u) * ldq];
 #pragma unroll
         for (int v = 0; v < NB; ++v) fb[v] = F[(colb + v) * ldq];
-        pair_xi<LA, LB>(h, a.prims, s_tab, cx, cy, cz, xi);
+        pair_xi<LA, LB>(h, a.prims, a.shell_xyz + 3 * h.sa, s_tab, cx, cy, cz, xi);
 #pragma unroll
         for (int u = 0; u < NA; ++u) {
           double g = 0.0;
@@ -803,15 +819,34 @@ __global__ void __launch_bounds__(kIntThreads) label_kernel(IntegralArgs a, cons
   }
 }
 
+// One shell pair's block at n points, by the recursion for every primitive pair
+// about its own centre P.  The contracted form of the builds takes P - A as
+// -sigma AB; the two differ by the rounding of P, about 1e-16 |R_p|, which only
+// shows in blocks that vanish by symmetry.  A few launches of latency, so the
+// operation count does not matter here.
 template <int LA, int LB>
-__global__ void debug_xi_kernel(const PairHdr* pair, const PrimPair* prims, const double* boys, int64_t n,
-                                const double* xyz, double* out) {
+__global__ void debug_xi_kernel(const PairHdr* pair, const PrimPair* prims, const double* shell_xyz,
+                                const double* boys, int64_t n, const double* xyz, double* out) {
   using C = OsClass<LA, LB>;
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i >= n) return;
   const double* tab = boys + (size_t)C::L * kBoysRows * kBoysCols;
+  const PairHdr h = *pair;
+  const double* A = shell_xyz + 3 * h.sa;
+  const double cx = xyz[3 * i], cy = xyz[3 * i + 1], cz = xyz[3 * i + 2];
+  double acc[C::NACC];
+#pragma unroll
+  for (int k = 0; k < C::NACC; ++k) acc[k] = 0.0;
+  for (int q = 0; q < h.pp_n; ++q) {
+    const PrimPair pp = prims[h.pp_off + q];
+    const double PCx = pp.Px - cx, PCy = pp.Py - cy, PCz = pp.Pz - cz;
+    const double T = pp.zeta * fma(PCx, PCx, fma(PCy, PCy, PCz * PCz));
+    double S[C::L + 1];
+    boys_seeds<C::L>(T, pp.pref, pp.pref_far, tab, S);
+    C::vrr(S, pp.Px - A[0], pp.Py - A[1], pp.Pz - A[2], PCx, PCy, PCz, pp.c01, 2.0 * pp.c01, 3.0 * pp.c01, acc);
+  }
   double xi[C::NA * C::NB];
-  pair_xi<LA, LB>(*pair, prims, tab, xyz[3 * i], xyz[3 * i + 1], xyz[3 * i + 2], xi);
+  C::hrr(acc, h.ABx, h.ABy, h.ABz, xi);
   for (int k = 0; k < C::NA * C::NB; ++k) out[i * C::NA * C::NB + k] = xi[k];
 }
 
@@ -934,18 +969,18 @@ cudaError_t launch_labels(cudaStream_t st, int cls, const IntegralArgs& a, int g
   return cudaGetLastError();
 }
 
-cudaError_t launch_debug_A(cudaStream_t st, int cls, const PairHdr* pair, const PrimPair* prims, const double* boys,
-                           int64_t n, const double* xyz, double* xi) {
+cudaError_t launch_debug_A(cudaStream_t st, int cls, const PairHdr* pair, const PrimPair* prims,
+                           const double* shell_xyz, const double* boys, int64_t n, const double* xyz, double* xi) {
   if (n == 0) return cudaSuccess;
   const int th = 128;
   const unsigned blocks = (unsigned)((n + th - 1) / th);
   switch (cls) {
-    case 0: debug_xi_kernel<0, 0><<<blocks, th, 0, st>>>(pair, prims, boys, n, xyz, xi); break;
-    case 1: debug_xi_kernel<1, 0><<<blocks, th, 0, st>>>(pair, prims, boys, n, xyz, xi); break;
-    case 2: debug_xi_kernel<1, 1><<<blocks, th, 0, st>>>(pair, prims, boys, n, xyz, xi); break;
-    case 3: debug_xi_kernel<2, 0><<<blocks, th, 0, st>>>(pair, prims, boys, n, xyz, xi); break;
-    case 4: debug_xi_kernel<2, 1><<<blocks, th, 0, st>>>(pair, prims, boys, n, xyz, xi); break;
-    case 5: debug_xi_kernel<2, 2><<<blocks, th, 0, st>>>(pair, prims, boys, n, xyz, xi); break;
+    case 0: debug_xi_kernel<0, 0><<<blocks, th, 0, st>>>(pair, prims, shell_xyz, boys, n, xyz, xi); break;
+    case 1: debug_xi_kernel<1, 0><<<blocks, th, 0, st>>>(pair, prims, shell_xyz, boys, n, xyz, xi); break;
+    case 2: debug_xi_kernel<1, 1><<<blocks, th, 0, st>>>(pair, prims, shell_xyz, boys, n, xyz, xi); break;
+    case 3: debug_xi_kernel<2, 0><<<blocks, th, 0, st>>>(pair, prims, shell_xyz, boys, n, xyz, xi); break;
+    case 4: debug_xi_kernel<2, 1><<<blocks, th, 0, st>>>(pair, prims, shell_xyz, boys, n, xyz, xi); break;
+    case 5: debug_xi_kernel<2, 2><<<blocks, th, 0, st>>>(pair, prims, shell_xyz, boys, n, xyz, xi); break;
     default: return cudaErrorInvalidValue;
   }
   return cudaGetLastError();
@@ -962,16 +997,15 @@ cudaError_t launch_debug_boys(cudaStream_t st, const double* boys, int64_t n, co
 // Algorithmic FP64 flops per (grid point, contracted shell pair), FMA = 2:
 // per primitive pair the T evaluation (8), the Boys seeds counted at the
 // cheaper large-T form (1 for L = 0, else 3 + 2L; the library rsqrt is not
-// counted) and the
-// generated VRR; per contracted pair the generated HRR and the G_a
-// contraction (2 NA NB).  The G_b half of off-diagonal pairs is not counted.
+// counted) and the generated contraction into the scalars; per contracted pair
+// the generated VRR and HRR and the G_a contraction (2 NA NB).  The G_b half of off-diagonal pairs is not counted.
 void class_flops(int cls, double* per_prim, double* per_pair) {
-  int vrr = 0, hrr = 0, L = 0, na = 1, nb = 1;
+  int prim = 0, pair = 0, L = 0, na = 1, nb = 1;
   switch (cls) {
 #define SNK_CASE(c, A, B)          \
   case c:                          \
-    vrr = OsClass<A, B>::VRR_FLOPS; \
-    hrr = OsClass<A, B>::HRR_FLOPS; \
+    prim = OsClass<A, B>::PRIM_FLOPS; \
+    pair = OsClass<A, B>::PAIR_FLOPS; \
     L = OsClass<A, B>::L;           \
     na = OsClass<A, B>::NA;         \
     nb = OsClass<A, B>::NB;         \
@@ -985,8 +1019,8 @@ void class_flops(int cls, double* per_prim, double* per_pair) {
 #undef SNK_CASE
   }
   const double boys = L == 0 ? 1.0 : 3.0 + 2.0 * L;
-  *per_prim = 8.0 + boys + vrr;
-  *per_pair = hrr + 2.0 * na * nb;
+  *per_prim = 8.0 + boys + prim;
+  *per_pair = pair + 2.0 * na * nb;
 }
 
 }  // namespace snk

@@ -1,24 +1,41 @@
 // Generated by gen_os.py -- do not edit.
-// Straight-line Obara-Saika VRR (App. A, Eq. vrr) and HRR (Eq. hrr) for the
-// 3c-CP integrals of one shell-pair class, with the FP64 operation counts.
+// Straight-line 3c-CP integral code of one shell-pair class: the Obara-Saika VRR
+// (App. A, Eq. vrr) with the primitive pairs contracted into scalars first (the
+// derivation is in gen_os.py), and the HRR (Eq. hrr), with the operation counts.
 #pragma once
 
 namespace snk {
 
+// sigma^i kappa^j of one primitive pair, c<i><j>; a class reads those with i + 2j <= L
+template <typename R> struct OsCoef {
+  R c10, c20, c30, c40, c01, c11, c21, c02;
+};
+
 template <int LA, int LB> struct OsClass;
 
-// class (0,0): 2 VRR statements, VRR 1 flops per primitive pair,
-// HRR 0 flops per contracted pair
+// class (0,0): 1 operations (1 flops) per primitive pair,
+// 0 (0 flops) per contracted pair
 template <> struct OsClass<0, 0> {
   static constexpr int L = 0;
+  static constexpr int NM = 1;
   static constexpr int NACC = 1;
   static constexpr int NA = 1;
   static constexpr int NB = 1;
-  static constexpr int KMAX = 0;
-  static constexpr int VRR_FLOPS = 1;
-  static constexpr int VRR_OPS = 1;
-  static constexpr int HRR_FLOPS = 0;
-  static constexpr int HRR_OPS = 0;
+  static constexpr int PRIM_FLOPS = 1;
+  static constexpr int PAIR_FLOPS = 0;
+  template <typename R, typename A>
+  __device__ static __forceinline__ void prim(const R* S, const OsCoef<R>& c, A* M) {
+    (void)c;
+    const R w0_0 = S[0];
+    acc_add(M[0], w0_0);
+  }
+  template <typename R, typename A>
+  __device__ static __forceinline__ void build(const A* M, R nABx, R nABy, R nABz, R nACx, R nACy, R nACz,
+                                               R* acc) {
+    (void)nABx; (void)nABy; (void)nABz; (void)nACx; (void)nACy; (void)nACz;
+    const R v000_000 = acc_get(M[0]);
+    acc[0] = v000_000;
+  }
   template <typename R>
   __device__ static __forceinline__ void vrr(const R* S, R PAx, R PAy, R PAz, R PCx, R PCy, R PCz,
                                              R k1, R k2, R k3, R* acc) {
@@ -34,18 +51,38 @@ template <> struct OsClass<0, 0> {
   }
 };
 
-// class (1,0): 8 VRR statements, VRR 12 flops per primitive pair,
-// HRR 0 flops per contracted pair
+// class (1,0): 3 operations (4 flops) per primitive pair,
+// 6 (9 flops) per contracted pair
 template <> struct OsClass<1, 0> {
   static constexpr int L = 1;
+  static constexpr int NM = 2;
   static constexpr int NACC = 3;
   static constexpr int NA = 3;
   static constexpr int NB = 1;
-  static constexpr int KMAX = 0;
-  static constexpr int VRR_FLOPS = 12;
-  static constexpr int VRR_OPS = 9;
-  static constexpr int HRR_FLOPS = 0;
-  static constexpr int HRR_OPS = 0;
+  static constexpr int PRIM_FLOPS = 4;
+  static constexpr int PAIR_FLOPS = 9;
+  template <typename R, typename A>
+  __device__ static __forceinline__ void prim(const R* S, const OsCoef<R>& c, A* M) {
+    (void)c;
+    const R w0_0 = S[0];
+    const R w0_1 = S[1];
+    const R w1_0 = w0_0 - w0_1;
+    acc_add(M[0], w0_1);
+    acc_mac(M[1], c.c10, w1_0);
+  }
+  template <typename R, typename A>
+  __device__ static __forceinline__ void build(const A* M, R nABx, R nABy, R nABz, R nACx, R nACy, R nACz,
+                                               R* acc) {
+    (void)nABx; (void)nABy; (void)nABz; (void)nACx; (void)nACy; (void)nACz;
+    const R v000_001 = acc_get(M[0]);
+    const R v000_100 = acc_get(M[1]);
+    const R v100_000 = dot2(nABx, v000_100, nACx, v000_001);
+    const R v010_000 = dot2(nABy, v000_100, nACy, v000_001);
+    const R v001_000 = dot2(nABz, v000_100, nACz, v000_001);
+    acc[0] = v100_000;
+    acc[1] = v010_000;
+    acc[2] = v001_000;
+  }
   template <typename R>
   __device__ static __forceinline__ void vrr(const R* S, R PAx, R PAy, R PAz, R PCx, R PCy, R PCz,
                                              R k1, R k2, R k3, R* acc) {
@@ -71,18 +108,67 @@ template <> struct OsClass<1, 0> {
   }
 };
 
-// class (1,1): 25 VRR statements, VRR 52 flops per primitive pair,
-// HRR 18 flops per contracted pair
+// class (1,1): 9 operations (13 flops) per primitive pair,
+// 42 (66 flops) per contracted pair
 template <> struct OsClass<1, 1> {
   static constexpr int L = 2;
+  static constexpr int NM = 6;
   static constexpr int NACC = 9;
   static constexpr int NA = 3;
   static constexpr int NB = 3;
-  static constexpr int KMAX = 1;
-  static constexpr int VRR_FLOPS = 52;
-  static constexpr int VRR_OPS = 37;
-  static constexpr int HRR_FLOPS = 18;
-  static constexpr int HRR_OPS = 9;
+  static constexpr int PRIM_FLOPS = 13;
+  static constexpr int PAIR_FLOPS = 66;
+  template <typename R, typename A>
+  __device__ static __forceinline__ void prim(const R* S, const OsCoef<R>& c, A* M) {
+    (void)c;
+    const R w0_0 = S[0];
+    const R w0_1 = S[1];
+    const R w0_2 = S[2];
+    const R w1_0 = w0_0 - w0_1;
+    const R w1_1 = w0_1 - w0_2;
+    const R w2_0 = w1_0 - w1_1;
+    acc_add(M[0], w0_1);
+    acc_mac(M[1], c.c10, w1_0);
+    acc_add(M[2], w0_2);
+    acc_mac(M[3], c.c10, w1_1);
+    acc_mac(M[4], c.c20, w2_0);
+    acc_mac(M[5], c.c01, w1_0);
+  }
+  template <typename R, typename A>
+  __device__ static __forceinline__ void build(const A* M, R nABx, R nABy, R nABz, R nACx, R nACy, R nACz,
+                                               R* acc) {
+    (void)nABx; (void)nABy; (void)nABz; (void)nACx; (void)nACy; (void)nACz;
+    const R v000_001 = acc_get(M[0]);
+    const R v000_002 = acc_get(M[2]);
+    const R v000_010 = acc_get(M[5]);
+    const R v000_100 = acc_get(M[1]);
+    const R v000_101 = acc_get(M[3]);
+    const R v000_200 = acc_get(M[4]);
+    const R v100_000 = dot2(nABx, v000_100, nACx, v000_001);
+    const R v100_001 = dot2(nABx, v000_101, nACx, v000_002);
+    const R v100_100 = dot2(nABx, v000_200, nACx, v000_101);
+    const R v010_000 = dot2(nABy, v000_100, nACy, v000_001);
+    const R v010_001 = dot2(nABy, v000_101, nACy, v000_002);
+    const R v010_100 = dot2(nABy, v000_200, nACy, v000_101);
+    const R v001_000 = dot2(nABz, v000_100, nACz, v000_001);
+    const R v001_001 = dot2(nABz, v000_101, nACz, v000_002);
+    const R v001_100 = dot2(nABz, v000_200, nACz, v000_101);
+    const R v200_000 = dot2_add<1>(nABx, v100_100, nACx, v100_001, v000_010);
+    const R v110_000 = dot2(nABy, v100_100, nACy, v100_001);
+    const R v101_000 = dot2(nABz, v100_100, nACz, v100_001);
+    const R v020_000 = dot2_add<1>(nABy, v010_100, nACy, v010_001, v000_010);
+    const R v011_000 = dot2(nABy, v001_100, nACy, v001_001);
+    const R v002_000 = dot2_add<1>(nABz, v001_100, nACz, v001_001, v000_010);
+    acc[0] = v100_000;
+    acc[1] = v010_000;
+    acc[2] = v001_000;
+    acc[3] = v200_000;
+    acc[4] = v110_000;
+    acc[5] = v101_000;
+    acc[6] = v020_000;
+    acc[7] = v011_000;
+    acc[8] = v002_000;
+  }
   template <typename R>
   __device__ static __forceinline__ void vrr(const R* S, R PAx, R PAy, R PAz, R PCx, R PCy, R PCz,
                                              R k1, R k2, R k3, R* acc) {
@@ -96,13 +182,12 @@ template <> struct OsClass<1, 1> {
     const R t010_1 = fma(PAy, t000_1, -PCy * t000_2);
     const R t001_0 = fma(PAz, t000_0, -PCz * t000_1);
     const R t001_1 = fma(PAz, t000_1, -PCz * t000_2);
-    const R d000_0 = t000_0 - t000_1;
-    const R t200_0 = fma(k1, d000_0, fma(PAx, t100_0, -PCx * t100_1));
+    const R t200_0 = fma(k1, t000_0 - t000_1, fma(PAx, t100_0, -PCx * t100_1));
     const R t110_0 = fma(PAx, t010_0, -PCx * t010_1);
     const R t101_0 = fma(PAx, t001_0, -PCx * t001_1);
-    const R t020_0 = fma(k1, d000_0, fma(PAy, t010_0, -PCy * t010_1));
+    const R t020_0 = fma(k1, t000_0 - t000_1, fma(PAy, t010_0, -PCy * t010_1));
     const R t011_0 = fma(PAy, t001_0, -PCy * t001_1);
-    const R t002_0 = fma(k1, d000_0, fma(PAz, t001_0, -PCz * t001_1));
+    const R t002_0 = fma(k1, t000_0 - t000_1, fma(PAz, t001_0, -PCz * t001_1));
     acc[0] += t100_0;
     acc[1] += t010_0;
     acc[2] += t001_0;
@@ -146,18 +231,57 @@ template <> struct OsClass<1, 1> {
   }
 };
 
-// class (2,0): 22 VRR statements, VRR 49 flops per primitive pair,
-// HRR 0 flops per contracted pair
+// class (2,0): 7 operations (10 flops) per primitive pair,
+// 27 (39 flops) per contracted pair
 template <> struct OsClass<2, 0> {
   static constexpr int L = 2;
+  static constexpr int NM = 4;
   static constexpr int NACC = 6;
   static constexpr int NA = 6;
   static constexpr int NB = 1;
-  static constexpr int KMAX = 1;
-  static constexpr int VRR_FLOPS = 49;
-  static constexpr int VRR_OPS = 34;
-  static constexpr int HRR_FLOPS = 0;
-  static constexpr int HRR_OPS = 0;
+  static constexpr int PRIM_FLOPS = 10;
+  static constexpr int PAIR_FLOPS = 39;
+  template <typename R, typename A>
+  __device__ static __forceinline__ void prim(const R* S, const OsCoef<R>& c, A* M) {
+    (void)c;
+    const R w0_0 = S[0];
+    const R w0_1 = S[1];
+    const R w0_2 = S[2];
+    const R w1_0 = w0_0 - w0_1;
+    const R w1_1 = w0_1 - w0_2;
+    const R w2_0 = w1_0 - w1_1;
+    acc_add(M[0], w0_2);
+    acc_mac(M[1], c.c10, w1_1);
+    acc_mac(M[2], c.c20, w2_0);
+    acc_mac(M[3], c.c01, w1_0);
+  }
+  template <typename R, typename A>
+  __device__ static __forceinline__ void build(const A* M, R nABx, R nABy, R nABz, R nACx, R nACy, R nACz,
+                                               R* acc) {
+    (void)nABx; (void)nABy; (void)nABz; (void)nACx; (void)nACy; (void)nACz;
+    const R v000_002 = acc_get(M[0]);
+    const R v000_010 = acc_get(M[3]);
+    const R v000_101 = acc_get(M[1]);
+    const R v000_200 = acc_get(M[2]);
+    const R v100_001 = dot2(nABx, v000_101, nACx, v000_002);
+    const R v100_100 = dot2(nABx, v000_200, nACx, v000_101);
+    const R v010_001 = dot2(nABy, v000_101, nACy, v000_002);
+    const R v010_100 = dot2(nABy, v000_200, nACy, v000_101);
+    const R v001_001 = dot2(nABz, v000_101, nACz, v000_002);
+    const R v001_100 = dot2(nABz, v000_200, nACz, v000_101);
+    const R v200_000 = dot2_add<1>(nABx, v100_100, nACx, v100_001, v000_010);
+    const R v110_000 = dot2(nABy, v100_100, nACy, v100_001);
+    const R v101_000 = dot2(nABz, v100_100, nACz, v100_001);
+    const R v020_000 = dot2_add<1>(nABy, v010_100, nACy, v010_001, v000_010);
+    const R v011_000 = dot2(nABy, v001_100, nACy, v001_001);
+    const R v002_000 = dot2_add<1>(nABz, v001_100, nACz, v001_001, v000_010);
+    acc[0] = v200_000;
+    acc[1] = v110_000;
+    acc[2] = v101_000;
+    acc[3] = v020_000;
+    acc[4] = v011_000;
+    acc[5] = v002_000;
+  }
   template <typename R>
   __device__ static __forceinline__ void vrr(const R* S, R PAx, R PAy, R PAz, R PCx, R PCy, R PCz,
                                              R k1, R k2, R k3, R* acc) {
@@ -171,13 +295,12 @@ template <> struct OsClass<2, 0> {
     const R t010_1 = fma(PAy, t000_1, -PCy * t000_2);
     const R t001_0 = fma(PAz, t000_0, -PCz * t000_1);
     const R t001_1 = fma(PAz, t000_1, -PCz * t000_2);
-    const R d000_0 = t000_0 - t000_1;
-    const R t200_0 = fma(k1, d000_0, fma(PAx, t100_0, -PCx * t100_1));
+    const R t200_0 = fma(k1, t000_0 - t000_1, fma(PAx, t100_0, -PCx * t100_1));
     const R t110_0 = fma(PAx, t010_0, -PCx * t010_1);
     const R t101_0 = fma(PAx, t001_0, -PCx * t001_1);
-    const R t020_0 = fma(k1, d000_0, fma(PAy, t010_0, -PCy * t010_1));
+    const R t020_0 = fma(k1, t000_0 - t000_1, fma(PAy, t010_0, -PCy * t010_1));
     const R t011_0 = fma(PAy, t001_0, -PCy * t001_1);
-    const R t002_0 = fma(k1, d000_0, fma(PAz, t001_0, -PCz * t001_1));
+    const R t002_0 = fma(k1, t000_0 - t000_1, fma(PAz, t001_0, -PCz * t001_1));
     acc[0] += t200_0;
     acc[1] += t110_0;
     acc[2] += t101_0;
@@ -203,18 +326,113 @@ template <> struct OsClass<2, 0> {
   }
 };
 
-// class (2,1): 54 VRR statements, VRR 126 flops per primitive pair,
-// HRR 36 flops per contracted pair
+// class (2,1): 16 operations (24 flops) per primitive pair,
+// 114 (177 flops) per contracted pair
 template <> struct OsClass<2, 1> {
   static constexpr int L = 3;
+  static constexpr int NM = 10;
   static constexpr int NACC = 16;
   static constexpr int NA = 6;
   static constexpr int NB = 3;
-  static constexpr int KMAX = 2;
-  static constexpr int VRR_FLOPS = 126;
-  static constexpr int VRR_OPS = 88;
-  static constexpr int HRR_FLOPS = 36;
-  static constexpr int HRR_OPS = 18;
+  static constexpr int PRIM_FLOPS = 24;
+  static constexpr int PAIR_FLOPS = 177;
+  template <typename R, typename A>
+  __device__ static __forceinline__ void prim(const R* S, const OsCoef<R>& c, A* M) {
+    (void)c;
+    const R w0_0 = S[0];
+    const R w0_1 = S[1];
+    const R w0_2 = S[2];
+    const R w0_3 = S[3];
+    const R w1_0 = w0_0 - w0_1;
+    const R w1_1 = w0_1 - w0_2;
+    const R w1_2 = w0_2 - w0_3;
+    const R w2_0 = w1_0 - w1_1;
+    const R w2_1 = w1_1 - w1_2;
+    const R w3_0 = w2_0 - w2_1;
+    acc_add(M[0], w0_2);
+    acc_mac(M[1], c.c10, w1_1);
+    acc_mac(M[2], c.c20, w2_0);
+    acc_mac(M[3], c.c01, w1_0);
+    acc_add(M[4], w0_3);
+    acc_mac(M[5], c.c10, w1_2);
+    acc_mac(M[6], c.c20, w2_1);
+    acc_mac(M[7], c.c30, w3_0);
+    acc_mac(M[8], c.c01, w1_1);
+    acc_mac(M[9], c.c11, w2_0);
+  }
+  template <typename R, typename A>
+  __device__ static __forceinline__ void build(const A* M, R nABx, R nABy, R nABz, R nACx, R nACy, R nACz,
+                                               R* acc) {
+    (void)nABx; (void)nABy; (void)nABz; (void)nACx; (void)nACy; (void)nACz;
+    const R v000_002 = acc_get(M[0]);
+    const R v000_003 = acc_get(M[4]);
+    const R v000_010 = acc_get(M[3]);
+    const R v000_011 = acc_get(M[8]);
+    const R v000_101 = acc_get(M[1]);
+    const R v000_102 = acc_get(M[5]);
+    const R v000_110 = acc_get(M[9]);
+    const R v000_200 = acc_get(M[2]);
+    const R v000_201 = acc_get(M[6]);
+    const R v000_300 = acc_get(M[7]);
+    const R v100_001 = dot2(nABx, v000_101, nACx, v000_002);
+    const R v100_002 = dot2(nABx, v000_102, nACx, v000_003);
+    const R v100_010 = dot2(nABx, v000_110, nACx, v000_011);
+    const R v100_100 = dot2(nABx, v000_200, nACx, v000_101);
+    const R v100_101 = dot2(nABx, v000_201, nACx, v000_102);
+    const R v100_200 = dot2(nABx, v000_300, nACx, v000_201);
+    const R v010_001 = dot2(nABy, v000_101, nACy, v000_002);
+    const R v010_002 = dot2(nABy, v000_102, nACy, v000_003);
+    const R v010_010 = dot2(nABy, v000_110, nACy, v000_011);
+    const R v010_100 = dot2(nABy, v000_200, nACy, v000_101);
+    const R v010_101 = dot2(nABy, v000_201, nACy, v000_102);
+    const R v010_200 = dot2(nABy, v000_300, nACy, v000_201);
+    const R v001_001 = dot2(nABz, v000_101, nACz, v000_002);
+    const R v001_002 = dot2(nABz, v000_102, nACz, v000_003);
+    const R v001_010 = dot2(nABz, v000_110, nACz, v000_011);
+    const R v001_100 = dot2(nABz, v000_200, nACz, v000_101);
+    const R v001_101 = dot2(nABz, v000_201, nACz, v000_102);
+    const R v001_200 = dot2(nABz, v000_300, nACz, v000_201);
+    const R v200_000 = dot2_add<1>(nABx, v100_100, nACx, v100_001, v000_010);
+    const R v200_001 = dot2_add<1>(nABx, v100_101, nACx, v100_002, v000_011);
+    const R v200_100 = dot2_add<1>(nABx, v100_200, nACx, v100_101, v000_110);
+    const R v110_000 = dot2(nABx, v010_100, nACx, v010_001);
+    const R v110_001 = dot2(nABx, v010_101, nACx, v010_002);
+    const R v110_100 = dot2(nABx, v010_200, nACx, v010_101);
+    const R v101_000 = dot2(nABz, v100_100, nACz, v100_001);
+    const R v020_000 = dot2_add<1>(nABy, v010_100, nACy, v010_001, v000_010);
+    const R v020_001 = dot2_add<1>(nABy, v010_101, nACy, v010_002, v000_011);
+    const R v020_100 = dot2_add<1>(nABy, v010_200, nACy, v010_101, v000_110);
+    const R v011_000 = dot2(nABz, v010_100, nACz, v010_001);
+    const R v002_000 = dot2_add<1>(nABz, v001_100, nACz, v001_001, v000_010);
+    const R v002_001 = dot2_add<1>(nABz, v001_101, nACz, v001_002, v000_011);
+    const R v002_100 = dot2_add<1>(nABz, v001_200, nACz, v001_101, v000_110);
+    const R v300_000 = dot2_add<2>(nABx, v200_100, nACx, v200_001, v100_010);
+    const R v210_000 = dot2(nABy, v200_100, nACy, v200_001);
+    const R v201_000 = dot2(nABz, v200_100, nACz, v200_001);
+    const R v120_000 = dot2(nABx, v020_100, nACx, v020_001);
+    const R v111_000 = dot2(nABz, v110_100, nACz, v110_001);
+    const R v102_000 = dot2(nABx, v002_100, nACx, v002_001);
+    const R v030_000 = dot2_add<2>(nABy, v020_100, nACy, v020_001, v010_010);
+    const R v021_000 = dot2(nABz, v020_100, nACz, v020_001);
+    const R v012_000 = dot2(nABy, v002_100, nACy, v002_001);
+    const R v003_000 = dot2_add<2>(nABz, v002_100, nACz, v002_001, v001_010);
+    acc[0] = v200_000;
+    acc[1] = v110_000;
+    acc[2] = v101_000;
+    acc[3] = v020_000;
+    acc[4] = v011_000;
+    acc[5] = v002_000;
+    acc[6] = v300_000;
+    acc[7] = v210_000;
+    acc[8] = v201_000;
+    acc[9] = v120_000;
+    acc[10] = v111_000;
+    acc[11] = v102_000;
+    acc[12] = v030_000;
+    acc[13] = v021_000;
+    acc[14] = v012_000;
+    acc[15] = v003_000;
+  }
   template <typename R>
   __device__ static __forceinline__ void vrr(const R* S, R PAx, R PAy, R PAz, R PCx, R PCy, R PCz,
                                              R k1, R k2, R k3, R* acc) {
@@ -232,31 +450,26 @@ template <> struct OsClass<2, 1> {
     const R t001_0 = fma(PAz, t000_0, -PCz * t000_1);
     const R t001_1 = fma(PAz, t000_1, -PCz * t000_2);
     const R t001_2 = fma(PAz, t000_2, -PCz * t000_3);
-    const R d000_0 = t000_0 - t000_1;
-    const R t200_0 = fma(k1, d000_0, fma(PAx, t100_0, -PCx * t100_1));
-    const R d000_1 = t000_1 - t000_2;
-    const R t200_1 = fma(k1, d000_1, fma(PAx, t100_1, -PCx * t100_2));
+    const R t200_0 = fma(k1, t000_0 - t000_1, fma(PAx, t100_0, -PCx * t100_1));
+    const R t200_1 = fma(k1, t000_1 - t000_2, fma(PAx, t100_1, -PCx * t100_2));
     const R t110_0 = fma(PAx, t010_0, -PCx * t010_1);
     const R t101_0 = fma(PAx, t001_0, -PCx * t001_1);
-    const R t020_0 = fma(k1, d000_0, fma(PAy, t010_0, -PCy * t010_1));
-    const R t020_1 = fma(k1, d000_1, fma(PAy, t010_1, -PCy * t010_2));
+    const R t020_0 = fma(k1, t000_0 - t000_1, fma(PAy, t010_0, -PCy * t010_1));
+    const R t020_1 = fma(k1, t000_1 - t000_2, fma(PAy, t010_1, -PCy * t010_2));
     const R t011_0 = fma(PAy, t001_0, -PCy * t001_1);
     const R t011_1 = fma(PAy, t001_1, -PCy * t001_2);
-    const R t002_0 = fma(k1, d000_0, fma(PAz, t001_0, -PCz * t001_1));
-    const R t002_1 = fma(k1, d000_1, fma(PAz, t001_1, -PCz * t001_2));
-    const R d100_0 = t100_0 - t100_1;
-    const R t300_0 = fma(k2, d100_0, fma(PAx, t200_0, -PCx * t200_1));
+    const R t002_0 = fma(k1, t000_0 - t000_1, fma(PAz, t001_0, -PCz * t001_1));
+    const R t002_1 = fma(k1, t000_1 - t000_2, fma(PAz, t001_1, -PCz * t001_2));
+    const R t300_0 = fma(k2, t100_0 - t100_1, fma(PAx, t200_0, -PCx * t200_1));
     const R t210_0 = fma(PAy, t200_0, -PCy * t200_1);
     const R t201_0 = fma(PAz, t200_0, -PCz * t200_1);
     const R t120_0 = fma(PAx, t020_0, -PCx * t020_1);
     const R t111_0 = fma(PAx, t011_0, -PCx * t011_1);
     const R t102_0 = fma(PAx, t002_0, -PCx * t002_1);
-    const R d010_0 = t010_0 - t010_1;
-    const R t030_0 = fma(k2, d010_0, fma(PAy, t020_0, -PCy * t020_1));
+    const R t030_0 = fma(k2, t010_0 - t010_1, fma(PAy, t020_0, -PCy * t020_1));
     const R t021_0 = fma(PAz, t020_0, -PCz * t020_1);
     const R t012_0 = fma(PAy, t002_0, -PCy * t002_1);
-    const R d001_0 = t001_0 - t001_1;
-    const R t003_0 = fma(k2, d001_0, fma(PAz, t002_0, -PCz * t002_1));
+    const R t003_0 = fma(k2, t001_0 - t001_1, fma(PAz, t002_0, -PCz * t002_1));
     acc[0] += t200_0;
     acc[1] += t110_0;
     acc[2] += t101_0;
@@ -332,18 +545,208 @@ template <> struct OsClass<2, 1> {
   }
 };
 
-// class (2,2): 106 VRR statements, VRR 259 flops per primitive pair,
-// HRR 158 flops per contracted pair
+// class (2,2): 29 operations (45 flops) per primitive pair,
+// 313 (503 flops) per contracted pair
 template <> struct OsClass<2, 2> {
   static constexpr int L = 4;
+  static constexpr int NM = 19;
   static constexpr int NACC = 31;
   static constexpr int NA = 6;
   static constexpr int NB = 6;
-  static constexpr int KMAX = 3;
-  static constexpr int VRR_FLOPS = 259;
-  static constexpr int VRR_OPS = 180;
-  static constexpr int HRR_FLOPS = 158;
-  static constexpr int HRR_OPS = 79;
+  static constexpr int PRIM_FLOPS = 45;
+  static constexpr int PAIR_FLOPS = 503;
+  template <typename R, typename A>
+  __device__ static __forceinline__ void prim(const R* S, const OsCoef<R>& c, A* M) {
+    (void)c;
+    const R w0_0 = S[0];
+    const R w0_1 = S[1];
+    const R w0_2 = S[2];
+    const R w0_3 = S[3];
+    const R w0_4 = S[4];
+    const R w1_0 = w0_0 - w0_1;
+    const R w1_1 = w0_1 - w0_2;
+    const R w1_2 = w0_2 - w0_3;
+    const R w1_3 = w0_3 - w0_4;
+    const R w2_0 = w1_0 - w1_1;
+    const R w2_1 = w1_1 - w1_2;
+    const R w2_2 = w1_2 - w1_3;
+    const R w3_0 = w2_0 - w2_1;
+    const R w3_1 = w2_1 - w2_2;
+    const R w4_0 = w3_0 - w3_1;
+    acc_add(M[0], w0_2);
+    acc_mac(M[1], c.c10, w1_1);
+    acc_mac(M[2], c.c20, w2_0);
+    acc_mac(M[3], c.c01, w1_0);
+    acc_add(M[4], w0_3);
+    acc_mac(M[5], c.c10, w1_2);
+    acc_mac(M[6], c.c20, w2_1);
+    acc_mac(M[7], c.c30, w3_0);
+    acc_mac(M[8], c.c01, w1_1);
+    acc_mac(M[9], c.c11, w2_0);
+    acc_add(M[10], w0_4);
+    acc_mac(M[11], c.c10, w1_3);
+    acc_mac(M[12], c.c20, w2_2);
+    acc_mac(M[13], c.c30, w3_1);
+    acc_mac(M[14], c.c40, w4_0);
+    acc_mac(M[15], c.c01, w1_2);
+    acc_mac(M[16], c.c11, w2_1);
+    acc_mac(M[17], c.c21, w3_0);
+    acc_mac(M[18], c.c02, w2_0);
+  }
+  template <typename R, typename A>
+  __device__ static __forceinline__ void build(const A* M, R nABx, R nABy, R nABz, R nACx, R nACy, R nACz,
+                                               R* acc) {
+    (void)nABx; (void)nABy; (void)nABz; (void)nACx; (void)nACy; (void)nACz;
+    const R v000_002 = acc_get(M[0]);
+    const R v000_003 = acc_get(M[4]);
+    const R v000_004 = acc_get(M[10]);
+    const R v000_010 = acc_get(M[3]);
+    const R v000_011 = acc_get(M[8]);
+    const R v000_012 = acc_get(M[15]);
+    const R v000_020 = acc_get(M[18]);
+    const R v000_101 = acc_get(M[1]);
+    const R v000_102 = acc_get(M[5]);
+    const R v000_103 = acc_get(M[11]);
+    const R v000_110 = acc_get(M[9]);
+    const R v000_111 = acc_get(M[16]);
+    const R v000_200 = acc_get(M[2]);
+    const R v000_201 = acc_get(M[6]);
+    const R v000_202 = acc_get(M[12]);
+    const R v000_210 = acc_get(M[17]);
+    const R v000_300 = acc_get(M[7]);
+    const R v000_301 = acc_get(M[13]);
+    const R v000_400 = acc_get(M[14]);
+    const R v100_001 = dot2(nABx, v000_101, nACx, v000_002);
+    const R v100_002 = dot2(nABx, v000_102, nACx, v000_003);
+    const R v100_003 = dot2(nABx, v000_103, nACx, v000_004);
+    const R v100_010 = dot2(nABx, v000_110, nACx, v000_011);
+    const R v100_011 = dot2(nABx, v000_111, nACx, v000_012);
+    const R v100_100 = dot2(nABx, v000_200, nACx, v000_101);
+    const R v100_101 = dot2(nABx, v000_201, nACx, v000_102);
+    const R v100_102 = dot2(nABx, v000_202, nACx, v000_103);
+    const R v100_110 = dot2(nABx, v000_210, nACx, v000_111);
+    const R v100_200 = dot2(nABx, v000_300, nACx, v000_201);
+    const R v100_201 = dot2(nABx, v000_301, nACx, v000_202);
+    const R v100_300 = dot2(nABx, v000_400, nACx, v000_301);
+    const R v010_001 = dot2(nABy, v000_101, nACy, v000_002);
+    const R v010_002 = dot2(nABy, v000_102, nACy, v000_003);
+    const R v010_003 = dot2(nABy, v000_103, nACy, v000_004);
+    const R v010_010 = dot2(nABy, v000_110, nACy, v000_011);
+    const R v010_011 = dot2(nABy, v000_111, nACy, v000_012);
+    const R v010_100 = dot2(nABy, v000_200, nACy, v000_101);
+    const R v010_101 = dot2(nABy, v000_201, nACy, v000_102);
+    const R v010_102 = dot2(nABy, v000_202, nACy, v000_103);
+    const R v010_110 = dot2(nABy, v000_210, nACy, v000_111);
+    const R v010_200 = dot2(nABy, v000_300, nACy, v000_201);
+    const R v010_201 = dot2(nABy, v000_301, nACy, v000_202);
+    const R v010_300 = dot2(nABy, v000_400, nACy, v000_301);
+    const R v001_001 = dot2(nABz, v000_101, nACz, v000_002);
+    const R v001_002 = dot2(nABz, v000_102, nACz, v000_003);
+    const R v001_003 = dot2(nABz, v000_103, nACz, v000_004);
+    const R v001_010 = dot2(nABz, v000_110, nACz, v000_011);
+    const R v001_011 = dot2(nABz, v000_111, nACz, v000_012);
+    const R v001_100 = dot2(nABz, v000_200, nACz, v000_101);
+    const R v001_101 = dot2(nABz, v000_201, nACz, v000_102);
+    const R v001_102 = dot2(nABz, v000_202, nACz, v000_103);
+    const R v001_110 = dot2(nABz, v000_210, nACz, v000_111);
+    const R v001_200 = dot2(nABz, v000_300, nACz, v000_201);
+    const R v001_201 = dot2(nABz, v000_301, nACz, v000_202);
+    const R v001_300 = dot2(nABz, v000_400, nACz, v000_301);
+    const R v200_000 = dot2_add<1>(nABx, v100_100, nACx, v100_001, v000_010);
+    const R v200_001 = dot2_add<1>(nABx, v100_101, nACx, v100_002, v000_011);
+    const R v200_002 = dot2_add<1>(nABx, v100_102, nACx, v100_003, v000_012);
+    const R v200_010 = dot2_add<1>(nABx, v100_110, nACx, v100_011, v000_020);
+    const R v200_100 = dot2_add<1>(nABx, v100_200, nACx, v100_101, v000_110);
+    const R v200_101 = dot2_add<1>(nABx, v100_201, nACx, v100_102, v000_111);
+    const R v200_200 = dot2_add<1>(nABx, v100_300, nACx, v100_201, v000_210);
+    const R v110_000 = dot2(nABx, v010_100, nACx, v010_001);
+    const R v101_000 = dot2(nABx, v001_100, nACx, v001_001);
+    const R v101_001 = dot2(nABx, v001_101, nACx, v001_002);
+    const R v101_100 = dot2(nABx, v001_200, nACx, v001_101);
+    const R v020_000 = dot2_add<1>(nABy, v010_100, nACy, v010_001, v000_010);
+    const R v020_001 = dot2_add<1>(nABy, v010_101, nACy, v010_002, v000_011);
+    const R v020_002 = dot2_add<1>(nABy, v010_102, nACy, v010_003, v000_012);
+    const R v020_010 = dot2_add<1>(nABy, v010_110, nACy, v010_011, v000_020);
+    const R v020_100 = dot2_add<1>(nABy, v010_200, nACy, v010_101, v000_110);
+    const R v020_101 = dot2_add<1>(nABy, v010_201, nACy, v010_102, v000_111);
+    const R v020_200 = dot2_add<1>(nABy, v010_300, nACy, v010_201, v000_210);
+    const R v011_000 = dot2(nABy, v001_100, nACy, v001_001);
+    const R v002_000 = dot2_add<1>(nABz, v001_100, nACz, v001_001, v000_010);
+    const R v002_001 = dot2_add<1>(nABz, v001_101, nACz, v001_002, v000_011);
+    const R v002_002 = dot2_add<1>(nABz, v001_102, nACz, v001_003, v000_012);
+    const R v002_010 = dot2_add<1>(nABz, v001_110, nACz, v001_011, v000_020);
+    const R v002_100 = dot2_add<1>(nABz, v001_200, nACz, v001_101, v000_110);
+    const R v002_101 = dot2_add<1>(nABz, v001_201, nACz, v001_102, v000_111);
+    const R v002_200 = dot2_add<1>(nABz, v001_300, nACz, v001_201, v000_210);
+    const R v300_000 = dot2_add<2>(nABx, v200_100, nACx, v200_001, v100_010);
+    const R v300_001 = dot2_add<2>(nABx, v200_101, nACx, v200_002, v100_011);
+    const R v300_100 = dot2_add<2>(nABx, v200_200, nACx, v200_101, v100_110);
+    const R v210_000 = dot2(nABy, v200_100, nACy, v200_001);
+    const R v201_000 = dot2(nABz, v200_100, nACz, v200_001);
+    const R v201_001 = dot2(nABz, v200_101, nACz, v200_002);
+    const R v201_100 = dot2(nABz, v200_200, nACz, v200_101);
+    const R v120_000 = dot2(nABx, v020_100, nACx, v020_001);
+    const R v120_001 = dot2(nABx, v020_101, nACx, v020_002);
+    const R v120_100 = dot2(nABx, v020_200, nACx, v020_101);
+    const R v111_000 = dot2(nABy, v101_100, nACy, v101_001);
+    const R v102_000 = dot2(nABx, v002_100, nACx, v002_001);
+    const R v030_000 = dot2_add<2>(nABy, v020_100, nACy, v020_001, v010_010);
+    const R v030_001 = dot2_add<2>(nABy, v020_101, nACy, v020_002, v010_011);
+    const R v030_100 = dot2_add<2>(nABy, v020_200, nACy, v020_101, v010_110);
+    const R v021_000 = dot2(nABz, v020_100, nACz, v020_001);
+    const R v012_000 = dot2(nABy, v002_100, nACy, v002_001);
+    const R v012_001 = dot2(nABy, v002_101, nACy, v002_002);
+    const R v012_100 = dot2(nABy, v002_200, nACy, v002_101);
+    const R v003_000 = dot2_add<2>(nABz, v002_100, nACz, v002_001, v001_010);
+    const R v003_001 = dot2_add<2>(nABz, v002_101, nACz, v002_002, v001_011);
+    const R v003_100 = dot2_add<2>(nABz, v002_200, nACz, v002_101, v001_110);
+    const R v400_000 = dot2_add<3>(nABx, v300_100, nACx, v300_001, v200_010);
+    const R v310_000 = dot2(nABy, v300_100, nACy, v300_001);
+    const R v301_000 = dot2(nABz, v300_100, nACz, v300_001);
+    const R v220_000 = dot2_add<1>(nABx, v120_100, nACx, v120_001, v020_010);
+    const R v211_000 = dot2(nABy, v201_100, nACy, v201_001);
+    const R v202_000 = dot2_add<1>(nABz, v201_100, nACz, v201_001, v200_010);
+    const R v130_000 = dot2(nABx, v030_100, nACx, v030_001);
+    const R v121_000 = dot2(nABz, v120_100, nACz, v120_001);
+    const R v112_000 = dot2(nABx, v012_100, nACx, v012_001);
+    const R v103_000 = dot2(nABx, v003_100, nACx, v003_001);
+    const R v040_000 = dot2_add<3>(nABy, v030_100, nACy, v030_001, v020_010);
+    const R v031_000 = dot2(nABz, v030_100, nACz, v030_001);
+    const R v022_000 = dot2_add<1>(nABy, v012_100, nACy, v012_001, v002_010);
+    const R v013_000 = dot2(nABy, v003_100, nACy, v003_001);
+    const R v004_000 = dot2_add<3>(nABz, v003_100, nACz, v003_001, v002_010);
+    acc[0] = v200_000;
+    acc[1] = v110_000;
+    acc[2] = v101_000;
+    acc[3] = v020_000;
+    acc[4] = v011_000;
+    acc[5] = v002_000;
+    acc[6] = v300_000;
+    acc[7] = v210_000;
+    acc[8] = v201_000;
+    acc[9] = v120_000;
+    acc[10] = v111_000;
+    acc[11] = v102_000;
+    acc[12] = v030_000;
+    acc[13] = v021_000;
+    acc[14] = v012_000;
+    acc[15] = v003_000;
+    acc[16] = v400_000;
+    acc[17] = v310_000;
+    acc[18] = v301_000;
+    acc[19] = v220_000;
+    acc[20] = v211_000;
+    acc[21] = v202_000;
+    acc[22] = v130_000;
+    acc[23] = v121_000;
+    acc[24] = v112_000;
+    acc[25] = v103_000;
+    acc[26] = v040_000;
+    acc[27] = v031_000;
+    acc[28] = v022_000;
+    acc[29] = v013_000;
+    acc[30] = v004_000;
+  }
   template <typename R>
   __device__ static __forceinline__ void vrr(const R* S, R PAx, R PAy, R PAz, R PCx, R PCy, R PCz,
                                              R k1, R k2, R k3, R* acc) {
@@ -365,26 +768,21 @@ template <> struct OsClass<2, 2> {
     const R t001_1 = fma(PAz, t000_1, -PCz * t000_2);
     const R t001_2 = fma(PAz, t000_2, -PCz * t000_3);
     const R t001_3 = fma(PAz, t000_3, -PCz * t000_4);
-    const R d000_0 = t000_0 - t000_1;
-    const R t200_0 = fma(k1, d000_0, fma(PAx, t100_0, -PCx * t100_1));
-    const R d000_1 = t000_1 - t000_2;
-    const R t200_1 = fma(k1, d000_1, fma(PAx, t100_1, -PCx * t100_2));
-    const R d000_2 = t000_2 - t000_3;
-    const R t200_2 = fma(k1, d000_2, fma(PAx, t100_2, -PCx * t100_3));
+    const R t200_0 = fma(k1, t000_0 - t000_1, fma(PAx, t100_0, -PCx * t100_1));
+    const R t200_1 = fma(k1, t000_1 - t000_2, fma(PAx, t100_1, -PCx * t100_2));
+    const R t200_2 = fma(k1, t000_2 - t000_3, fma(PAx, t100_2, -PCx * t100_3));
     const R t110_0 = fma(PAx, t010_0, -PCx * t010_1);
     const R t101_0 = fma(PAx, t001_0, -PCx * t001_1);
-    const R t020_0 = fma(k1, d000_0, fma(PAy, t010_0, -PCy * t010_1));
-    const R t020_1 = fma(k1, d000_1, fma(PAy, t010_1, -PCy * t010_2));
-    const R t020_2 = fma(k1, d000_2, fma(PAy, t010_2, -PCy * t010_3));
+    const R t020_0 = fma(k1, t000_0 - t000_1, fma(PAy, t010_0, -PCy * t010_1));
+    const R t020_1 = fma(k1, t000_1 - t000_2, fma(PAy, t010_1, -PCy * t010_2));
+    const R t020_2 = fma(k1, t000_2 - t000_3, fma(PAy, t010_2, -PCy * t010_3));
     const R t011_0 = fma(PAy, t001_0, -PCy * t001_1);
     const R t011_1 = fma(PAy, t001_1, -PCy * t001_2);
-    const R t002_0 = fma(k1, d000_0, fma(PAz, t001_0, -PCz * t001_1));
-    const R t002_1 = fma(k1, d000_1, fma(PAz, t001_1, -PCz * t001_2));
-    const R t002_2 = fma(k1, d000_2, fma(PAz, t001_2, -PCz * t001_3));
-    const R d100_0 = t100_0 - t100_1;
-    const R t300_0 = fma(k2, d100_0, fma(PAx, t200_0, -PCx * t200_1));
-    const R d100_1 = t100_1 - t100_2;
-    const R t300_1 = fma(k2, d100_1, fma(PAx, t200_1, -PCx * t200_2));
+    const R t002_0 = fma(k1, t000_0 - t000_1, fma(PAz, t001_0, -PCz * t001_1));
+    const R t002_1 = fma(k1, t000_1 - t000_2, fma(PAz, t001_1, -PCz * t001_2));
+    const R t002_2 = fma(k1, t000_2 - t000_3, fma(PAz, t001_2, -PCz * t001_3));
+    const R t300_0 = fma(k2, t100_0 - t100_1, fma(PAx, t200_0, -PCx * t200_1));
+    const R t300_1 = fma(k2, t100_1 - t100_2, fma(PAx, t200_1, -PCx * t200_2));
     const R t210_0 = fma(PAy, t200_0, -PCy * t200_1);
     const R t201_0 = fma(PAz, t200_0, -PCz * t200_1);
     const R t201_1 = fma(PAz, t200_1, -PCz * t200_2);
@@ -393,36 +791,29 @@ template <> struct OsClass<2, 2> {
     const R t111_0 = fma(PAx, t011_0, -PCx * t011_1);
     const R t102_0 = fma(PAx, t002_0, -PCx * t002_1);
     const R t102_1 = fma(PAx, t002_1, -PCx * t002_2);
-    const R d010_0 = t010_0 - t010_1;
-    const R t030_0 = fma(k2, d010_0, fma(PAy, t020_0, -PCy * t020_1));
-    const R d010_1 = t010_1 - t010_2;
-    const R t030_1 = fma(k2, d010_1, fma(PAy, t020_1, -PCy * t020_2));
+    const R t030_0 = fma(k2, t010_0 - t010_1, fma(PAy, t020_0, -PCy * t020_1));
+    const R t030_1 = fma(k2, t010_1 - t010_2, fma(PAy, t020_1, -PCy * t020_2));
     const R t021_0 = fma(PAz, t020_0, -PCz * t020_1);
     const R t021_1 = fma(PAz, t020_1, -PCz * t020_2);
     const R t012_0 = fma(PAy, t002_0, -PCy * t002_1);
     const R t012_1 = fma(PAy, t002_1, -PCy * t002_2);
-    const R d001_0 = t001_0 - t001_1;
-    const R t003_0 = fma(k2, d001_0, fma(PAz, t002_0, -PCz * t002_1));
-    const R d001_1 = t001_1 - t001_2;
-    const R t003_1 = fma(k2, d001_1, fma(PAz, t002_1, -PCz * t002_2));
-    const R d200_0 = t200_0 - t200_1;
-    const R t400_0 = fma(k3, d200_0, fma(PAx, t300_0, -PCx * t300_1));
+    const R t003_0 = fma(k2, t001_0 - t001_1, fma(PAz, t002_0, -PCz * t002_1));
+    const R t003_1 = fma(k2, t001_1 - t001_2, fma(PAz, t002_1, -PCz * t002_2));
+    const R t400_0 = fma(k3, t200_0 - t200_1, fma(PAx, t300_0, -PCx * t300_1));
     const R t310_0 = fma(PAy, t300_0, -PCy * t300_1);
     const R t301_0 = fma(PAz, t300_0, -PCz * t300_1);
-    const R d020_0 = t020_0 - t020_1;
-    const R t220_0 = fma(k1, d020_0, fma(PAx, t120_0, -PCx * t120_1));
+    const R t220_0 = fma(k1, t020_0 - t020_1, fma(PAx, t120_0, -PCx * t120_1));
     const R t211_0 = fma(PAy, t201_0, -PCy * t201_1);
-    const R d002_0 = t002_0 - t002_1;
-    const R t202_0 = fma(k1, d002_0, fma(PAx, t102_0, -PCx * t102_1));
+    const R t202_0 = fma(k1, t002_0 - t002_1, fma(PAx, t102_0, -PCx * t102_1));
     const R t130_0 = fma(PAx, t030_0, -PCx * t030_1);
     const R t121_0 = fma(PAx, t021_0, -PCx * t021_1);
     const R t112_0 = fma(PAx, t012_0, -PCx * t012_1);
     const R t103_0 = fma(PAx, t003_0, -PCx * t003_1);
-    const R t040_0 = fma(k3, d020_0, fma(PAy, t030_0, -PCy * t030_1));
+    const R t040_0 = fma(k3, t020_0 - t020_1, fma(PAy, t030_0, -PCy * t030_1));
     const R t031_0 = fma(PAz, t030_0, -PCz * t030_1);
-    const R t022_0 = fma(k1, d002_0, fma(PAy, t012_0, -PCy * t012_1));
+    const R t022_0 = fma(k1, t002_0 - t002_1, fma(PAy, t012_0, -PCy * t012_1));
     const R t013_0 = fma(PAy, t003_0, -PCy * t003_1);
-    const R t004_0 = fma(k3, d002_0, fma(PAz, t003_0, -PCz * t003_1));
+    const R t004_0 = fma(k3, t002_0 - t002_1, fma(PAz, t003_0, -PCz * t003_1));
     acc[0] += t200_0;
     acc[1] += t110_0;
     acc[2] += t101_0;

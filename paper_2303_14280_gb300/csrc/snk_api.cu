@@ -1284,28 +1284,31 @@ int create(int n_mol, const snk_basis* bases, const snk_grid* grids, const snk_o
            }
            SNK_CK(cp, upload(cp->pair_ab, pab, st));
            SNK_CK(cp, upload(cp->pair_a, pa, st));
-           std::vector<float> pds(s.prims.size() * 24);
+           std::vector<float> pds(s.prims.size() * 2 * kPrimWords);
            for (size_t q = 0; q < s.prims.size(); ++q) {
              const double* v = reinterpret_cast<const double*>(&s.prims[q]);
-             for (int m = 0; m < 12; ++m) {
+             for (int m = 0; m < kPrimWords; ++m) {
                const float h = (float)v[m];
-               pds[q * 24 + 2 * m] = h;
-               pds[q * 24 + 2 * m + 1] = (float)(v[m] - (double)h);
+               pds[(q * kPrimWords + m) * 2] = h;
+               pds[(q * kPrimWords + m) * 2 + 1] = (float)(v[m] - (double)h);
              }
            }
            SNK_CK(cp, upload(cp->prims_ds, pds, st));
            std::vector<float> pf(s.prims.size() * 8, 0.0f);
-           for (size_t q = 0; q < s.prims.size(); ++q) {
-             const PrimPair& P = s.prims[q];
-             float* r = &pf[q * 8];
-             r[0] = (float)P.zeta;
-             r[1] = (float)P.PAx;
-             r[2] = (float)P.PAy;
-             r[3] = (float)P.PAz;
-             r[4] = (float)P.pref;
-             r[5] = (float)P.pref_far;
-             r[6] = (float)P.k1;
-             r[7] = (float)s.prim_rel[q];
+           for (const PairHdr& h : s.pairs) {
+             const double* A = &s.center[3 * (size_t)h.sa];
+             for (int q = h.pp_off; q < h.pp_off + h.pp_n; ++q) {
+               const PrimPair& P = s.prims[q];
+               float* r = &pf[(size_t)q * 8];
+               r[0] = (float)P.zeta;
+               r[1] = (float)(P.Px - A[0]);
+               r[2] = (float)(P.Py - A[1]);
+               r[3] = (float)(P.Pz - A[2]);
+               r[4] = (float)P.pref;
+               r[5] = (float)P.pref_far;
+               r[6] = (float)P.c01;
+               r[7] = (float)s.prim_rel[q];
+             }
            }
            SNK_CK(cp, upload(cp->prims_f32, pf, st));
            SNK_CK(cp, upload(cp->boys_ds, s.boys_ds, st));
@@ -1903,7 +1906,8 @@ int snk_debug_shell_A(snk_ctx* c, int32_t sa, int32_t sb, int64_t n, const doubl
   SNK_CK(c, dxyz.ensure(3 * n));
   SNK_CK(c, dxi.ensure((size_t)n * ca * cb));
   SNK_CK(c, cudaMemcpyAsync(dxyz.p, xyz, sizeof(double) * 3 * n, cudaMemcpyHostToDevice, c->stream));
-  SNK_CK(c, launch_debug_A(c->stream, s.pair_class[p], c->pairs.p + p, c->prims.p, c->boys.p, n, dxyz.p, dxi.p));
+  SNK_CK(c, launch_debug_A(c->stream, s.pair_class[p], c->pairs.p + p, c->prims.p, c->center.p, c->boys.p, n, dxyz.p,
+                           dxi.p));
   std::vector<double> xi((size_t)n * ca * cb);
   SNK_CK(c, cudaMemcpyAsync(xi.data(), dxi.p, sizeof(double) * xi.size(), cudaMemcpyDeviceToHost, c->stream));
   SNK_CK(c, cudaStreamSynchronize(c->stream));
@@ -2088,7 +2092,8 @@ extern "C" int snk_shell_A_noalloc(snk_ctx* c, int32_t sa, int32_t sb, int64_t n
   }
   const PairHdr& h = s.pairs[p];
   const int ca = ncart(s.l[h.sa]), cb = ncart(s.l[h.sb]);
-  SNK_CK(c, launch_debug_A(c->stream, s.pair_class[p], c->pairs.p + p, c->prims.p, c->boys.p, n, xyz, scratch));
+  SNK_CK(c, launch_debug_A(c->stream, s.pair_class[p], c->pairs.p + p, c->prims.p, c->center.p, c->boys.p, n, xyz,
+                           scratch));
   const int64_t tot = n * na * nb;
   finish_shell_A_kernel<<<(unsigned)((tot + 255) / 256), 256, 0, c->stream>>>(
       scratch, n, ca, cb, h.sa != sa ? 1 : 0, c->fcomp.p + s.foff[sa], c->fcomp.p + s.foff[sb], out);

@@ -80,15 +80,16 @@ inline int class_of(int la, int lb) {  // la >= lb
   return la * (la + 1) / 2 + lb;
 }
 
-// Per primitive pair data used by the integral kernel (12 doubles).
+// Per primitive pair data used by the integral kernels.
 struct PrimPair {
   double zeta;          // zeta_a + zeta_b
   double Px, Py, Pz;    // Gaussian product centre R_p
-  double PAx, PAy, PAz; // R_p - R_a
   double pref;          // 2 pi / zeta * exp(-zeta_a zeta_b |AB|^2 / zeta) * d_a d_b
   double pref_far;      // pref * sqrt(pi) / 2  (large-T seed)
-  double k1, k2, k3;    // 1, 2, 3 times 1 / (2 zeta)
+  double c10, c20, c30, c40;  // sigma^i, sigma = zeta_b / zeta (R_p - R_a = -sigma (R_a - R_b))
+  double c01, c11, c21, c02;  // sigma^i kappa^j, kappa = 1 / (2 zeta)
 };
+constexpr int kPrimWords = sizeof(PrimPair) / sizeof(double);
 
 // Shell pair header.  The pair's primitive pairs are stored largest bound
 // first; the FP32 tier uses the first pp_n32 of them.
@@ -306,7 +307,7 @@ struct IntegralArgs {
   // mixed form: (hi, lo) float splits of the pair data, read by the FP32 and
   // ds kernels; hi_ds selects integral_kernel_ds for the FP64 lists
   const float2* boys_ds;   // (hi, lo) Boys table, nodes rounded to ds values
-  const float2* prims_ds;  // 12 (hi, lo) pairs per primitive pair, PrimPair order
+  const float2* prims_ds;  // kPrimWords (hi, lo) pairs per primitive pair, PrimPair order
   const float2* pair_ab;   // 4 per shell pair: R_a - R_b as 3 (hi, lo) pairs, padding
   // FP32 record per primitive pair (32 bytes): {zeta, PAx, PAy, PAz}, {pref, pref_far, 1/(2 zeta),
   // its bound / the shell pair's bound}
@@ -333,7 +334,7 @@ struct IntegralArgs {
 cudaError_t launch_integrals(cudaStream_t st, int cls, const IntegralArgs& a, int grid_ctas);
 int integral_max_ctas(int cls, int num_sms, bool ds, int n_dens);
 cudaError_t launch_debug_A(cudaStream_t st, int cls, const PairHdr* pair, const PrimPair* prims,
-                           const double* boys, int64_t n, const double* xyz, double* xi);
+                           const double* shell_xyz, const double* boys, int64_t n, const double* xyz, double* xi);
 cudaError_t launch_debug_boys(cudaStream_t st, const double* boys, int64_t n, const double* T,
                               int nmax, double* out);
 
