@@ -27,8 +27,7 @@
 // pairs per shell pair, against the recursion per primitive pair: FP64, 24
 // atoms and 72,000 points, 260 -> 172 ms a build (dd 33 -> 15, dp 65 -> 34, pp
 // 40 -> 27, ps 57 -> 48, ss 20); double-FP32, 96 atoms and 768,000 points, 491
-// -> 333 ms (dp 143 -> 74, dd 160 -> 122).  The FP32 tier keeps the recursion
-// per primitive pair: its rounding is what the tier's error consists of.  The mixed
+// -> 333 ms (dp 143 -> 74, dd 160 -> 122).  The mixed
 // form adds an FP32 kernel for its low-estimate pairs and a double-FP32 one
 // (ds_arith.cuh) for the rest; all three take the number of densities sharing
 // each 3c-CP block as a template parameter.
@@ -38,6 +37,7 @@
 
 #include "async_copy.cuh"
 #include "ds_arith.cuh"
+#include "f2_arith.cuh"
 #include "os_generated.cuh"
 #include "snk_internal.h"
 
@@ -46,9 +46,9 @@ namespace snk {
 namespace {
 
 constexpr int kIntThreads = kPointTile;
-constexpr int kMaxRun = 128;  // most pairs per staging step (the autotuner's largest candidate)
+constexpr int kMaxRun = kMaxPairsPerStep;
+constexpr int kPrimF4 = kPrimF32Words / 4;  // float4 per FP32 primitive record
 constexpr unsigned long long kCopyWaitNs = 2000000000ull;  // 2 s per wait on a bulk copy, then give up
-static_assert(kMaxRun == kIntThreads, "the FP32 kernel stages a step's pairs one per thread");
 constexpr long long kBoysTMaxBits = 0x4049000000000000LL;  // bit pattern of 50.0
 static_assert(kBoysTMax == 50.0, "kBoysTMaxBits encodes 50.0");
 
@@ -200,52 +200,112 @@ __global__ void __launch_bounds__(kIntThreads) integral_kernel(IntegralArgs a) {
 
 // ---------------------------------------------------------------- FP32 pairs (mixed form)
 
-// FP32 seeds S_n = pref F_n(T): 4-term Taylor about the nearest node of a
-// 0.05-spaced float table below T = 30 (|T - T_k| <= 0.025: truncation below
-// 2e-8 relative; one 16-byte row per lookup, the node fl32(k * 0.05f) formed
-// in registers), the asymptotic form above (e^{-T} < 1e-13 is below FP32
-// resolution).  e^{-T} of the downward recursion comes from the hardware
-// exponential (__expf, ~2^-21 relative).
+// FP32 seeds S_n = pref F_n(T) at two points: 4-term Taylor about the nearest
+// node of a 0.05-spaced float table below T = 30 (|T - T_k| <= 0.025:
+// truncation below 2e-8 relative; one 16-byte row per lookup, the node fl32(k *
+// 0.05f) formed in registers), the asymptotic form above (e^{-T} < 1e-13 is
+// below FP32 resolution).  e^{-T} of the downward recursion comes from the
+// hardware exponential (__expf, ~2^-21 relative).  The lookups and the
+// polynomial run per point (the two rows' coefficients sit in different
+// registers, and pairing them up costs more moves than it saves), everything
+// else on both points at once.
+// The argument is -T (the records hold -zeta): the expansion, the exponential
+// and the row index then need no negation, which has no packed form.  Both
+// forms are chosen by warp votes: the points of a warp are close together, so
+// most primitive pairs are near or far for all of them, and the branches stay
+// uniform.  Every lane of the warp must call it.
+__device__ __forceinline__ float ex2_ftz(float x) {  // 2^x, |x| < 126 here
+  float y;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+__device__ __forceinline__ float rsqrt_ftz(float x) {  // normal x only
+  float y;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+__device__ __forceinline__ float4 lds_f4(uint32_t addr) {
+  float4 v;
+  asm("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr));
+  return v;
+}
+// k = round(20 T) is formed by adding 1.5 2^23: the sum's bit pattern is
+// kRowMagic + k, so that row k of the table at the shared address tab is at
+// (tab - 16 kRowMagic) + 16 pattern (mod 2^32)
+constexpr float kRowMagicF = 12582912.0f;
+constexpr uint32_t kRowMagic = 0x4B400000u;
+
 template <int L>
-__device__ __forceinline__ void boys_seeds_f32(float T, float pref, float pref_far, const float* tab, float* S) {
-  if (T < kBoysTMaxF) {
-    static_assert(kBoysColsF == 4 && kBoysTermsF == 4, "an FP32 table row is one float4");
-    const int k = __float2int_rn(T * (1.0f / kBoysHF));
-    const float4 r = reinterpret_cast<const float4*>(tab)[k];  // F_{L+m}(T_k)/m!, m = 0..3
-    const float x = (float)k * kBoysHF - T;
-    float f = fmaf(r.w, x, r.z);
-    f = fmaf(f, x, r.y);
-    f = fmaf(f, x, r.x);
-    S[L] = pref * f;
+__device__ __forceinline__ void boys_seeds_f32(f2 nT, f2 pref, f2 pref_far, uint32_t tab_adj, f2* S) {
+  static_assert(kBoysColsF == 4 && kBoysTermsF == 4, "an FP32 table row is one float4");
+  const bool near0 = nT.v.x > -kBoysTMaxF, near1 = nT.v.y > -kBoysTMaxF;
+  const bool any_far = __any_sync(0xffffffffu, !(near0 && near1));
+  if (__any_sync(0xffffffffu, near0 || near1)) {
+    // a far point reads the last row and is replaced below
+    const f2 Tc(fmaxf(nT.v.x, -kBoysTMaxF), fmaxf(nT.v.y, -kBoysTMaxF));
+    const f2 u = fma(Tc, f2(-1.0f / kBoysHF), f2(kRowMagicF));
+    const float4 r0 = lds_f4(tab_adj + 16u * __float_as_uint(u.v.x));
+    const float4 r1 = lds_f4(tab_adj + 16u * __float_as_uint(u.v.y));
+    const f2 x = fma(u + f2(-kRowMagicF), f2(kBoysHF), Tc);  // T_k - T
+    const f2 F(fmaf(fmaf(fmaf(r0.w, x.v.x, r0.z), x.v.x, r0.y), x.v.x, r0.x),
+               fmaf(fmaf(fmaf(r1.w, x.v.y, r1.z), x.v.y, r1.y), x.v.y, r1.x));
+    S[L] = pref * F;
     if (L > 0) {
-      const float pe = pref * __expf(-T);
-      const float T2 = T + T;
+      const f2 y = Tc * f2(1.44269504088896341f);
+      const f2 pe = pref * f2(ex2_ftz(y.v.x), ex2_ftz(y.v.y));
+      const f2 T2 = Tc * f2(-2.0f);
 #pragma unroll
-      for (int n = L - 1; n >= 0; --n) S[n] = fmaf(T2, S[n + 1], pe) * (1.0f / (2 * n + 1));
+      for (int n = L - 1; n >= 0; --n) S[n] = n ? fma(T2, S[n + 1], pe) * f2(1.0f / (2 * n + 1)) : fma(T2, S[n + 1], pe);
     }
-  } else {
-    const float r = rsqrtf(T);
-    S[0] = pref_far * r;
-    if (L > 0) {
-      const float o = 0.5f * (r * r);
+  }
+  if (any_far) {
+    const f2 r(rsqrt_ftz(-nT.v.x), rsqrt_ftz(-nT.v.y));
+    f2 F = pref_far * r;
+    const f2 o = f2(0.5f) * (r * r);
 #pragma unroll
-      for (int n = 0; n < L; ++n) S[n + 1] = S[n] * ((2 * n + 1) * o);
+    for (int n = 0; n <= L; ++n) {
+      S[n] = f2(near0 ? S[n].v.x : F.v.x, near1 ? S[n].v.y : F.v.y);
+      if (n < L) F = F * (f2((float)(2 * n + 1)) * o);
     }
   }
 }
 
-// The FP32 lists of the mixed form.  Each primitive pair is a 32-byte FP32
-// record {zeta, P - A, pref, pref_far, 1/(2 zeta)}; per (pair, point) the
-// kernel forms A - r_i once from the (hi, lo) float splits of A and r_i, and
-// P - r_i = (P - A) + (A - r_i) per primitive: accurate to FP32 relative to
-// the larger of |P - A| and |A - r_i| wherever the molecule sits, which is
-// what the VRR terms PA_x Theta and PC_x Theta need.  A tile is a batch's
-// whole list on 128 points, taken in steps of a.run pairs: each step's pair
-// headers, columns, R_a - R_b and R_a are staged in shared memory (one per
-// thread, after the tile screen), and the tile's batch descriptor sits in
-// shared memory too, so that nothing of the tile stays in registers across
-// the pair loop.  Per pair each warp needs the pair's primitive records and
-// the F columns of shell b at its 32 points:
+// The FP64 value of v by integer operations: the conversion instruction runs on
+// the FP64 pipe (2 lanes per clock and SM), which the G updates kept 20-35 %
+// busy.  Below 2^-126 gives zero; infinities and NaN become numbers of 2^128
+// and more, outside the range the K accumulator accepts.
+__device__ __forceinline__ double f32_to_f64_bits(float v) {
+  const uint32_t b = __float_as_uint(v), m = b & 0x7fffffffu;
+  const uint32_t hi = (b & 0x80000000u) | ((m >> 3) + 0x38000000u);
+  return m < 0x00800000u ? 0.0 : __hiloint2double((int)hi, (int)(b << 29));
+}
+
+// The FP32 lists of the mixed form, two points per thread in packed FP32
+// arithmetic (f2).  One thread per point was bound by instruction issue (71-82
+// % of the slots, the FMA pipe 26-58 % busy): a packed instruction does both
+// points' operation in one slot, and the records, loop control and staging are
+// paid once for the two.  The FMA pipe's lane rate is the same either way.
+//
+// A tile is a batch's whole list on 128 points, a CTA of two warps per tile;
+// a lane holds the points l and l + 32 of its warp's 64, so that every F load
+// and G reduction of a warp is a full row.  The list is taken in steps of
+// a.run pairs: each step's pair headers, columns, R_a - R_b and R_a are staged
+// in shared memory (after the tile screen), and the tile's batch descriptor
+// sits in shared memory too, so that nothing of the tile stays in registers
+// across the pair loop.
+//
+// A primitive pair is a 64-byte record of scalars stored twice, {-zeta, PAx,
+// pref, pref_far, PAy, PAz, kappa, -sigma}, so that a 16-byte load gives two
+// packed operands.  Per (pair, point) the kernel forms A - r_i once from the
+// (hi, lo) float splits of A and r_i, and P - r_i = (P - A) + (A - r_i) per
+// primitive: accurate to FP32 relative to the larger of |P - A| and |A - r_i|
+// wherever the molecule sits, which is what the VRR terms PA_x Theta and PC_x
+// Theta need.  In ps and ds (f32_early) the primitive pairs are contracted
+// before the recursion as in the other kernels; the other classes keep the
+// recursion per primitive pair and with it their rounding.
+//
+// Per pair each warp needs the pair's primitive records and the F columns of
+// shell b at its 64 points:
 //   - heavy classes (L >= 2): a ring of three slots per warp, filled by TMA
 //     bulk copies that lane 0 issues two pairs ahead, each slot completing
 //     on its own mbarrier (bounded waits);
@@ -253,28 +313,45 @@ __device__ __forceinline__ void boys_seeds_f32(float T, float pref, float pref_f
 //     its records into a second shared buffer while the current pair
 //     computes (fewer instructions per pair than the ring, whose serial
 //     issue does not pay for a pair of a few primitives).
+//
+// 96 atoms and 768,000 points, ms per build before / now: ss 37.3 / 28.2, ps 87.5
+// / 70.3, pp 68.5 / 61.4, ds 66.8 / 47.1, dp 105.9 / 94.5, dd 43.3 / 39.7.  What
+// bounds it now is latency (IPC 0.5 per scheduler, fixed-latency and shared-
+// memory waits): two points double the registers, so half as many warps fit.
+constexpr int kF32Threads = kPointTile / 2;
+// CTAs per SM asked of the compiler.  96 atoms and 768,000 points, ms per build
+// without / with: ss 30.5 / 29.1, ps 75.9 / 72.5, pp 65.8 / 60.1, dp 107 / 95; ds
+// and dd lose (47.3 / 48.8 in ds).
+constexpr int f32_min_ctas(int la, int lb) {
+  return la == 0 ? 11 : la == 1 ? (lb == 0 ? 10 : 8) : lb == 1 ? 5 : 1;
+}
+
 template <int LA, int LB, int ND>
-__global__ void __launch_bounds__(kIntThreads) integral_kernel_f32(IntegralArgs a) {
+__global__ void __launch_bounds__(kF32Threads, f32_min_ctas(LA, LB)) integral_kernel_f32(IntegralArgs a) {
   using C = OsClass<LA, LB>;
   constexpr int NA = C::NA, NB = C::NB;
-  constexpr int kStage = 16;               // primitive records of a pair staged (32 float4)
+  constexpr bool kEarly = f32_early(LA, LB);  // contraction before the recursion
+  constexpr int kStage = 16;                      // primitive records of a pair staged
   constexpr bool RING = C::L >= 2;
   constexpr int kRing = 3;
-  constexpr int kRecF4 = 2 * kStage;       // float4 of records per slot
-  constexpr int kFbF4 = ND * NB * 32 / 4;  // float4 of F_b per ring slot
-  constexpr int kW = kIntThreads / 32;
+  constexpr int kRF4 = C::L == 0 ? 3 : kPrimF4;  // float4 of a record that the class reads
+  constexpr int kRecF4 = kRF4 * kStage;  // float4 of records per slot
+  constexpr int kFbF4 = ND * NB * 64 / 4;   // float4 of F_b per ring slot
+  constexpr int kW = kF32Threads / 32;
+  constexpr int kHalves = kMaxRun / kF32Threads;  // pairs a thread stages per step
   extern __shared__ __align__(16) float s_tabf[];
+  const uint32_t tab = smem_u32(s_tabf) - 16u * kRowMagic;  // see kRowMagic
   const float* gtab = a.boys_f + (size_t)C::L * kBoysRowsF * kBoysColsF;
   for (int e = threadIdx.x; e < kBoysRowsF * kBoysColsF; e += blockDim.x) s_tabf[e] = gtab[e];
   __shared__ int s_ppo[kMaxRun], s_ppn[kMaxRun], s_sa[kMaxRun], s_sb[kMaxRun], s_ca[kMaxRun], s_cb[kMaxRun];
-  __shared__ float2 s_ab[kMaxRun][3];  // (hi, lo)
-  __shared__ float2 s_A[kMaxRun][3];   // (hi, lo)
+  __shared__ float2 s_ab[kMaxRun][3];  // R_a - R_b (FP32), stored twice
+  __shared__ float2 s_A[kMaxRun][3];   // R_a as (hi, lo)
   __shared__ __align__(128) float4 s_ring[RING ? kW : 1][RING ? kRing : 1][RING ? kRecF4 + kFbF4 : 1];
   __shared__ __align__(8) uint64_t s_full[kW][kRing];
   __shared__ float4 s_pr[RING ? 1 : kW][2][RING ? 1 : kRecF4];
   __shared__ Tile s_t;
   __shared__ BatchDesc s_bd;
-  __shared__ int s_tid, s_wcnt[kW];
+  __shared__ int s_tid, s_wcnt[kHalves][kW];
   __shared__ volatile int s_abort;  // a wait ran out: the CTA stops taking work
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   if (threadIdx.x == 0) s_abort = 0;
@@ -299,22 +376,25 @@ __global__ void __launch_bounds__(kIntThreads) integral_kernel_f32(IntegralArgs 
     // the tile's list in steps of a.run pairs (block-uniform loop: every
     // thread passes the same barriers)
     for (int kb = s_t.k0; kb < s_t.k1; kb += a.run) {
-      // stage the step's pairs (one per thread, order kept); with the tile screen
-      // only those whose bound on this tile's points reaches eps_tile
-      int nrun;
-      {
-        const int r = threadIdx.x, n = min(a.run, s_t.k1 - kb);  // n <= kMaxRun = blockDim
-        int p = 0, ca = 0, cb = 0, npp_keep = 0;
-        PairHdr h{};
-        bool keep = r < n;
-        if (keep) {
-          const int* cmap = a.colmap + s_bd.cm_off - s_bd.ms0;  // indexed by global shell id
-          p = a.pairlist[kb + r];
-          h = a.pairs[p];
-          ca = cmap[h.sa];
-          cb = cmap[h.sb];
-          npp_keep = h.pp_n32;  // the leading primitive pairs the FP32 tier keeps
+      // stage the step's pairs (kHalves per thread, order kept); with the tile
+      // screen only those whose bound on this tile's points reaches eps_tile
+      const int n = min(a.run, s_t.k1 - kb);  // n <= kMaxRun
+      int pp_[kHalves], keep_n[kHalves];      // pair, primitive pairs kept (0: pair left out)
+      unsigned bal[kHalves];
+      unsigned npp_sum = 0;
+#pragma unroll
+      for (int hf = 0; hf < kHalves; ++hf) {
+        const int r = threadIdx.x + hf * kF32Threads;
+        keep_n[hf] = 0;
+        pp_[hf] = 0;
+        if (r < n) {
+          const int p = a.pairlist[kb + r];
+          const PairHdr h = a.pairs[p];
+          pp_[hf] = p;
+          int npp = h.pp_n32;  // the leading primitive pairs the FP32 tier keeps
           if (a.eps_tile > 0.f) {
+            const int* cmap = a.colmap + s_bd.cm_off - s_bd.ms0;  // indexed by global shell id
+            const int ca = cmap[h.sa], cb = cmap[h.sb];
             const float* ts = a.tsum + s_bd.ssoff + (int64_t)(s_t.i0 / kPointTile) * (s_bd.nS + 4);
             float sa = 0.f, sb = 0.f;
 #pragma unroll
@@ -334,79 +414,102 @@ __global__ void __launch_bounds__(kIntThreads) integral_kernel_f32(IntegralArgs 
             const float glob = (float)a.pbound[p], smax = fmaxf(sa, sb);
             float bnd = glob;
             if (d > 0.f) bnd = fminf(bnd, (float)a.qbound[p] / d);
-            keep = bnd * smax >= a.eps_tile;
-            if (keep) {
+            if (bnd * smax >= a.eps_tile) {
               // primitive pairs come largest bound first: leave out the tail whose
               // bounds on this tile add up to less than eps_tile
-              const float4* rec = a.prims_f32 + (size_t)h.pp_off * 2;
+              const float* share = a.prim_share + h.pp_off;
               float tail = 0.f;
-              int n = h.pp_n32;
-              while (n > 1) {
-                const float t2 = tail + rec[2 * (n - 1) + 1].w * glob * smax;
+              while (npp > 1) {
+                const float t2 = tail + share[npp - 1] * glob * smax;
                 if (t2 >= a.eps_tile) break;
                 tail = t2;
-                --n;
+                --npp;
               }
-              npp_keep = n;
+            } else {
+              npp = 0;
             }
           }
+          keep_n[hf] = npp;
+          npp_sum += (unsigned)npp;
         }
-        const unsigned bal = __ballot_sync(0xffffffffu, keep);
-        if (lane == 0) s_wcnt[wid] = __popc(bal);
-        __syncthreads();
-        int before = 0;
-        nrun = 0;
+        bal[hf] = __ballot_sync(0xffffffffu, keep_n[hf] > 0);
+        if (lane == 0) s_wcnt[hf][wid] = __popc(bal[hf]);
+      }
+      npp_sum = __reduce_add_sync(0xffffffffu, npp_sum);
+      __syncthreads();
+      int nrun = 0;
+#pragma unroll
+      for (int hf = 0; hf < kHalves; ++hf) {
+        int q = nrun + __popc(bal[hf] & ((1u << lane) - 1u));
 #pragma unroll
         for (int w = 0; w < kW; ++w) {
-          before += w < wid ? s_wcnt[w] : 0;
-          nrun += s_wcnt[w];
+          q += w < wid ? s_wcnt[hf][w] : 0;
+          nrun += s_wcnt[hf][w];
         }
-        if (keep) {
-          const int q = before + __popc(bal & ((1u << lane) - 1u));
+        if (keep_n[hf] > 0) {
+          const int p = pp_[hf];
+          const PairHdr h = a.pairs[p];
+          const int* cmap = a.colmap + s_bd.cm_off - s_bd.ms0;
           s_ppo[q] = h.pp_off;
-          s_ppn[q] = npp_keep;
+          s_ppn[q] = keep_n[hf];
           s_sa[q] = h.sa;
           s_sb[q] = h.sb;
-          s_ca[q] = ca;
-          s_cb[q] = cb;
+          s_ca[q] = cmap[h.sa];
+          s_cb[q] = cmap[h.sb];
           const float2* ab = a.pair_ab + 4 * (size_t)p;
           const float2* pa = a.pair_a + 4 * (size_t)p;
 #pragma unroll
           for (int m = 0; m < 3; ++m) {
-            s_ab[q][m] = ab[m];
+            s_ab[q][m] = make_float2(ab[m].x, ab[m].x);
             s_A[q][m] = pa[m];
           }
         }
       }
-      __syncthreads();
-      if (threadIdx.x == 0 && nrun > 0) {  // the work this step computes, for the flop counts
-        unsigned long long npp = 0;
-        for (int r = 0; r < nrun; ++r) npp += (unsigned long long)s_ppn[r];
+      if (lane == 0 && npp_sum > 0) {  // the work this step computes, for the flop counts
+        unsigned kept = 0;
+#pragma unroll
+        for (int hf = 0; hf < kHalves; ++hf) kept += __popc(bal[hf]);
         const unsigned long long pts = (unsigned long long)min(kPointTile, s_bd.q - s_t.i0);
-        atomicAdd(&a.exec[0], npp * pts);
-        atomicAdd(&a.exec[1], (unsigned long long)nrun * pts);
+        atomicAdd(&a.exec[0], (unsigned long long)npp_sum * pts);
+        atomicAdd(&a.exec[1], (unsigned long long)kept * pts);
       }
-      const int i = s_t.i0 + threadIdx.x;
-      const bool active = i < s_bd.q;  // inactive lanes of a partly active warp follow along
-      if (nrun <= 0 || s_abort || __all_sync(0xffffffffu, !active)) continue;
-      ds cx = ds_make(0.f, 0.f), cy = cx, cz = cx;
-      if (active) {
-        cx = ds_from(a.xyz[3 * (s_bd.p0 + i)]);
-        cy = ds_from(a.xyz[3 * (s_bd.p0 + i) + 1]);
-        cz = ds_from(a.xyz[3 * (s_bd.p0 + i) + 2]);
+      __syncthreads();
+      // this lane's points i and i + 32 (rows up to ldq exist, and F is zero
+      // beyond the batch's points, so a point past the end adds zero to G)
+      const int iw = s_t.i0 + 64 * wid, i = iw + lane;
+      if (nrun <= 0 || s_abort || iw >= s_bd.q) continue;
+      ds cx[2], cy[2], cz[2];
+#pragma unroll
+      for (int w = 0; w < 2; ++w) {
+        cx[w] = cy[w] = cz[w] = ds_make(0.f, 0.f);
+        if (i + 32 * w < s_bd.q) {
+          const double* c = a.xyz + 3 * (s_bd.p0 + i + 32 * w);
+          cx[w] = ds_from(c[0]);
+          cy[w] = ds_from(c[1]);
+          cz[w] = ds_from(c[2]);
+        }
       }
-      const int64_t ldq = s_bd.ldq, dstr = (int64_t)s_bd.ldq * s_bd.nS;  // density d's F / G: + d dstr
+      const int ldq = s_bd.ldq;
+      const int64_t dstr = (int64_t)s_bd.ldq * s_bd.nS;  // density d's F / G: + d dstr
       const float* F = a.ws32 + s_bd.foff32 + i;
       double* G64 = a.ws + s_bd.goff + i;
       // the FP32 contributions are added to the FP64 G with FP64 reductions;
       // each G entry of the launch has one writer (its point's thread), so
       // they land in list order and G is the same from run to run
-      auto gadd = [&](int d, int col, float v) { atomicAdd(G64 + d * dstr + col * ldq, (double)v); };
-      float ga[ND][NA], fa[ND][NA];
+      auto gadd = [&](int d, int col, f2 v) {
+        double* g = G64 + d * dstr + (int64_t)col * ldq;
+        atomicAdd(g, f32_to_f64_bits(v.v.x));
+        atomicAdd(g + 32, f32_to_f64_bits(v.v.y));
+      };
+      auto fload = [&](int d, int col) {
+        const float* f = F + d * dstr + (int64_t)col * ldq;
+        return f2(f[0], f[32]);
+      };
+      f2 ga[ND][NA], fa[ND][NA];
       int cur = -1, cola = 0;
-      // pair r at this thread's point, from its records (shared memory, or
+      // pair r at this thread's points, from its records (shared memory, or
       // global memory for more than kStage primitive pairs) and F_b
-      auto compute = [&](int r, const float4* rec, const float (&fb)[ND][NB]) {
+      auto compute = [&](int r, const float4* rec, const f2 (&fb)[ND][NB]) {
         const int sa = s_sa[r];
         if (sa != cur) {
           if (cur >= 0) {
@@ -421,58 +524,82 @@ __global__ void __launch_bounds__(kIntThreads) integral_kernel_f32(IntegralArgs 
           for (int d = 0; d < ND; ++d)
 #pragma unroll
             for (int u = 0; u < NA; ++u) {
-              ga[d][u] = 0.f;
-              fa[d][u] = F[d * dstr + (cola + u) * ldq];
+              ga[d][u] = f2(0.f);
+              fa[d][u] = fload(d, cola + u);
             }
         }
         // A - r_i, once per pair and point
-        const float ACx = (s_A[r][0].x - cx.hi) + (s_A[r][0].y - cx.lo);
-        const float ACy = (s_A[r][1].x - cy.hi) + (s_A[r][1].y - cy.lo);
-        const float ACz = (s_A[r][2].x - cz.hi) + (s_A[r][2].y - cz.lo);
-        float acc[C::NACC];
+        auto ac = [&](int m, const ds* c) {
+          const float2 A = s_A[r][m];
+          return f2((A.x - c[0].hi) + (A.y - c[0].lo), (A.x - c[1].hi) + (A.y - c[1].lo));
+        };
+        const f2 ACx = ac(0, cx), ACy = ac(1, cy), ACz = ac(2, cz);
+        const f2 ABx(s_ab[r][0]), ABy(s_ab[r][1]), ABz(s_ab[r][2]);
+        f2 acc[C::NACC], M[C::NM];
+        if (kEarly) {
 #pragma unroll
-        for (int u = 0; u < C::NACC; ++u) acc[u] = 0.f;
-        auto prim = [&](float4 r0, float4 r1) {
-          const float PCx = r0.y + ACx, PCy = r0.z + ACy, PCz = r0.w + ACz;
-          const float T = r0.x * fmaf(PCx, PCx, fmaf(PCy, PCy, PCz * PCz));
-          float S[C::L + 1];
-          boys_seeds_f32<C::L>(T, r1.x, r1.y, s_tabf, S);
-          C::vrr(S, r0.y, r0.z, r0.w, PCx, PCy, PCz, r1.z, 2.0f * r1.z, 3.0f * r1.z, acc);
+          for (int u = 0; u < C::NM; ++u) M[u] = f2(0.f);
+        } else {
+#pragma unroll
+          for (int u = 0; u < C::NACC; ++u) acc[u] = f2(0.f);
+        }
+        auto prim = [&](const float4* q) {
+          const float4 r0 = q[0], r1 = q[1], r2 = q[2];
+          const f2 nz(r0.x, r0.y), PAx(r0.z, r0.w), PAy(r2.x, r2.y), PAz(r2.z, r2.w);
+          const f2 PCx = PAx + ACx, PCy = PAy + ACy, PCz = PAz + ACz;
+          f2 S[C::L + 1];
+          boys_seeds_f32<C::L>(nz * fma(PCx, PCx, fma(PCy, PCy, PCz * PCz)), f2(r1.x, r1.y), f2(r1.z, r1.w), tab, S);
+          f2 kp(0.f), nsg(0.f);
+          if (C::L > 0) {
+            const float4 r3 = q[3];
+            kp = f2(r3.x, r3.y);
+            nsg = f2(r3.z, r3.w);
+          }
+          if (kEarly) {
+            OsCoef<f2> c;
+            c.c10 = nsg;
+            c.c20 = nsg * nsg;
+            c.c01 = kp;
+            C::prim(S, c, M);
+          } else {
+            C::vrr(S, PAx, PAy, PAz, PCx, PCy, PCz, kp, f2(2.0f) * kp, f2(3.0f) * kp, acc);
+          }
         };
         const int ppn = s_ppn[r];
         if (ppn <= kStage) {
-#pragma unroll 2
-          for (int q = 0; q < ppn; ++q) prim(rec[2 * q], rec[2 * q + 1]);
+#pragma unroll 1
+          for (int q = 0; q < ppn; ++q) prim(rec + kRF4 * q);
         } else {  // more primitive pairs than staged: global memory
-          const float4* pp = a.prims_f32 + (size_t)s_ppo[r] * 2;
-          for (int q = 0; q < ppn; ++q) prim(pp[2 * q], pp[2 * q + 1]);
+          const float4* pp = a.prims_f32 + (size_t)s_ppo[r] * kPrimF4;
+          for (int q = 0; q < ppn; ++q) prim(pp + kPrimF4 * q);
         }
-        float xi[NA * NB];
-        C::hrr(acc, s_ab[r][0].x, s_ab[r][1].x, s_ab[r][2].x, xi);
+        if (kEarly) C::build(M, ABx, ABy, ABz, -ACx, -ACy, -ACz, acc);  // powers of -sigma in M
+        f2 xi[NA * NB];
+        C::hrr(acc, ABx, ABy, ABz, xi);
 #pragma unroll
         for (int d = 0; d < ND; ++d)
 #pragma unroll
           for (int u = 0; u < NA; ++u)
 #pragma unroll
-            for (int v = 0; v < NB; ++v) ga[d][u] = fmaf(xi[u * NB + v], fb[d][v], ga[d][u]);
+            for (int v = 0; v < NB; ++v) ga[d][u] = fma(xi[u * NB + v], fb[d][v], ga[d][u]);
         if (sa != s_sb[r]) {
           const int colb = s_cb[r];
 #pragma unroll
           for (int d = 0; d < ND; ++d)
 #pragma unroll
             for (int v = 0; v < NB; ++v) {
-              float g = 0.f;
+              f2 g(0.f);
 #pragma unroll
-              for (int u = 0; u < NA; ++u) g = fmaf(xi[u * NB + v], fa[d][u], g);
+              for (int u = 0; u < NA; ++u) g = fma(xi[u * NB + v], fa[d][u], g);
               gadd(d, colb + v, g);
             }
         }
       };
       if constexpr (RING) {
-        // the warp's 32 points of every F column: 128 contiguous, 16-byte
+        // the warp's 64 points of every F column: 256 contiguous, 16-byte
         // aligned bytes (foff32, ldq and i0 are multiples of 128 floats, and
         // the columns are ldq >= i0 + 128 long)
-        const float* Fw = a.ws32 + s_bd.foff32 + s_t.i0 + 32 * wid;
+        const float* Fw = a.ws32 + s_bd.foff32 + iw;
         // pair r into the next slot: its records (at most kStage primitive
         // pairs; longer contractions are read from global memory) and its
         // F_b columns, one bulk copy each, all on the slot's barrier.  The
@@ -483,17 +610,17 @@ __global__ void __launch_bounds__(kIntThreads) integral_kernel_f32(IntegralArgs 
             const int sl = prod % kRing;
             uint64_t* bar = &s_full[wid][sl];
             const int ppn = s_ppn[r];
-            const uint32_t rec_bytes = ppn <= kStage ? 32u * (uint32_t)ppn : 0u;
+            const uint32_t rec_bytes = ppn <= kStage ? 16u * kPrimF4 * (uint32_t)ppn : 0u;
             fence_proxy_async_smem();
-            mbar_expect_tx(bar, rec_bytes + ND * NB * 128);
-            if (rec_bytes) bulk_copy(s_ring[wid][sl], a.prims_f32 + (size_t)s_ppo[r] * 2, rec_bytes, bar);
+            mbar_expect_tx(bar, rec_bytes + ND * NB * 256);
+            if (rec_bytes) bulk_copy(s_ring[wid][sl], a.prims_f32 + (size_t)s_ppo[r] * kPrimF4, rec_bytes, bar);
             float* fdst = reinterpret_cast<float*>(s_ring[wid][sl] + kRecF4);
             const int cb = s_cb[r];
 #pragma unroll
             for (int d = 0; d < ND; ++d)
 #pragma unroll
               for (int v = 0; v < NB; ++v)
-                bulk_copy(fdst + (d * NB + v) * 32, Fw + d * dstr + (int64_t)(cb + v) * ldq, 128, bar);
+                bulk_copy(fdst + (d * NB + v) * 64, Fw + d * dstr + (int64_t)(cb + v) * ldq, 256, bar);
           }
           ++prod;
         };
@@ -512,59 +639,59 @@ __global__ void __launch_bounds__(kIntThreads) integral_kernel_f32(IntegralArgs 
             cons = prod;
             break;
           }
-          if (active) {
-            const float* fsl = reinterpret_cast<const float*>(s_ring[wid][sl] + kRecF4);
-            float fb[ND][NB];
+          const float* fsl = reinterpret_cast<const float*>(s_ring[wid][sl] + kRecF4);
+          f2 fb[ND][NB];
 #pragma unroll
-            for (int d = 0; d < ND; ++d)
+          for (int d = 0; d < ND; ++d)
 #pragma unroll
-              for (int v = 0; v < NB; ++v) fb[d][v] = fsl[(d * NB + v) * 32 + lane];
-            compute(r, s_ring[wid][sl], fb);
-          }
+            for (int v = 0; v < NB; ++v) fb[d][v] = f2(fsl[(d * NB + v) * 64 + lane], fsl[(d * NB + v) * 64 + 32 + lane]);
+          compute(r, s_ring[wid][sl], fb);
           __syncwarp();  // every lane is done with slot sl: it takes pair r + kRing
           if (r + kRing < nrun) issue(r + kRing);
         }
       } else {
-        {  // the first pair's records
-          const int n2 = min(s_ppn[0], kStage) * 2;
-          const float4* src = a.prims_f32 + (size_t)s_ppo[0] * 2;
-          if (lane < n2) s_pr[RING ? 0 : wid][0][lane] = src[lane];
+        constexpr int kRecL = (kRecF4 + 31) / 32;  // float4 of a pair's records per lane
+        auto rec_load = [&](int r, float4 (&pre)[kRecL]) {
+          const int n4 = min(s_ppn[r], kStage) * kRF4;
+          const float4* src = a.prims_f32 + (size_t)s_ppo[r] * kPrimF4;
+#pragma unroll
+          for (int m = 0; m < kRecL; ++m) {
+            const int e = lane + 32 * m;
+            if (e < n4) pre[m] = src[(e / kRF4) * kPrimF4 + e % kRF4];
+          }
+          return n4;
+        };
+        auto rec_store = [&](int buf, int n4, const float4 (&pre)[kRecL]) {
+#pragma unroll
+          for (int m = 0; m < kRecL; ++m)
+            if (lane + 32 * m < n4) s_pr[RING ? 0 : wid][buf][lane + 32 * m] = pre[m];
           __syncwarp();
-        }
-        float fn[ND][NB];
+        };
+        float4 pre[kRecL];
+        rec_store(0, rec_load(0, pre), pre);
+        f2 fn[ND][NB];
 #pragma unroll
         for (int d = 0; d < ND; ++d)
 #pragma unroll
-          for (int v = 0; v < NB; ++v) fn[d][v] = active ? F[d * dstr + (s_cb[0] + v) * ldq] : 0.f;
+          for (int v = 0; v < NB; ++v) fn[d][v] = fload(d, s_cb[0] + v);
         for (int r = 0; r < nrun; ++r) {
           // the next pair's records and F are in flight while this pair computes
-          float4 pre = make_float4(0.f, 0.f, 0.f, 0.f);
-          int n2n = 0;
-          if (r + 1 < nrun) {
-            n2n = min(s_ppn[r + 1], kStage) * 2;
-            const float4* src = a.prims_f32 + (size_t)s_ppo[r + 1] * 2;
-            if (lane < n2n) pre = src[lane];
-          }
-          float fb[ND][NB];
+          const int n4 = r + 1 < nrun ? rec_load(r + 1, pre) : 0;
+          f2 fb[ND][NB];
 #pragma unroll
           for (int d = 0; d < ND; ++d)
 #pragma unroll
-            for (int v = 0; v < NB; ++v) fb[d][v] = fn[d][v];
-          if (active && r + 1 < nrun) {
-            const int cn = s_cb[r + 1];
-#pragma unroll
-            for (int d = 0; d < ND; ++d)
-#pragma unroll
-              for (int v = 0; v < NB; ++v) fn[d][v] = F[d * dstr + (cn + v) * ldq];
-          }
-          if (active) compute(r, s_pr[RING ? 0 : wid][r & 1], fb);
+            for (int v = 0; v < NB; ++v) {
+              fb[d][v] = fn[d][v];
+              if (r + 1 < nrun) fn[d][v] = fload(d, s_cb[r + 1] + v);
+            }
+          compute(r, s_pr[RING ? 0 : wid][r & 1], fb);
           // every lane is past its reads of the other buffer (the previous
           // iteration's closing __syncwarp), so it can take the next records
-          if (lane < n2n) s_pr[RING ? 0 : wid][(r + 1) & 1][lane] = pre;
-          __syncwarp();
+          rec_store((r + 1) & 1, n4, pre);
         }
       }
-      if (active && cur >= 0) {
+      if (cur >= 0) {
 #pragma unroll
         for (int d = 0; d < ND; ++d)
 #pragma unroll
@@ -876,16 +1003,17 @@ constexpr size_t kSmem32 = sizeof(float) * kBoysRowsF * kBoysColsF;
 // list < kNumClasses: FP64 kernel of that class; otherwise the FP32 kernel of
 // class list - kNumClasses.
 template <class K>
-cudaError_t launch_kernel(K kernel, size_t smem, cudaStream_t st, const IntegralArgs& a, int grid) {
+cudaError_t launch_kernel(K kernel, size_t smem, cudaStream_t st, const IntegralArgs& a, int grid,
+                          int threads = kIntThreads) {
   cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  kernel<<<grid, kIntThreads, smem, st>>>(a);
+  kernel<<<grid, threads, smem, st>>>(a);
   return cudaGetLastError();
 }
 
 template <int LA, int LB, int ND>
 cudaError_t launch_class_nd(cudaStream_t st, bool f32, const IntegralArgs& a, int grid) {
-  if (f32) return launch_kernel(integral_kernel_f32<LA, LB, ND>, kSmem32, st, a, grid);
+  if (f32) return launch_kernel(integral_kernel_f32<LA, LB, ND>, kSmem32, st, a, grid, kF32Threads);
   if (a.hi_ds) return launch_kernel(integral_kernel_ds<LA, LB, ND>, kSmem64, st, a, grid);
   return launch_kernel(integral_kernel<LA, LB, ND>, kSmem64, st, a, grid);
 }
@@ -896,17 +1024,17 @@ cudaError_t launch_class(cudaStream_t st, bool f32, const IntegralArgs& a, int g
 }
 
 template <class K>
-int ctas_for(K kernel, size_t smem, int num_sms) {
+int ctas_for(K kernel, size_t smem, int num_sms, int threads = kIntThreads) {
   cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   int per_sm = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kIntThreads, smem) != cudaSuccess || per_sm < 1)
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, smem) != cudaSuccess || per_sm < 1)
     per_sm = 1;
   return per_sm * num_sms;
 }
 
 template <int LA, int LB, int ND>
 int max_ctas_nd(bool f32, bool ds, int num_sms) {
-  return f32  ? ctas_for(integral_kernel_f32<LA, LB, ND>, kSmem32, num_sms)
+  return f32  ? ctas_for(integral_kernel_f32<LA, LB, ND>, kSmem32, num_sms, kF32Threads)
          : ds ? ctas_for(integral_kernel_ds<LA, LB, ND>, kSmem64, num_sms)
               : ctas_for(integral_kernel<LA, LB, ND>, kSmem64, num_sms);
 }

@@ -94,8 +94,8 @@ struct DevBuf {
 
 // pairs per integral tile for each class (cheap classes take longer runs);
 // the autotuner replaces these per list
-constexpr int kDefaultStep = 128;  // pairs staged per step of the FP32 kernel, before autotuning
-constexpr int kRunCandidates[] = {2, 4, 8, 16, 32, 64, 128};
+constexpr int kDefaultStep = kMaxPairsPerStep;  // pairs staged per step of the FP32 kernel, before autotuning
+constexpr int kRunCandidates[] = {2, 4, 8, 16, 32, 64};
 // per chunk: collocation, F operands, F high tier, F rest, integral lists, K operands, K high tier, K rest
 constexpr int kPhaseEvents = 7 + kNumLists;
 
@@ -115,7 +115,7 @@ struct snk_ctx {
   // geometry (device)
   DevBuf<int> l, poff, nprim, foff, fshell, bshell, bshell_col, xfunc;
   DevBuf<double> center, exps, d, fcomp, xyz, w, boys, bound, qbound, bcenter, bradius, phit_f, phit_b;
-  DevBuf<float> boys_f, boys_ds, prims_ds, pair_ab, pair_a, prims_f32;  // mixed form: FP32 and (hi, lo) copies
+  DevBuf<float> boys_f, boys_ds, prims_ds, pair_ab, pair_a, prims_f32, prim_share;  // mixed form: FP32 and (hi, lo) copies
   DevBuf<PairHdr> pairs;
   DevBuf<PrimPair> prims;
   DevBuf<MolDesc> mols;
@@ -212,7 +212,7 @@ struct snk_ctx {
     f(l), f(poff), f(nprim), f(foff), f(fshell), f(bshell), f(bshell_col), f(xfunc);
     f(center), f(exps), f(d), f(fcomp), f(xyz), f(w), f(boys), f(bound), f(qbound), f(bcenter), f(bradius);
     f(phit_f), f(phit_b);
-    f(boys_f), f(boys_ds), f(prims_ds), f(pair_ab), f(pair_a), f(prims_f32);
+    f(boys_f), f(boys_ds), f(prims_ds), f(pair_ab), f(pair_a), f(prims_f32), f(prim_share);
     f(pairs), f(prims), f(mols), f(mlp_w), f(shell_feat), f(keep);
     f(P), f(Pscr), f(ft), f(sym), f(Khat), f(K), f(P2);
     f(counts), f(list), f(list2), f(sfunc), f(colmap), f(tickets), f(ppcounts), f(sflag), f(list_off), f(tstart);
@@ -368,8 +368,8 @@ int make_tiles(snk_ctx* c, cudaStream_t st) {
     for (int k = 0; k < kNumLists; ++k) {
       ch.tile_off[k] = tot;
       const int run = c->run[k];
-      if (run < 1 || run > 128)  // the FP32 kernel stages at most 128 pairs per step
-        return fail(c, SNK_ERR_INVALID_ARG, "pairs per step outside 1..128");
+      if (run < 1 || run > kMaxPairsPerStep)
+        return fail(c, SNK_ERR_INVALID_ARG, "pairs per step outside 1.." + std::to_string(kMaxPairsPerStep));
       order.resize(ch.b1 - ch.b0);
       cost.resize(ch.b1 - ch.b0);
       for (int t = ch.b0; t < ch.b1; ++t) {
@@ -865,6 +865,7 @@ IntegralArgs integral_args(snk_ctx* c, size_t ci, int k) {
   a.prims_ds = reinterpret_cast<const float2*>(c->prims_ds.p);
   a.pair_ab = reinterpret_cast<const float2*>(c->pair_ab.p);
   a.prims_f32 = reinterpret_cast<const float4*>(c->prims_f32.p);
+  a.prim_share = c->prim_share.p;
   a.pair_a = reinterpret_cast<const float2*>(c->pair_a.p);
   a.hi_ds = (c->opt.precision == SNK_PREC_MIXED && c->opt.ds_integrals) ? 1 : 0;
   a.tsum = c->tsum.p;
@@ -1294,23 +1295,18 @@ int create(int n_mol, const snk_basis* bases, const snk_grid* grids, const snk_o
              }
            }
            SNK_CK(cp, upload(cp->prims_ds, pds, st));
-           std::vector<float> pf(s.prims.size() * 8, 0.0f);
+           std::vector<float> pf(s.prims.size() * kPrimF32Words, 0.0f);
            for (const PairHdr& h : s.pairs) {
              const double* A = &s.center[3 * (size_t)h.sa];
              for (int q = h.pp_off; q < h.pp_off + h.pp_n; ++q) {
                const PrimPair& P = s.prims[q];
-               float* r = &pf[(size_t)q * 8];
-               r[0] = (float)P.zeta;
-               r[1] = (float)(P.Px - A[0]);
-               r[2] = (float)(P.Py - A[1]);
-               r[3] = (float)(P.Pz - A[2]);
-               r[4] = (float)P.pref;
-               r[5] = (float)P.pref_far;
-               r[6] = (float)P.c01;
-               r[7] = (float)s.prim_rel[q];
+               const double v[kPrimF32Words / 2] = {-P.zeta,    P.Px - A[0], P.pref, P.pref_far,
+                                                    P.Py - A[1], P.Pz - A[2], P.c01,  -P.c10};
+               for (int m = 0; m < kPrimF32Words; ++m) pf[(size_t)q * kPrimF32Words + m] = (float)v[m / 2];
              }
            }
            SNK_CK(cp, upload(cp->prims_f32, pf, st));
+           SNK_CK(cp, upload(cp->prim_share, std::vector<float>(s.prim_rel.begin(), s.prim_rel.end()), st));
            SNK_CK(cp, upload(cp->boys_ds, s.boys_ds, st));
          }
          SNK_CK(cp, upload(cp->xyz, s.xyz, st));

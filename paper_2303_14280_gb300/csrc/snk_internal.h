@@ -15,6 +15,7 @@ constexpr int kLMax = 2;
 constexpr int kNumClasses = 6;  // (0,0) (1,0) (1,1) (2,0) (2,1) (2,2)
 constexpr int kNumLists = 2 * kNumClasses;  // per batch: FP64 lists, then FP32 lists
 constexpr int kPointTile = 128;  // grid points per integral tile (one per thread)
+constexpr int kMaxPairsPerStep = 64;  // pairs the FP32 integral kernel stages at once
 constexpr int kLdqAlign = 128;   // leading-dimension padding of batch matrices
 
 // K-hat accumulator: every entry is a pair of 64-bit integers (hi, lo) worth
@@ -90,6 +91,14 @@ struct PrimPair {
   double c01, c11, c21, c02;  // sigma^i kappa^j, kappa = 1 / (2 zeta)
 };
 constexpr int kPrimWords = sizeof(PrimPair) / sizeof(double);
+constexpr int kPrimF32Words = 16;  // floats per primitive record of the FP32 tier
+// Classes whose FP32-tier primitive pairs are contracted before the recursion.
+// With l_b > 0 the horizontal recursion cancels powers of P - A, the rounding of
+// the recursion is most of the tier's error, and contracting first would move
+// K's largest deviation by up to 2.7e-8 (pp), 2.4e-8 (dp) and 1.6e-7 (dd) of its
+// rms at 96 atoms, for 61 -> 50, 95 -> 63 and no gain in ms; ps and ds move it by
+// less than 5e-9.  In ss there is nothing to contract.
+constexpr bool f32_early(int la, int lb) { return la > 0 && lb == 0; }
 
 // Shell pair header.  The pair's primitive pairs are stored largest bound
 // first; the FP32 tier uses the first pp_n32 of them.
@@ -309,9 +318,10 @@ struct IntegralArgs {
   const float2* boys_ds;   // (hi, lo) Boys table, nodes rounded to ds values
   const float2* prims_ds;  // kPrimWords (hi, lo) pairs per primitive pair, PrimPair order
   const float2* pair_ab;   // 4 per shell pair: R_a - R_b as 3 (hi, lo) pairs, padding
-  // FP32 record per primitive pair (32 bytes): {zeta, PAx, PAy, PAz}, {pref, pref_far, 1/(2 zeta),
-  // its bound / the shell pair's bound}
+  // FP32 record per primitive pair (64 bytes), each scalar stored twice: {-zeta, PAx}, {pref,
+  // pref_far}, {PAy, PAz}, {kappa, -sigma}; prim_share: its bound / the shell pair's bound
   const float4* prims_f32;
+  const float* prim_share;
   const float2* pair_a;    // 4 per shell pair: R_a as 3 (hi, lo) pairs, padding
   int hi_ds;
   int n_dens;      // densities: F and G of density d at foff / goff (F32: foff32) + d ldq nS
