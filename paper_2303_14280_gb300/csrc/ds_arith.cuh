@@ -130,6 +130,19 @@ __device__ __forceinline__ ds ds_mul_raw(ds x, ds y) {
   return ds_make(p, e);
 }
 
+// x^2 + y^2 + z^2 as an unnormalised sum (28 operations; 37 with fma)
+__device__ __forceinline__ ds ds_sqr_raw(ds x) {
+  const float p = __fmul_rn(x.hi, x.hi);
+  return ds_make(p, __fmaf_rn(__fadd_rn(x.hi, x.hi), x.lo, __fmaf_rn(x.hi, x.hi, -p)));
+}
+__device__ __forceinline__ ds ds_two_sum(float a, float b);
+__device__ __forceinline__ ds ds_norm2_raw(ds x, ds y, ds z) {
+  const ds p = ds_sqr_raw(x), q = ds_sqr_raw(y), r = ds_sqr_raw(z);
+  const ds s = ds_two_sum(p.hi, q.hi);
+  const ds t = ds_two_sum(s.hi, r.hi);
+  return ds_make(t.hi, __fadd_rn(__fadd_rn(t.lo, s.lo), __fadd_rn(__fadd_rn(p.lo, q.lo), r.lo)));
+}
+
 // a + b = s + e exactly
 __device__ __forceinline__ ds ds_two_sum(float a, float b) {
   const float s = __fadd_rn(a, b);
