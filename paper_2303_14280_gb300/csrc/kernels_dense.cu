@@ -18,6 +18,7 @@
 
 #include <algorithm>
 #include <cstdint>
+#include <type_traits>
 
 #include "ds_arith.cuh"
 #include "snk_internal.h"
@@ -48,21 +49,24 @@ __device__ __forceinline__ int mol_of_packed(const MolDesc* mols, int n_mol, int
 
 constexpr int TM = 64, TN = 64, TK = 16, GEMM_THREADS = 256;
 
-// C[m][n] = sum_k A(m,k) B(k,n) for the 64 x 64 tile at (m0, n0), K = kdim.
-// la(m, k), lb(k, n) return 0 outside the operands; st(m, n, c) stores.
+// C[m][n] = sum_k A(m,k) B(k,n) for the 64 x 64 tile at (m0, n0) over k in
+// [kbeg, kend).  la(m, k), lb(k, n) return 0 outside the operands; st(m, n, c)
+// stores.  A tile at the operands' edge leaves out its empty groups of 16 rows
+// and 16 columns (block-uniform).
 template <class T = double, class LA, class LB, class ST>
-__device__ __forceinline__ void gemm_tile(int m0, int n0, int mdim, int ndim, int kdim, LA la, LB lb,
+__device__ __forceinline__ void gemm_tile(int m0, int n0, int mdim, int ndim, int kbeg, int kend, LA la, LB lb,
                                           ST st, bool a_k_fast, bool b_k_fast) {
   __shared__ T As[TK][TM + 1];
   __shared__ T Bs[TK][TN + 1];
   const int tid = threadIdx.x;
   const int tx = tid % 16, ty = tid / 16;
+  const int mq = min(4, (mdim - m0 + 15) / 16), nq = min(4, (ndim - n0 + 15) / 16);
   T acc[4][4];
 #pragma unroll
   for (int a = 0; a < 4; ++a)
 #pragma unroll
     for (int b = 0; b < 4; ++b) acc[a][b] = T(0);
-  for (int k0 = 0; k0 < kdim; k0 += TK) {
+  for (int k0 = kbeg; k0 < kend; k0 += TK) {
 #pragma unroll
     for (int r = 0; r < 4; ++r) {
       int e = tid + r * GEMM_THREADS;  // 0..1023
@@ -75,7 +79,7 @@ __device__ __forceinline__ void gemm_tile(int m0, int n0, int mdim, int ndim, in
         kk = e / TM;
       }
       int m = m0 + mm, k = k0 + kk;
-      As[kk][mm] = (m < mdim && k < kdim) ? T(la(m, k)) : T(0);
+      As[kk][mm] = (m < mdim && k < kend) ? T(la(m, k)) : T(0);
       int nn;
       if (b_k_fast) {
         kk = e % TK;
@@ -86,22 +90,29 @@ __device__ __forceinline__ void gemm_tile(int m0, int n0, int mdim, int ndim, in
       }
       int n = n0 + nn;
       k = k0 + kk;
-      Bs[kk][nn] = (n < ndim && k < kdim) ? T(lb(k, n)) : T(0);
+      Bs[kk][nn] = (n < ndim && k < kend) ? T(lb(k, n)) : T(0);
     }
     __syncthreads();
+    auto steps = [&](auto inner) {
 #pragma unroll
-    for (int kk = 0; kk < TK; ++kk) {
-      T a[4], b[4];
+      for (int kk = 0; kk < TK; ++kk) {
+        T a[4], b[4];
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        a[q] = As[kk][ty + 16 * q];
-        b[q] = Bs[kk][tx + 16 * q];
+        for (int q = 0; q < 4; ++q) {
+          a[q] = As[kk][ty + 16 * q];
+          b[q] = Bs[kk][tx + 16 * q];
+        }
+#pragma unroll
+        for (int p = 0; p < 4; ++p)
+#pragma unroll
+          for (int q = 0; q < 4; ++q)
+            if (inner || (p < mq && q < nq)) acc[p][q] = fma(a[p], b[q], acc[p][q]);
       }
-#pragma unroll
-      for (int p = 0; p < 4; ++p)
-#pragma unroll
-        for (int q = 0; q < 4; ++q) acc[p][q] = fma(a[p], b[q], acc[p][q]);
-    }
+    };
+    if (mq == 4 && nq == 4)
+      steps(std::true_type());
+    else
+      steps(std::false_type());
     __syncthreads();
   }
 #pragma unroll
@@ -139,11 +150,12 @@ __device__ __forceinline__ void df32_mac(float2 a, float2 b, float& s, float& c)
   c = __fadd_rn(c, __fadd_rn(err, e));
 }
 
-// C[m][n] = sum_k A(m,k) B(k,n) for the 64 x 64 tile at (m0, n0) with float2
-// (hi, lo) operands; la(m, k), lb(k, n) return (0, 0) outside the operands.
+// C[m][n] = sum_k A(m,k) B(k,n) for the 64 x 64 tile at (m0, n0) over k in
+// [kbeg, kend) with float2 (hi, lo) operands; la(m, k), lb(k, n) return (0, 0)
+// outside the operands.  Empty groups are left out as in gemm_tile.
 template <class LA, class LB, class ST>
-__device__ __forceinline__ void df32_tile(int m0, int n0, int mdim, int ndim, int kdim, LA la, LB lb, ST st,
-                                          bool a_k_fast, bool b_k_fast) {
+__device__ __forceinline__ void df32_tile(int m0, int n0, int mdim, int ndim, int kbeg, int kend, LA la, LB lb,
+                                          ST st, bool a_k_fast, bool b_k_fast) {
   __shared__ float2 As[TK][TM + 1];
   __shared__ float2 Bs[TK][TN + 1];
   const int tid = threadIdx.x;
@@ -153,8 +165,9 @@ __device__ __forceinline__ void df32_tile(int m0, int n0, int mdim, int ndim, in
   for (int a = 0; a < 4; ++a)
 #pragma unroll
     for (int b = 0; b < 4; ++b) s[a][b] = c[a][b] = 0.f;
+  const int mq = min(4, (mdim - m0 + 15) / 16), nq = min(4, (ndim - n0 + 15) / 16);
   const float2 zero = make_float2(0.f, 0.f);
-  for (int k0 = 0; k0 < kdim; k0 += TK) {
+  for (int k0 = kbeg; k0 < kend; k0 += TK) {
 #pragma unroll
     for (int r = 0; r < 4; ++r) {
       const int e = tid + r * GEMM_THREADS;
@@ -167,7 +180,7 @@ __device__ __forceinline__ void df32_tile(int m0, int n0, int mdim, int ndim, in
         kk = e / TM;
       }
       int m = m0 + mm, k = k0 + kk;
-      As[kk][mm] = (m < mdim && k < kdim) ? la(m, k) : zero;
+      As[kk][mm] = (m < mdim && k < kend) ? la(m, k) : zero;
       int nn;
       if (b_k_fast) {
         kk = e % TK;
@@ -178,22 +191,29 @@ __device__ __forceinline__ void df32_tile(int m0, int n0, int mdim, int ndim, in
       }
       const int n = n0 + nn;
       k = k0 + kk;
-      Bs[kk][nn] = (n < ndim && k < kdim) ? lb(k, n) : zero;
+      Bs[kk][nn] = (n < ndim && k < kend) ? lb(k, n) : zero;
     }
     __syncthreads();
+    auto steps = [&](auto inner) {
 #pragma unroll 4
-    for (int kk = 0; kk < TK; ++kk) {
-      float2 a[4], b[4];
+      for (int kk = 0; kk < TK; ++kk) {
+        float2 a[4], b[4];
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        a[q] = As[kk][ty + 16 * q];
-        b[q] = Bs[kk][tx + 16 * q];
+        for (int q = 0; q < 4; ++q) {
+          a[q] = As[kk][ty + 16 * q];
+          b[q] = Bs[kk][tx + 16 * q];
+        }
+#pragma unroll
+        for (int p = 0; p < 4; ++p)
+#pragma unroll
+          for (int q = 0; q < 4; ++q)
+            if (inner || (p < mq && q < nq)) df32_mac(a[p], b[q], s[p][q], c[p][q]);
       }
-#pragma unroll
-      for (int p = 0; p < 4; ++p)
-#pragma unroll
-        for (int q = 0; q < 4; ++q) df32_mac(a[p], b[q], s[p][q], c[p][q]);
-    }
+    };
+    if (mq == 4 && nq == 4)
+      steps(std::true_type());
+    else
+      steps(std::false_type());
     __syncthreads();
   }
 #pragma unroll
@@ -425,7 +445,7 @@ __global__ void __launch_bounds__(GEMM_THREADS) ftilde_kernel(const MolDesc* __r
   // a screening estimate: FP32 sums of non-negative terms (relative error
   // below k 2^-24 <= 3e-4 for k <= 5,000 terms), rounded up by 1e-3
   gemm_tile<float>(
-      m0, n0, md.nf, md.nb, md.nf, [&](int m, int k) { return (float)fabs(Pm[(int64_t)m * md.nf + k]); },
+      m0, n0, md.nf, md.nb, 0, md.nf, [&](int m, int k) { return (float)fabs(Pm[(int64_t)m * md.nf + k]); },
       [&](int k, int n) { return (float)ph[(int64_t)n * md.nf + k]; },
       [&](int m, int n, float c) {
         atomic_max_nonneg(&ft[(int64_t)n * md.ns + (fshell[md.mf0 + m] - md.ms0)], (double)c * (1.0 + 1e-3));
@@ -572,7 +592,7 @@ __global__ void __launch_bounds__(SCR_THREADS) pair_write_kernel(ScreenArgs a, c
 // mixed form an FP32 copy is written for the FP32 pairs.
 // MODE: 0 FP64, 2 double-FP32 on (hi, lo) operands
 template <int MODE>
-__global__ void __launch_bounds__(GEMM_THREADS, MODE >= 2 ? 2 : 3)
+__global__ void __launch_bounds__(GEMM_THREADS, 2)
     fgemm_kernel(const BatchDesc* __restrict__ batches, const double* __restrict__ P, const float2* __restrict__ P2,
                  const int* __restrict__ xfunc, const int* __restrict__ sfunc, const double* __restrict__ fcomp,
                  const double* __restrict__ w, double* __restrict__ ws, float* __restrict__ ws32, int dens) {
@@ -596,25 +616,30 @@ __global__ void __launch_bounds__(GEMM_THREADS, MODE >= 2 ? 2 : 3)
     const float2* Pm2 = P2 + bd.pk_off;
     auto la = [&](int m, int k) { return X2[(int64_t)k * bd.ldq + m]; };
     auto lb = [&](int k, int n) { return Pm2[(int64_t)xf[k] * bd.nfm + sf[n]]; };
-    df32_tile(m0, n0, bd.ldq, bd.nS, bd.nB, la, lb, st, false, false);
+    df32_tile(m0, n0, bd.ldq, bd.nS, 0, bd.nB, la, lb, st, false, false);
   } else {
     const double* X = ws + bd.xoff;
     const double* Pm = P + bd.pk_off;
     auto la = [&](int m, int k) { return X[(int64_t)k * bd.ldq + m]; };
     auto lb = [&](int k, int n) { return Pm[(int64_t)xf[k] * bd.nfm + sf[n]]; };
-    gemm_tile(m0, n0, bd.ldq, bd.nS, bd.nB, la, lb, st, false, false);
+    gemm_tile(m0, n0, bd.ldq, bd.nS, 0, bd.nB, la, lb, st, false, false);
   }
 }
 
 // Kt_{s nu} += sum_i G-hat_{s i} X_{nu i}, scattered into the molecule's block
-// of the packed accumulator (several batches add to the same entries).
+// of the packed accumulator (several batches add to the same entries).  The
+// points of a batch are shared out to blocks of klen (point_split): the
+// accumulator's additions are exact, so the split changes nothing but the
+// rounding inside a block's own sum.
 template <int MODE>
-__global__ void __launch_bounds__(GEMM_THREADS, MODE >= 2 ? 2 : 3)
+__global__ void __launch_bounds__(GEMM_THREADS, 2)
     kgemm_kernel(const BatchDesc* __restrict__ batches, const int* __restrict__ xfunc, const int* __restrict__ sfunc,
-                 const double* __restrict__ ws, unsigned long long* __restrict__ Khat, int dens, int* err) {
+                 const double* __restrict__ ws, unsigned long long* __restrict__ Khat, int dens, int klen, int mtiles,
+                 int* err) {
   const BatchDesc bd = batches[blockIdx.z];
-  const int m0 = blockIdx.x * TM, n0 = blockIdx.y * TN;
-  if (m0 >= bd.nS || n0 >= bd.nB) return;
+  const int m0 = (blockIdx.x % mtiles) * TM, n0 = blockIdx.y * TN;
+  const int kbeg = (blockIdx.x / mtiles) * klen, kend = min(kbeg + klen, bd.q);  // this block's points
+  if (m0 >= bd.nS || n0 >= bd.nB || kbeg >= kend) return;
   const int64_t dofs = (int64_t)dens * bd.ldq * bd.nS;  // density d's G block
   const int* xf = xfunc + bd.xfunc_off;
   const int* sf = sfunc + bd.sfunc_off;
@@ -625,13 +650,13 @@ __global__ void __launch_bounds__(GEMM_THREADS, MODE >= 2 ? 2 : 3)
     const float2* G2 = reinterpret_cast<const float2*>(ws + bd.goff) + dofs;
     auto la = [&](int m, int k) { return G2[(int64_t)m * bd.ldq + k]; };
     auto lb = [&](int k, int n) { return X2[(int64_t)n * bd.ldq + k]; };
-    df32_tile(m0, n0, bd.nS, bd.nB, bd.q, la, lb, st, true, true);
+    df32_tile(m0, n0, bd.nS, bd.nB, kbeg, kend, la, lb, st, true, true);
   } else {
     const double* X = ws + bd.xoff;
     const double* G = ws + bd.goff + dofs;
     auto la = [&](int m, int k) { return G[(int64_t)m * bd.ldq + k]; };
     auto lb = [&](int k, int n) { return X[(int64_t)n * bd.ldq + k]; };
-    gemm_tile(m0, n0, bd.nS, bd.nB, bd.q, la, lb, st, true, true);
+    gemm_tile(m0, n0, bd.nS, bd.nB, kbeg, kend, la, lb, st, true, true);
   }
 }
 
@@ -641,7 +666,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, MODE >= 2 ? 2 : 3)
 // FP64 tiles, MODE 2 double-FP32 tiles with the operands split as they are
 // staged (the FP64 X stays intact for the point kernel).
 template <int MODE>
-__global__ void __launch_bounds__(GEMM_THREADS, MODE >= 2 ? 2 : 3)
+__global__ void __launch_bounds__(GEMM_THREADS, 2)
     xc_fgemm_kernel(const BatchDesc* __restrict__ batches, const double* __restrict__ P,
                     const int* __restrict__ xfunc, double* __restrict__ ws) {
   const BatchDesc bd = batches[blockIdx.z];
@@ -655,21 +680,23 @@ __global__ void __launch_bounds__(GEMM_THREADS, MODE >= 2 ? 2 : 3)
   if (MODE == 2) {
     auto la = [&](int m, int k) { return df32_split(X[(int64_t)k * bd.ldq + m]); };
     auto lb = [&](int k, int n) { return df32_split(Pm[(int64_t)xf[k] * bd.nfm + xf[n]]); };
-    df32_tile(m0, n0, bd.ldq, bd.nB, bd.nB, la, lb, st, false, false);
+    df32_tile(m0, n0, bd.ldq, bd.nB, 0, bd.nB, la, lb, st, false, false);
   } else {
     auto la = [&](int m, int k) { return X[(int64_t)k * bd.ldq + m]; };
     auto lb = [&](int k, int n) { return Pm[(int64_t)xf[k] * bd.nfm + xf[n]]; };
-    gemm_tile(m0, n0, bd.ldq, bd.nB, bd.nB, la, lb, st, false, false);
+    gemm_tile(m0, n0, bd.ldq, bd.nB, 0, bd.nB, la, lb, st, false, false);
   }
 }
 
 template <int MODE>
-__global__ void __launch_bounds__(GEMM_THREADS, MODE >= 2 ? 2 : 3)
+__global__ void __launch_bounds__(GEMM_THREADS, 2)
     xc_vgemm_kernel(const BatchDesc* __restrict__ batches, const int* __restrict__ xfunc,
-                    const double* __restrict__ ws, unsigned long long* __restrict__ Vhat, int* err) {
+                    const double* __restrict__ ws, unsigned long long* __restrict__ Vhat, int klen, int mtiles,
+                    int* err) {
   const BatchDesc bd = batches[blockIdx.z];
-  const int m0 = blockIdx.x * TM, n0 = blockIdx.y * TN;
-  if (m0 >= bd.nB || n0 >= bd.nB) return;
+  const int m0 = (blockIdx.x % mtiles) * TM, n0 = blockIdx.y * TN;
+  const int kbeg = (blockIdx.x / mtiles) * klen, kend = min(kbeg + klen, bd.q);  // this block's points
+  if (m0 >= bd.nB || n0 >= bd.nB || kbeg >= kend) return;
   const double* X = ws + bd.xoff;
   const double* Z = ws + bd.foff;
   const int* xf = xfunc + bd.xfunc_off;
@@ -678,11 +705,11 @@ __global__ void __launch_bounds__(GEMM_THREADS, MODE >= 2 ? 2 : 3)
   if (MODE == 2) {
     auto la = [&](int m, int k) { return df32_split(Z[(int64_t)m * bd.ldq + k]); };
     auto lb = [&](int k, int n) { return df32_split(X[(int64_t)n * bd.ldq + k]); };
-    df32_tile(m0, n0, bd.nB, bd.nB, bd.q, la, lb, st, true, true);
+    df32_tile(m0, n0, bd.nB, bd.nB, kbeg, kend, la, lb, st, true, true);
   } else {
     auto la = [&](int m, int k) { return Z[(int64_t)m * bd.ldq + k]; };
     auto lb = [&](int k, int n) { return X[(int64_t)n * bd.ldq + k]; };
-    gemm_tile(m0, n0, bd.nB, bd.nB, bd.q, la, lb, st, true, true);
+    gemm_tile(m0, n0, bd.nB, bd.nB, kbeg, kend, la, lb, st, true, true);
   }
 }
 
@@ -832,15 +859,30 @@ cudaError_t launch_fgemm(cudaStream_t st, const BatchDesc* dbatch, int nbatch, i
   return cudaGetLastError();
 }
 
-cudaError_t launch_kgemm(cudaStream_t st, const BatchDesc* dbatch, int nbatch, int max_nS, int max_nB,
+// Points per block of a product over a batch's points: with few (tile, batch)
+// pairs the blocks share the points until there are about six per SM, at least
+// 64 points each (a block's 4,096 fixed-point additions are then 1 % of its
+// FP64 work).  4 atoms, 21 functions, 4 batches of 3,000 points: 4 blocks took
+// 3.14 ms, 188 take 0.04; from about 900 (tile, batch) pairs on nothing is split.
+int point_split(int tiles, int max_q, int* klen) {
+  const int want = 152 * 6;
+  const int nsplit = std::max(1, std::min((want + tiles - 1) / std::max(tiles, 1), (max_q + 63) / 64));
+  *klen = std::max(TK, ((max_q + nsplit - 1) / nsplit + TK - 1) / TK * TK);
+  return (max_q + *klen - 1) / *klen;
+}
+
+cudaError_t launch_kgemm(cudaStream_t st, const BatchDesc* dbatch, int nbatch, int max_ldq, int max_nS, int max_nB,
                          const int* xfunc, const int* sfunc, const double* ws, unsigned long long* Khat, int mode,
                          int dens, int* err) {
-  if (nbatch == 0 || max_nS == 0 || max_nB == 0) return cudaSuccess;
-  dim3 grid((max_nS + TM - 1) / TM, (max_nB + TN - 1) / TN, nbatch);
+  if (nbatch == 0 || max_ldq == 0 || max_nS == 0 || max_nB == 0) return cudaSuccess;
+  const int mt = (max_nS + TM - 1) / TM, nt = (max_nB + TN - 1) / TN;
+  int klen = 0;
+  const int nsplit = point_split(mt * nt * nbatch, max_ldq, &klen);
+  dim3 grid(mt * nsplit, nt, nbatch);
   if (mode == 2)
-    kgemm_kernel<2><<<grid, GEMM_THREADS, 0, st>>>(dbatch, xfunc, sfunc, ws, Khat, dens, err);
+    kgemm_kernel<2><<<grid, GEMM_THREADS, 0, st>>>(dbatch, xfunc, sfunc, ws, Khat, dens, klen, mt, err);
   else
-    kgemm_kernel<0><<<grid, GEMM_THREADS, 0, st>>>(dbatch, xfunc, sfunc, ws, Khat, dens, err);
+    kgemm_kernel<0><<<grid, GEMM_THREADS, 0, st>>>(dbatch, xfunc, sfunc, ws, Khat, dens, klen, mt, err);
   return cudaGetLastError();
 }
 
@@ -899,14 +941,17 @@ cudaError_t launch_xc_fgemm(cudaStream_t st, const BatchDesc* dbatch, int nbatch
   return cudaGetLastError();
 }
 
-cudaError_t launch_xc_vgemm(cudaStream_t st, const BatchDesc* dbatch, int nbatch, int max_nB, const int* xfunc,
-                            const double* ws, unsigned long long* Vhat, int mode, int* err) {
-  if (nbatch == 0 || max_nB == 0) return cudaSuccess;
-  dim3 grid((max_nB + TM - 1) / TM, (max_nB + TN - 1) / TN, nbatch);
+cudaError_t launch_xc_vgemm(cudaStream_t st, const BatchDesc* dbatch, int nbatch, int max_ldq, int max_nB,
+                            const int* xfunc, const double* ws, unsigned long long* Vhat, int mode, int* err) {
+  if (nbatch == 0 || max_ldq == 0 || max_nB == 0) return cudaSuccess;
+  const int mt = (max_nB + TM - 1) / TM;
+  int klen = 0;
+  const int nsplit = point_split(mt * mt * nbatch, max_ldq, &klen);
+  dim3 grid(mt * nsplit, mt, nbatch);
   if (mode == 2)
-    xc_vgemm_kernel<2><<<grid, GEMM_THREADS, 0, st>>>(dbatch, xfunc, ws, Vhat, err);
+    xc_vgemm_kernel<2><<<grid, GEMM_THREADS, 0, st>>>(dbatch, xfunc, ws, Vhat, klen, mt, err);
   else
-    xc_vgemm_kernel<0><<<grid, GEMM_THREADS, 0, st>>>(dbatch, xfunc, ws, Vhat, err);
+    xc_vgemm_kernel<0><<<grid, GEMM_THREADS, 0, st>>>(dbatch, xfunc, ws, Vhat, klen, mt, err);
   return cudaGetLastError();
 }
 

@@ -986,7 +986,7 @@ int enqueue_build(snk_ctx* c, cudaStream_t st, double* dK, bool timed) {
       SNK_CK(c, oz_gemm(ch, 2));
     } else {
       for (int d = 0; d < nd; ++d) {
-        SNK_CK(c, launch_kgemm(st, db, nbc, ch.max_nS, ch.max_nB, c->xfunc.p, c->sfunc.p, c->ws.p,
+        SNK_CK(c, launch_kgemm(st, db, nbc, ch.max_ldq, ch.max_nS, ch.max_nB, c->xfunc.p, c->sfunc.p, c->ws.p,
                                c->Khat.p + 2 * d * pk, gmode, d, c->ozerr.p));
         ++c->launches_build;
       }
@@ -1548,7 +1548,7 @@ int build_vxc(snk_ctx* c, int fn, double* dV, double* E_host) {
     if (tc) {
       if (int rc = xc_tc_product(c, ch, 1, Vhat)) return rc;
     } else {
-      SNK_CK(c, launch_xc_vgemm(st, db, n, ch.max_nB, c->xfunc.p, c->xcws.p, Vhat, mode, c->ozerr.p));
+      SNK_CK(c, launch_xc_vgemm(st, db, n, ch.max_ldq, ch.max_nB, c->xfunc.p, c->xcws.p, Vhat, mode, c->ozerr.p));
     }
     if (&ch == &c->xc_chunks.back()) SNK_CK(c, launch_xc_finish(st, c->mols.p, nm, pk, Vhat, Ehat, dV, c->xcE.p));
     SNK_CK(c, cudaEventRecord(c->xcev[ev++], st));

@@ -265,7 +265,7 @@ cudaError_t launch_pair_write(cudaStream_t st, const ScreenArgs& a, int nbatch, 
 cudaError_t launch_fgemm(cudaStream_t st, const BatchDesc* dbatch, int nbatch, int max_ldq, int max_nS,
                          const double* P, const float2* P2, const int* xfunc, const int* sfunc,
                          const double* fcomp, const double* w, double* ws, float* ws32, int mode, int dens);
-cudaError_t launch_kgemm(cudaStream_t st, const BatchDesc* dbatch, int nbatch, int max_nS, int max_nB,
+cudaError_t launch_kgemm(cudaStream_t st, const BatchDesc* dbatch, int nbatch, int max_ldq, int max_nS, int max_nB,
                          const int* xfunc, const int* sfunc, const double* ws, unsigned long long* Khat, int mode,
                          int dens, int* err);
 // In place, each double of buf[0, n) becomes the float pair (fl32(v), fl32(v - fl32(v))).
@@ -290,7 +290,7 @@ cudaError_t launch_xc_fgemm(cudaStream_t st, const BatchDesc* dbatch, int nbatch
                             const double* P, const int* xfunc, double* ws, int mode);
 cudaError_t launch_xc_point(cudaStream_t st, const BatchDesc* dbatch, int nbatch, int max_ldq, const double* w,
                             int functional, double* ws, unsigned long long* Ehat, int* err);
-cudaError_t launch_xc_vgemm(cudaStream_t st, const BatchDesc* dbatch, int nbatch, int max_nB, const int* xfunc,
+cudaError_t launch_xc_vgemm(cudaStream_t st, const BatchDesc* dbatch, int nbatch, int max_ldq, int max_nB, const int* xfunc,
                             const double* ws, unsigned long long* Vhat, int mode, int* err);
 // V = V-hat + V-hat^T in every molecule block of the packed matrices, and
 // E[m] = E-hat of molecule m (two words per molecule).
