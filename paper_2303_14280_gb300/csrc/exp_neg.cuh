@@ -1,0 +1,39 @@
+// e^{-x} for 0 <= x < 700 in FP64 with nine FP64 operations, by the table-driven
+// method (P. T. P. Tang, ACM Trans. Math. Softw. 15, 144, 1989): x = k ln2/256 +
+// r with |r| <= ln2/512, e^{-x} = 2^{-k/256} e^{-r}; 2^{-j/256}, j < 256, comes from a
+// table in shared memory, the remaining power of two goes into the exponent
+// bits, and e^{-r} - 1 is its Taylor polynomial of degree 4 (the next term is
+// below 4e-17).  ln2/256 is split into a 32-bit head, so that k head is exact,
+// and a tail.  Relative error about one unit in the last place.
+//
+// FP64 issues at 2 lanes per clock and SM on GB300, so the number of FP64
+// operations is what the collocation kernels cost.
+#pragma once
+
+#include <cuda_runtime.h>
+
+#include "snk_internal.h"
+
+namespace snk {
+
+__device__ __forceinline__ void exp_table_load(double* tab, const double* __restrict__ gtab) {
+  for (int e = threadIdx.x; e < kExpTable; e += blockDim.x) tab[e] = gtab[e];
+  __syncthreads();
+}
+
+__device__ __forceinline__ double exp_neg(double x, const double* tab) {
+  constexpr double kMagic = 0x1.8p52;  // adding it rounds to an integer in the low word
+  const double t = fma(x, 0x1.71547652b82fep+8, kMagic);  // 256 / ln2
+  const int k = __double2loint(t);
+  const double kd = t - kMagic;
+  double r = fma(-kd, 0x1.62e42fee00000p-9, x);
+  r = fma(-kd, 0x1.a39ef35793c76p-41, r);
+  double q = fma(r, 1.0 / 24.0, -1.0 / 6.0);
+  q = fma(q, r, 0.5);
+  q = fma(q, r, -1.0);
+  const double T = tab[k & (kExpTable - 1)];
+  const double e = fma(T, q * r, T);
+  return __hiloint2double(__double2hiint(e) - ((k >> 8) << 20), __double2loint(e));
+}
+
+}  // namespace snk

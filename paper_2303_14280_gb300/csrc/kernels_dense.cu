@@ -21,6 +21,7 @@
 #include <type_traits>
 
 #include "ds_arith.cuh"
+#include "exp_neg.cuh"
 #include "snk_internal.h"
 
 namespace snk {
@@ -251,7 +252,10 @@ __global__ void __launch_bounds__(COL_THREADS) collocation_kernel(const BatchDes
   const BatchDesc bd = batches[blockIdx.z];
   const int i = blockIdx.x * COL_THREADS + threadIdx.x;
   const int t0 = blockIdx.y * COL_SHELLS;
-  if (i >= bd.ldq || t0 >= bd.nBshell) return;
+  if (blockIdx.x * COL_THREADS >= bd.ldq || t0 >= bd.nBshell) return;  // block-uniform
+  __shared__ double s_exp[kExpTable];
+  exp_table_load(s_exp, B.exptab);
+  if (i >= bd.ldq) return;
   const int t1 = min(t0 + COL_SHELLS, bd.nBshell);
   const bool valid = i < bd.q;
   double x = 0.0, y = 0.0, z = 0.0;
@@ -277,7 +281,7 @@ __global__ void __launch_bounds__(COL_THREADS) collocation_kernel(const BatchDes
       // e^{-60} ~ 9e-27: primitives that far out add nothing representable next to
       // the batch's other values, and skipping the FP64 exponential is the saving
       const double x = B.exps[k] * r2;
-      if (x < kColExpCut) rad += B.d[k] * exp(-x);
+      if (x < kColExpCut) rad = fma(B.d[k], exp_neg(x, s_exp), rad);
     }
     const double* f = B.fcomp + B.foff[sh];
     if (l == 0) {

@@ -114,7 +114,7 @@ struct snk_ctx {
 
   // geometry (device)
   DevBuf<int> l, poff, nprim, foff, fshell, bshell, bshell_col, xfunc;
-  DevBuf<double> center, exps, d, fcomp, xyz, w, boys, bound, qbound, bcenter, bradius, phit_f, phit_b;
+  DevBuf<double> center, exps, d, fcomp, exptab, xyz, w, boys, bound, qbound, bcenter, bradius, phit_f, phit_b;
   DevBuf<float> boys_f, boys_ds, prims_ds, pair_ab, pair_a, prims_f32, prim_share;  // mixed form: FP32 and (hi, lo) copies
   DevBuf<PairHdr> pairs;
   DevBuf<PrimPair> prims;
@@ -210,7 +210,7 @@ struct snk_ctx {
   template <class F>
   void for_each_buffer(F f) {
     f(l), f(poff), f(nprim), f(foff), f(fshell), f(bshell), f(bshell_col), f(xfunc);
-    f(center), f(exps), f(d), f(fcomp), f(xyz), f(w), f(boys), f(bound), f(qbound), f(bcenter), f(bradius);
+    f(center), f(exps), f(d), f(fcomp), f(exptab), f(xyz), f(w), f(boys), f(bound), f(qbound), f(bcenter), f(bradius);
     f(phit_f), f(phit_b);
     f(boys_f), f(boys_ds), f(prims_ds), f(pair_ab), f(pair_a), f(prims_f32), f(prim_share);
     f(pairs), f(prims), f(mols), f(mlp_w), f(shell_feat), f(keep);
@@ -275,6 +275,7 @@ DeviceBasis dev_basis(snk_ctx* c) {
   b.d = c->d.p;
   b.fcomp = c->fcomp.p;
   b.foff = c->foff.p;
+  b.exptab = c->exptab.p;
   return b;
 }
 
@@ -1262,6 +1263,9 @@ int create(int n_mol, const snk_basis* bases, const snk_grid* grids, const snk_o
          SNK_CK(cp, upload(cp->exps, s.exps, st));
          SNK_CK(cp, upload(cp->d, s.d, st));
          SNK_CK(cp, upload(cp->fcomp, s.fcomp, st));
+         std::vector<double> et(kExpTable);
+         for (int e = 0; e < kExpTable; ++e) et[e] = std::exp2(-(double)e / kExpTable);
+         SNK_CK(cp, upload(cp->exptab, et, st));
          SNK_CK(cp, upload(cp->pairs, s.pairs, st));
          SNK_CK(cp, upload(cp->prims, s.prims, st));
          SNK_CK(cp, upload(cp->bound, s.bound, st));

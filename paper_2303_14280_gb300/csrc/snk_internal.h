@@ -47,6 +47,9 @@ __device__ __forceinline__ double khat_value(const unsigned long long* e) {
 // Boys table: rows T_k = k * kBoysH, k = 0..kBoysRows-1; for T >= kBoysTMax the
 // asymptotic form is used.  One table per L = 0..4 with kBoysCols doubles per
 // row: F_{L+m}(T_k)/m! for m = 0..7, exp(-T_k), T_k.
+// Table of the collocation kernels' e^{-x}: 2^{-j/256}.
+constexpr int kExpTable = 256;
+
 constexpr double kBoysH = 0.1;
 constexpr double kBoysTMax = 50.0;
 constexpr int kBoysRows = 502;
@@ -211,6 +214,7 @@ void host_boys(int nmax, double T, double* F);
 // ---------------------------------------------------------------- kernels
 
 struct DeviceBasis {
+  const double* exptab;  // 2^{-j/kExpTable} of exp_neg
   const int* l;
   const int* poff;
   const int* nprim;
