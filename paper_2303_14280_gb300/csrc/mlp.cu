@@ -13,6 +13,7 @@
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstdint>
 
 #include "snk_internal.h"
@@ -22,6 +23,7 @@ namespace snk {
 namespace {
 
 constexpr int NIN = kMlpIn, NH = kMlpHidden;
+constexpr int kMlpThreads = 128;  // samples per block of the backward pass
 constexpr int OW1 = 0, OB1 = OW1 + NIN * NH, OW2 = OB1 + NH, OB2 = OW2 + NH * NH, OW3 = OB2 + NH,
               OB3 = OW3 + NH * NH, OW4 = OB3 + NH, OB4 = OW4 + NH;
 static_assert(OB4 + 1 == kMlpWeights, "weight layout");
@@ -29,28 +31,29 @@ static_assert(OB4 + 1 == kMlpWeights, "weight layout");
 // ---------------------------------------------------------------- FP32 forward / backward
 
 // Forward for one sample with the weights in shared memory; stores the three
-// hidden pre-activations (z1, z2, z3) if zs != nullptr.  Returns the output.
-__device__ float mlp_forward_one(const float* __restrict__ w, const float* x, float* zs) {
+// hidden pre-activations (z1, z2, z3) if zs != nullptr, ldz floats apart (unit
+// by unit, so that a warp's samples make one row).  Returns the output.
+__device__ float mlp_forward_one(const float* __restrict__ w, const float* x, float* zs, int64_t ldz = 0) {
   float a[NH], b[NH];
 #pragma unroll 4
   for (int n = 0; n < NH; ++n) {
     float s = w[OB1 + n];
     for (int k = 0; k < NIN; ++k) s = fmaf(x[k], w[OW1 + k * NH + n], s);
-    if (zs) zs[n] = s;
+    if (zs) zs[n * ldz] = s;
     a[n] = fmaxf(s, 0.f);
   }
 #pragma unroll 4
   for (int n = 0; n < NH; ++n) {
     float s = w[OB2 + n];
     for (int k = 0; k < NH; ++k) s = fmaf(a[k], w[OW2 + k * NH + n], s);
-    if (zs) zs[NH + n] = s;
+    if (zs) zs[(NH + n) * ldz] = s;
     b[n] = fmaxf(s, 0.f);
   }
 #pragma unroll 4
   for (int n = 0; n < NH; ++n) {
     float s = w[OB3 + n];
     for (int k = 0; k < NH; ++k) s = fmaf(b[k], w[OW3 + k * NH + n], s);
-    if (zs) zs[2 * NH + n] = s;
+    if (zs) zs[(2 * NH + n) * ldz] = s;
     a[n] = fmaxf(s, 0.f);
   }
   float y = w[OB4];
@@ -72,99 +75,138 @@ __global__ void mlp_forward_kernel(const float* __restrict__ wg, const float* __
 
 // Asymmetric squared error: L = (1/n) sum_s c_s r_s^2, r = prediction - label,
 // c = 1 for over-prediction and c = under_weight for under-prediction (an
-// under-predicted block could be skipped wrongly).  Per sample it stores the
-// pre-activations and the output gradients dL/dz of every layer.
+// under-predicted block could be skipped wrongly).  Stores the pre-activations
+// and the output gradients dL/dz of every layer, unit by unit with the samples
+// fastest, and each block's part of the loss.
 __global__ void mlp_backward_kernel(const float* __restrict__ wg, const float* __restrict__ X,
                                     const float* __restrict__ Y, const int64_t* __restrict__ idx, int64_t n,
                                     float under_weight,
-                                    float* __restrict__ Z /* n x 3NH */, float* __restrict__ D /* n x (3NH+1) */,
-                                    float* __restrict__ loss) {
+                                    float* __restrict__ Z /* 3NH x n */, float* __restrict__ D /* (3NH+1) x n */,
+                                    double* __restrict__ loss_part) {
   __shared__ float w[kMlpWeights];
   for (int e = threadIdx.x; e < kMlpWeights; e += blockDim.x) w[e] = wg[e];
   __syncthreads();
+  __shared__ double red[kMlpThreads / 32];
   const int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (s >= n) return;
-  const int64_t row = idx ? idx[s] : s;
-  float x[NIN];
-  for (int k = 0; k < NIN; ++k) x[k] = X[row * NIN + k];
-  float* z = Z + s * 3 * NH;
-  const float y = mlp_forward_one(w, x, z);
-  const float r = y - Y[row];
-  const float c = r < 0.f ? under_weight : 1.f;
-  atomicAdd(loss, c * r * r / (float)n);
-  float* d = D + s * (3 * NH + 1);
-  const float dy = 2.f * c * r / (float)n;
-  d[3 * NH] = dy;
-  // layer 4 -> 3
-  float g3[NH], g2[NH];
-  for (int k = 0; k < NH; ++k) {
-    g3[k] = z[2 * NH + k] > 0.f ? dy * w[OW4 + k] : 0.f;
-    d[2 * NH + k] = g3[k];
+  double part = 0.0;
+  if (s < n) {
+    const int64_t row = idx ? idx[s] : s;
+    float x[NIN];
+    for (int k = 0; k < NIN; ++k) x[k] = X[row * NIN + k];
+    float* z = Z + s;
+    const float y = mlp_forward_one(w, x, z, n);
+    const float r = y - Y[row];
+    const float c = r < 0.f ? under_weight : 1.f;
+    part = (double)(c * r * r / (float)n);
+    float* d = D + s;
+    const float dy = 2.f * c * r / (float)n;
+    d[3 * NH * n] = dy;
+    // layer 4 -> 3
+    float g3[NH], g2[NH];
+    for (int k = 0; k < NH; ++k) {
+      g3[k] = z[(2 * NH + k) * n] > 0.f ? dy * w[OW4 + k] : 0.f;
+      d[(2 * NH + k) * n] = g3[k];
+    }
+    for (int k = 0; k < NH; ++k) {
+      float s2 = 0.f;
+      for (int m = 0; m < NH; ++m) s2 = fmaf(w[OW3 + k * NH + m], g3[m], s2);
+      g2[k] = z[(NH + k) * n] > 0.f ? s2 : 0.f;
+      d[(NH + k) * n] = g2[k];
+    }
+    for (int k = 0; k < NH; ++k) {
+      float s1 = 0.f;
+      for (int m = 0; m < NH; ++m) s1 = fmaf(w[OW2 + k * NH + m], g2[m], s1);
+      d[k * n] = z[k * n] > 0.f ? s1 : 0.f;
+    }
   }
-  for (int k = 0; k < NH; ++k) {
-    float s2 = 0.f;
-    for (int m = 0; m < NH; ++m) s2 = fmaf(w[OW3 + k * NH + m], g3[m], s2);
-    g2[k] = z[NH + k] > 0.f ? s2 : 0.f;
-    d[NH + k] = g2[k];
-  }
-  for (int k = 0; k < NH; ++k) {
-    float s1 = 0.f;
-    for (int m = 0; m < NH; ++m) s1 = fmaf(w[OW2 + k * NH + m], g2[m], s1);
-    d[k] = z[k] > 0.f ? s1 : 0.f;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = part;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double t = 0.0;
+    for (int k = 0; k < kMlpThreads / 32; ++k) t += red[k];
+    loss_part[blockIdx.x] = t;
   }
 }
 
-// Gradient of every weight, one thread per weight, summed over the samples:
-// dW_l[k][m] = sum_s a_{l-1}[s][k] d_l[s][m], db_l[m] = sum_s d_l[s][m].
-__global__ void mlp_grad_reduce_kernel(const float* __restrict__ X, const int64_t* __restrict__ idx,
-                                       const float* __restrict__ Z, const float* __restrict__ D, int64_t n,
-                                       float* __restrict__ grad) {
-  const int e = blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= kMlpWeights) return;
-  int layer, k = -1, m;
-  if (e < OB1) {
-    layer = 0;
-    k = (e - OW1) / NH;
-    m = (e - OW1) % NH;
-  } else if (e < OW2) {
-    layer = 0;
-    m = e - OB1;
-  } else if (e < OB2) {
-    layer = 1;
-    k = (e - OW2) / NH;
-    m = (e - OW2) % NH;
-  } else if (e < OW3) {
-    layer = 1;
-    m = e - OB2;
-  } else if (e < OB3) {
-    layer = 2;
-    k = (e - OW3) / NH;
-    m = (e - OW3) % NH;
-  } else if (e < OW4) {
-    layer = 2;
-    m = e - OB3;
-  } else if (e < OB4) {
-    layer = 3;
-    k = e - OW4;
-    m = 0;
-  } else {
-    layer = 3;
-    m = 0;
-  }
-  double acc = 0.0;  // FP64 sum over the samples (off the hot path)
-  for (int64_t s = 0; s < n; ++s) {
-    const float* d = D + s * (3 * NH + 1);
-    const float dz = layer == 3 ? d[3 * NH] : d[layer * NH + m];
-    float a = 1.f;
-    if (k >= 0) {
-      if (layer == 0)
-        a = X[(idx ? idx[s] : s) * NIN + k];
-      else
-        a = fmaxf(Z[s * 3 * NH + (layer - 1) * NH + k], 0.f);
+// Gradient of every weight in FP64, dW_l[k][m] = sum_s a_{l-1}[s][k] d_l[s][m] and
+// db_l[m] = sum_s d_l[s][m]: a product over the samples, one block per (range of
+// klen samples, layer) with 16 samples at a time staged in shared memory as
+// doubles and 4 x 4 sums per thread.  Bound by the FP64 pipe (9,473
+// multiply-adds per sample); the samples are shared out so that every SM has
+// work, and mlp_grad_sum_kernel adds the ranges in order.  One thread per weight
+// over all samples took 74 blocks and two conversions per multiply-add (the
+// conversions run on the FP64 pipe too); 32,768 samples, whole call: 11.1 -> 1.15 ms.
+constexpr int kGradK = 16;
+__global__ void __launch_bounds__(256) mlp_grad_part_kernel(const float* __restrict__ X, const int64_t* __restrict__ idx,
+                                                            const float* __restrict__ Z, const float* __restrict__ D,
+                                                            int64_t n, int klen, double* __restrict__ part) {
+  __shared__ double As[kGradK][NH + 1], Bs[kGradK][NH + 1];
+  const int layer = blockIdx.y;
+  const int mdim = layer == 0 ? NIN : NH, ndim = layer == 3 ? 1 : NH;
+  const int ow = layer == 0 ? OW1 : layer == 1 ? OW2 : layer == 2 ? OW3 : OW4;
+  const int64_t kbeg = (int64_t)blockIdx.x * klen, kend = kbeg + klen < n ? kbeg + klen : n;
+  const int tid = threadIdx.x, tx = tid % 16, ty = tid / 16;
+  const int mq = mdim / 16, nq = (ndim + 15) / 16;  // groups of 16 in use (block-uniform)
+  double acc[4][4], bias = 0.0;
+#pragma unroll
+  for (int p = 0; p < 4; ++p)
+#pragma unroll
+    for (int q = 0; q < 4; ++q) acc[p][q] = 0.0;
+  for (int64_t k0 = kbeg; k0 < kend; k0 += kGradK) {
+#pragma unroll
+    for (int r = 0; r < kGradK * NH / 256; ++r) {
+      const int e = tid + r * 256, kk = e % kGradK, mm = e / kGradK;
+      const int64_t s = k0 + kk;
+      float a = 0.f, d = 0.f;
+      if (s < kend) {
+        if (mm < mdim) a = layer == 0 ? X[(idx ? idx[s] : s) * NIN + mm] : fmaxf(Z[((layer - 1) * NH + mm) * n + s], 0.f);
+        if (mm < ndim) d = D[(layer * NH + mm) * n + s];
+      }
+      As[kk][mm] = (double)a;
+      Bs[kk][mm] = (double)d;
     }
-    acc += (double)a * dz;
+    __syncthreads();
+#pragma unroll
+    for (int kk = 0; kk < kGradK; ++kk) {
+#pragma unroll
+      for (int p = 0; p < 4; ++p)
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+          if (p < mq && q < nq) acc[p][q] = fma(As[kk][ty + 16 * p], Bs[kk][tx + 16 * q], acc[p][q]);
+    }
+    if (tid < ndim)
+      for (int kk = 0; kk < kGradK; ++kk) bias += Bs[kk][tid];
+    __syncthreads();
   }
-  grad[e] = (float)acc;
+  double* out = part + (int64_t)blockIdx.x * kMlpWeights + ow;
+#pragma unroll
+  for (int p = 0; p < 4; ++p)
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int k = ty + 16 * p, m = tx + 16 * q;
+      if (k < mdim && m < ndim) out[k * ndim + m] = acc[p][q];
+    }
+  if (tid < ndim) out[mdim * ndim + tid] = bias;  // the layer's biases follow its weights
+}
+
+// grad = sum of the ranges' parts, loss = sum of the blocks' parts, in order.
+__global__ void mlp_grad_sum_kernel(const double* __restrict__ part, int nsplit, const double* __restrict__ loss_part,
+                                    int nloss, float* __restrict__ grad, float* __restrict__ loss) {
+  const int e = blockIdx.x * blockDim.x + threadIdx.x;
+  if (e < kMlpWeights) {
+    double t = 0.0;
+    for (int k = 0; k < nsplit; ++k) t += part[(int64_t)k * kMlpWeights + e];
+    grad[e] = (float)t;
+  }
+  if (blockIdx.x == 0 && threadIdx.x < 32) {
+    double t = 0.0;
+    for (int k = threadIdx.x; k < nloss; k += 32) t += loss_part[k];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    if (threadIdx.x == 0) *loss = (float)t;
+  }
 }
 
 __global__ void adam_kernel(float* __restrict__ w, const float* __restrict__ g, float* __restrict__ m1,
@@ -533,13 +575,28 @@ cudaError_t launch_mlp_forward(cudaStream_t st, const float* w, const float* X, 
   return cudaGetLastError();
 }
 
+// ranges of samples of the gradient product: one per SM, at least 64 samples each
+static int mlp_grad_split(int64_t n, int* klen) {
+  const int64_t nsplit = std::max<int64_t>(1, std::min<int64_t>(152, (n + 63) / 64));
+  *klen = (int)((((n + nsplit - 1) / nsplit) + kGradK - 1) / kGradK * kGradK);
+  return (int)((n + *klen - 1) / *klen);
+}
+
+int64_t mlp_grad_workspace(int64_t n) {  // non-decreasing in n
+  return std::min<int64_t>(152, (n + 63) / 64) * kMlpWeights + (n + kMlpThreads - 1) / kMlpThreads;
+}
+
 cudaError_t launch_mlp_grad(cudaStream_t st, const float* w, const float* X, const float* Y, const int64_t* idx,
-                            int64_t n, float under_weight, float* Z, float* D, float* grad, float* loss) {
+                            int64_t n, float under_weight, float* Z, float* D, double* work, float* grad,
+                            float* loss) {
   if (n == 0) return cudaSuccess;
-  cudaError_t e = cudaMemsetAsync(loss, 0, sizeof(float), st);
-  if (e != cudaSuccess) return e;
-  mlp_backward_kernel<<<(unsigned)((n + 127) / 128), 128, 0, st>>>(w, X, Y, idx, n, under_weight, Z, D, loss);
-  mlp_grad_reduce_kernel<<<(kMlpWeights + 127) / 128, 128, 0, st>>>(X, idx, Z, D, n, grad);
+  int klen = 0;
+  const int nsplit = mlp_grad_split(n, &klen);
+  const int nblk = (int)((n + kMlpThreads - 1) / kMlpThreads);
+  double* loss_part = work + (int64_t)nsplit * kMlpWeights;
+  mlp_backward_kernel<<<nblk, kMlpThreads, 0, st>>>(w, X, Y, idx, n, under_weight, Z, D, loss_part);
+  mlp_grad_part_kernel<<<dim3(nsplit, 4), 256, 0, st>>>(X, idx, Z, D, n, klen, work);
+  mlp_grad_sum_kernel<<<(kMlpWeights + 127) / 128, 128, 0, st>>>(work, nsplit, loss_part, nblk, grad, loss);
   return cudaGetLastError();
 }
 

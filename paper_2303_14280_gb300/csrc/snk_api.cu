@@ -2244,20 +2244,32 @@ int snk_mlp_eval(const float* weights, const float* features, int64_t n, int32_t
 int snk_mlp_grad(const float* weights, const float* features, const float* labels, int64_t n, float under_weight,
                  float* grad, float* loss) {
   if (!weights || !grad || !loss || n <= 0 || !features || !labels) return SNK_ERR_INVALID_ARG;
-  DevBuf<float> dw, dx, dy, dz, dd, dg, dl;
-  if (dw.ensure(kMlpWeights) || dx.ensure((size_t)n * kMlpIn) || dy.ensure(n) ||
-      dz.ensure((size_t)n * 3 * kMlpHidden) || dd.ensure((size_t)n * (3 * kMlpHidden + 1)) ||
-      dg.ensure(kMlpWeights) || dl.ensure(1))
-    return SNK_ERR_OOM;
-  if (cudaMemcpy(dw.p, weights, sizeof(float) * kMlpWeights, cudaMemcpyHostToDevice) ||
-      cudaMemcpy(dx.p, features, sizeof(float) * n * kMlpIn, cudaMemcpyHostToDevice) ||
-      cudaMemcpy(dy.p, labels, sizeof(float) * n, cudaMemcpyHostToDevice))
+  // one device block for everything: each allocation and release costs about
+  // as much as a kernel
+  const size_t sizes[8] = {(size_t)kMlpWeights * 4,        (size_t)n * kMlpIn * 4,
+                           (size_t)n * 4,                  (size_t)n * 3 * kMlpHidden * 4,
+                           (size_t)n * (3 * kMlpHidden + 1) * 4, (size_t)(kMlpWeights + 1) * 4,
+                           (size_t)mlp_grad_workspace(n) * 8, 0};
+  size_t off[8], total = 0;
+  for (int k = 0; k < 8; ++k) {
+    off[k] = total;
+    total += (sizes[k] + 255) / 256 * 256;
+  }
+  DevBuf<uint8_t> all;
+  if (all.ensure(total)) return SNK_ERR_OOM;
+  auto f32 = [&](int k) { return reinterpret_cast<float*>(all.p + off[k]); };
+  float *dw = f32(0), *dx = f32(1), *dy = f32(2), *dg = f32(5);
+  if (cudaMemcpy(dw, weights, sizes[0], cudaMemcpyHostToDevice) ||
+      cudaMemcpy(dx, features, sizes[1], cudaMemcpyHostToDevice) ||
+      cudaMemcpy(dy, labels, sizes[2], cudaMemcpyHostToDevice))
     return SNK_ERR_CUDA;
-  if (launch_mlp_grad(0, dw.p, dx.p, dy.p, nullptr, n, under_weight, dz.p, dd.p, dg.p, dl.p) != cudaSuccess)
+  if (launch_mlp_grad(0, dw, dx, dy, nullptr, n, under_weight, f32(3), f32(4),
+                      reinterpret_cast<double*>(all.p + off[6]), dg, dg + kMlpWeights) != cudaSuccess)
     return SNK_ERR_CUDA;
-  if (cudaMemcpy(grad, dg.p, sizeof(float) * kMlpWeights, cudaMemcpyDeviceToHost) ||
-      cudaMemcpy(loss, dl.p, sizeof(float), cudaMemcpyDeviceToHost))
-    return SNK_ERR_CUDA;
+  std::vector<float> h(kMlpWeights + 1);
+  if (cudaMemcpy(h.data(), dg, sizes[5], cudaMemcpyDeviceToHost)) return SNK_ERR_CUDA;
+  std::copy(h.begin(), h.end() - 1, grad);
+  *loss = h.back();
   return SNK_OK;
 }
 
@@ -2285,11 +2297,12 @@ int snk_mlp_train(const float* features, const float* labels, int64_t n, int32_t
   const int64_t B = std::min<int64_t>(batch, n);
   DevBuf<float> dw, dx, dy, dz, dd, dg, dm1, dm2, dl;
   DevBuf<int64_t> didx;
+  DevBuf<double> dwork;
   const int64_t nsteps = (n + B - 1) / B;
   if (dw.ensure(kMlpWeights) || dx.ensure((size_t)n * kMlpIn) || dy.ensure(n) ||
       dz.ensure((size_t)B * 3 * kMlpHidden) || dd.ensure((size_t)B * (3 * kMlpHidden + 1)) ||
       dg.ensure(kMlpWeights) || dm1.ensure(kMlpWeights) || dm2.ensure(kMlpWeights) || dl.ensure(nsteps) ||
-      didx.ensure(n))
+      didx.ensure(n) || dwork.ensure((size_t)mlp_grad_workspace(B)))
     return SNK_ERR_OOM;
   if (cudaMemcpy(dw.p, w.data(), sizeof(float) * kMlpWeights, cudaMemcpyHostToDevice) ||
       cudaMemcpy(dx.p, features, sizeof(float) * n * kMlpIn, cudaMemcpyHostToDevice) ||
@@ -2305,7 +2318,8 @@ int snk_mlp_train(const float* features, const float* labels, int64_t n, int32_t
     if (cudaMemcpy(didx.p, idx.data(), sizeof(int64_t) * n, cudaMemcpyHostToDevice)) return SNK_ERR_CUDA;
     for (int64_t st = 0; st < nsteps; ++st) {
       const int64_t b0 = st * B, nb = std::min<int64_t>(B, n - b0);
-      if (launch_mlp_grad(0, dw.p, dx.p, dy.p, didx.p + b0, nb, under_weight, dz.p, dd.p, dg.p, dl.p + st) !=
+      if (launch_mlp_grad(0, dw.p, dx.p, dy.p, didx.p + b0, nb, under_weight, dz.p, dd.p, dwork.p, dg.p,
+                          dl.p + st) !=
               cudaSuccess ||
           launch_adam(0, dw.p, dg.p, dm1.p, dm2.p, ++t, lr) != cudaSuccess)
         return SNK_ERR_CUDA;

@@ -417,8 +417,11 @@ cudaError_t launch_wait_probe(cudaStream_t st, int* err, unsigned long long limi
 cudaError_t launch_labels(cudaStream_t st, int cls, const IntegralArgs& a, int grid, const int64_t* slot_base,
                           const int64_t* list_off, const double* xm, float* lab);
 cudaError_t launch_mlp_forward(cudaStream_t st, const float* w, const float* X, int64_t n, float* out, bool f16);
+// doubles of workspace launch_mlp_grad needs for n samples
+int64_t mlp_grad_workspace(int64_t n);
 cudaError_t launch_mlp_grad(cudaStream_t st, const float* w, const float* X, const float* Y, const int64_t* idx,
-                            int64_t n, float under_weight, float* Z, float* D, float* grad, float* loss);
+                            int64_t n, float under_weight, float* Z, float* D, double* work, float* grad,
+                            float* loss);
 cudaError_t launch_adam(cudaStream_t st, float* w, const float* g, float* m1, float* m2, int t, float lr);
 cudaError_t launch_features(cudaStream_t st, const ScreenArgs& a, const int* pairlist, const int64_t* list_off,
                             const int* counts, const int* sample_batches, const int64_t* sample_off, int n_sample,
