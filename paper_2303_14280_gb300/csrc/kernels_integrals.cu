@@ -841,11 +841,18 @@ __device__ __forceinline__ void pair_xi_ds(const PairHdr& h, const float2* __res
 
 // The FP64 lists of the mixed form in ds arithmetic: same tiles, tickets,
 // contraction and FP64 G atomics as integral_kernel; F is read in FP64 and
-// split, each G update is rounded to FP64 once.
+// split, each G update is rounded to FP64 once.  Bound by the FP32 FMA pipe
+// (70-80 % busy), dd by instruction fetch: its recursion, HRR and contraction
+// are about 5,000 straight-line instructions (80 KB), and warps in different
+// places of it evict each other's lines.  There the CTA's warps start every
+// pair together (a barrier per pair, block-uniform; threads past the batch's
+// points compute the last point and add nothing): 96 atoms, 768,000 points, dd
+// 89.6 -> 66.1 ms.  dp gains nothing from it (66.4 / 66.6).
 template <int LA, int LB, int ND>
 __global__ void __launch_bounds__(kIntThreads) integral_kernel_ds(IntegralArgs a) {
   using C = OsClass<LA, LB>;
   constexpr int NA = C::NA, NB = C::NB;
+  constexpr bool kLockstep = C::L == 4;
   extern __shared__ float2 s_tab2[];
   const float2* gtab = a.boys_ds + (size_t)C::L * kBoysRows * kBoysCols;
   for (int e = threadIdx.x; e < kBoysRows * kBoysCols; e += blockDim.x) s_tab2[e] = gtab[e];
@@ -859,8 +866,10 @@ __global__ void __launch_bounds__(kIntThreads) integral_kernel_ds(IntegralArgs a
     if (t >= a.n_tiles) break;
     const Tile tile = a.tiles[t];
     const BatchDesc bd = a.batches[tile.batch];
-    const int i = tile.i0 + threadIdx.x;
-    if (i >= bd.q) continue;
+    int i = tile.i0 + threadIdx.x;
+    const bool act = i < bd.q;
+    if (!kLockstep && !act) continue;
+    if (!act) i = bd.q - 1;
     const int64_t ldq = bd.ldq, dstr = (int64_t)bd.ldq * bd.nS;
     const ds cx = ds_from(a.xyz[3 * (bd.p0 + i)]), cy = ds_from(a.xyz[3 * (bd.p0 + i) + 1]),
              cz = ds_from(a.xyz[3 * (bd.p0 + i) + 2]);
@@ -869,7 +878,12 @@ __global__ void __launch_bounds__(kIntThreads) integral_kernel_ds(IntegralArgs a
     const int* cmap = a.colmap + bd.cm_off - bd.ms0;
     ds ga[ND][NA], fa[ND][NA];
     int cur = -1, cola = 0;
+    // act holds for every thread here but in lockstep
+    auto gadd = [&](int d, int col, ds v) {
+      if (act) atomicAdd(G + d * dstr + col * ldq, ds_to(v));
+    };
     for (int k = tile.k0; k < tile.k1; ++k) {
+      if (kLockstep) __syncthreads();
       const int p = a.pairlist[k];
       const PairHdr h = a.pairs[p];
       if (h.sa != cur) {
@@ -877,7 +891,7 @@ __global__ void __launch_bounds__(kIntThreads) integral_kernel_ds(IntegralArgs a
 #pragma unroll
           for (int d = 0; d < ND; ++d)
 #pragma unroll
-            for (int u = 0; u < NA; ++u) atomicAdd(G + d * dstr + (cola + u) * ldq, ds_to(ga[d][u]));
+            for (int u = 0; u < NA; ++u) gadd(d, cola + u, ga[d][u]);
         }
         cur = h.sa;
         cola = cmap[cur];
@@ -912,7 +926,7 @@ __global__ void __launch_bounds__(kIntThreads) integral_kernel_ds(IntegralArgs a
             ds g = ds_make(0.f, 0.f);
 #pragma unroll
             for (int u = 0; u < NA; ++u) acc_mac(g, xi[u * NB + v], fa[d][u]);
-            atomicAdd(G + d * dstr + (colb + v) * ldq, ds_to(g));
+            gadd(d, colb + v, g);
           }
       }
     }
@@ -920,7 +934,7 @@ __global__ void __launch_bounds__(kIntThreads) integral_kernel_ds(IntegralArgs a
 #pragma unroll
       for (int d = 0; d < ND; ++d)
 #pragma unroll
-        for (int u = 0; u < NA; ++u) atomicAdd(G + d * dstr + (cola + u) * ldq, ds_to(ga[d][u]));
+        for (int u = 0; u < NA; ++u) gadd(d, cola + u, ga[d][u]);
     }
   }
 }
