@@ -170,7 +170,9 @@ typedef struct {
   double ms_screen;            /* last set_density: upload, F-tilde, pair screen    */
   double ms_collocation, ms_fgemm, ms_integrals, ms_kgemm, ms_finish; /* last build  */
   double ms_build;             /* last build, first to last event                   */
-  double ms_integrals_class[6];/* per class ss ps pp ds dp dd (FP64 lists)          */
+  double ms_integrals_class[6];/* per class ss ps pp ds dp dd (FP64 lists); builds small
+                                  enough to run all lists side by side report their
+                                  whole time in the first entry                      */
   double integrals_class[6];
   double flops_class[6];
   int64_t pairs_kept_fp32;     /* mixed form: kept (batch, pair) entries run in FP32 */
@@ -298,7 +300,7 @@ int snk_build_Vxc_device(snk_ctx *ctx, int32_t functional, double *dV, double *E
 
 /* Autotuner of the integral kernels (after snk_set_density): for every FP32
  * list of the mixed form, times the kernel on the batches of the last
- * workspace chunk for 2..128 shell pairs staged (and tile-screened) per step
+ * workspace chunk for 2..64 shell pairs staged (and tile-screened) per step
  * of a 128-point tile and keeps the fastest; the choice holds for later builds
  * and densities of the handle.  runs (optional, 12 entries: FP64 ss ps pp ds
  * dp dd, then FP32) receives the steps (the FP64 lists take their whole list

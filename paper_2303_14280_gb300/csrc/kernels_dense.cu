@@ -751,6 +751,20 @@ __global__ void abs_sum_kernel(const double* __restrict__ P, int n_dens, int64_t
   }
 }
 
+// The copies of G that lists running side by side filled, added in a fixed
+// order into the first one (HBM bound: copies + 1 passes over G).
+__global__ void sum_copies_kernel(double2* __restrict__ g, int64_t n2, int copies) {
+  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n2; e += (int64_t)gridDim.x * blockDim.x) {
+    double2 v = g[e];
+    for (int c = 1; c < copies; ++c) {
+      const double2 w = g[c * n2 + e];
+      v.x += w.x;
+      v.y += w.y;
+    }
+    g[e] = v;
+  }
+}
+
 // K_{mu nu} = (f_mu Kt_{mu nu} + f_nu Kt_{nu mu}) / 2 in every molecule block,
 // Eq. (sn_k); the row factor f_mu is the Cartesian component factor that the
 // integral kernel leaves out.
@@ -901,6 +915,13 @@ cudaError_t launch_abs_sum(cudaStream_t st, const double* P, int n_dens, int64_t
   if (n <= 0) return cudaSuccess;
   const int grid = (int)std::min<int64_t>((n + 255) / 256, 152 * 16);
   abs_sum_kernel<<<grid, 256, 0, st>>>(P, n_dens, n, out);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_sum_copies(cudaStream_t st, double* g, int64_t n, int copies) {
+  if (n <= 0 || copies < 2) return cudaSuccess;
+  const int grid = (int)std::min<int64_t>((n / 2 + 255) / 256, 152 * 16);
+  sum_copies_kernel<<<grid, 256, 0, st>>>(reinterpret_cast<double2*>(g), n / 2, copies);
   return cudaGetLastError();
 }
 

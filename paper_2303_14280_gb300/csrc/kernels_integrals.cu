@@ -139,7 +139,7 @@ __global__ void __launch_bounds__(kIntThreads) integral_kernel(IntegralArgs a) {
     const int64_t ldq = bd.ldq, dstr = (int64_t)bd.ldq * bd.nS;
     const double cx = a.xyz[3 * (bd.p0 + i)], cy = a.xyz[3 * (bd.p0 + i) + 1], cz = a.xyz[3 * (bd.p0 + i) + 2];
     const double* F = a.ws + bd.foff + i;
-    double* G = a.ws + bd.goff + i;
+    double* G = a.ws + bd.goff + a.gshift + i;
     const int* cmap = a.colmap + bd.cm_off - bd.ms0;  // indexed by global shell id
     double ga[ND][NA], fa[ND][NA];
     int cur = -1, cola = 0;
@@ -492,7 +492,7 @@ __global__ void __launch_bounds__(kF32Threads, f32_min_ctas(LA, LB)) integral_ke
       const int ldq = s_bd.ldq;
       const int64_t dstr = (int64_t)s_bd.ldq * s_bd.nS;  // density d's F / G: + d dstr
       const float* F = a.ws32 + s_bd.foff32 + i;
-      double* G64 = a.ws + s_bd.goff + i;
+      double* G64 = a.ws + s_bd.goff + a.gshift + i;
       // the FP32 contributions are added to the FP64 G with FP64 reductions;
       // each G entry of the launch has one writer (its point's thread), so
       // they land in list order and G is the same from run to run
@@ -874,7 +874,7 @@ __global__ void __launch_bounds__(kIntThreads) integral_kernel_ds(IntegralArgs a
     const ds cx = ds_from(a.xyz[3 * (bd.p0 + i)]), cy = ds_from(a.xyz[3 * (bd.p0 + i) + 1]),
              cz = ds_from(a.xyz[3 * (bd.p0 + i) + 2]);
     const double* F = a.ws + bd.foff + i;
-    double* G = a.ws + bd.goff + i;
+    double* G = a.ws + bd.goff + a.gshift + i;
     const int* cmap = a.colmap + bd.cm_off - bd.ms0;
     ds ga[ND][NA], fa[ND][NA];
     int cur = -1, cola = 0;

@@ -95,6 +95,23 @@ struct DevBuf {
 // pairs per integral tile for each class (cheap classes take longer runs);
 // the autotuner replaces these per list
 constexpr int kDefaultStep = kMaxPairsPerStep;  // pairs staged per step of the FP32 kernel, before autotuning
+// Builds with few tiles run their pair lists side by side on three streams
+// ("lanes"), each adding into a G of its own.  A list's launch lasts at least the
+// latency of one warp walking the list, and ends with the SMs that got one tile
+// more than the others; one after another the twelve lists leave much of the
+// chip idle.  A lane's lists run in order, so every copy of G has one writer at a
+// time, and the copies are added in a fixed order: K stays the same bit for bit
+// from run to run.  Measured, lists one after another / side by side (tiles of
+// 128 points per SM in brackets): 17 atoms double-FP32 (5.4) 41.7 / 28.1 ms, 12
+// atoms mixed (3.2) 10.4 / 7.2, 24 atoms FP64 (3.8) 190 / 175, 4 atoms FP64 (0.6)
+// 1.23 / 1.13, 32 atoms mixed (13.5) 66.0 / 61.0; 24 molecules (30) 42.1 / 41.4 and 96
+// atoms mixed (39) 677 / 667 would pay two more copies of G (10 GB at 96 atoms) for
+// 1.5 %.  The line lies at kLaneTiles.  Six lanes are no better than three (17 atoms
+// 28.9, 12 atoms 7.7, 16 atoms with two densities 14.5 against 15.0).
+constexpr int kLanes = 3;
+constexpr int kLaneTiles = 16;  // 128-point tiles per SM
+constexpr int kLaneOf[kNumClasses] = {0, 1, 2, 2, 1, 0};     // ss ps pp ds dp dd: about equal work per lane
+constexpr int kLaneOrder[kNumClasses] = {5, 4, 3, 0, 1, 2};  // heavier list of every lane first
 constexpr int kRunCandidates[] = {2, 4, 8, 16, 32, 64};
 // per chunk: collocation, F operands, F high tier, F rest, integral lists, K operands, K high tier, K rest
 constexpr int kPhaseEvents = 7 + kNumLists;
@@ -159,7 +176,8 @@ struct snk_ctx {
 
   struct Chunk {
     int b0 = 0, b1 = 0;
-    int64_t bytes = 0, xn = 0, goff = 0, gbytes = 0;
+    int64_t bytes = 0, xn = 0, goff = 0, gn = 0;  // gn: doubles of one copy of G
+    int copies = 1;  // copies of G: kLanes when the lists run side by side
     int max_ldq = 0, max_nS = 0, max_nB = 0, max_nBshell = 0;
     int64_t tile_off[kNumLists] = {0}, tile_n[kNumLists] = {0};
     // SNK_GEMM_SPLIT: split jobs of the F and K phases, product jobs of F hi, F lo, K hi, K lo
@@ -199,6 +217,10 @@ struct snk_ctx {
   bool graph_valid = false;
   cudaEvent_t ev_in = nullptr, ev_out = nullptr;
 
+  // streams of the lanes after the first (made with the first small build)
+  cudaStream_t lane[kLanes - 1] = {};
+  cudaEvent_t ev_fork = nullptr, ev_lane[kLanes - 1] = {};
+
   // timing
   std::vector<cudaEvent_t> events;
   cudaEvent_t ev_screen0 = nullptr, ev_screen1 = nullptr;
@@ -227,6 +249,14 @@ struct snk_ctx {
 
   ~snk_ctx() {
     if (gstream) cudaStreamSynchronize(gstream);
+    for (auto l : lane)
+      if (l) {
+        cudaStreamSynchronize(l);
+        cudaStreamDestroy(l);
+      }
+    if (ev_fork) cudaEventDestroy(ev_fork);
+    for (auto e : ev_lane)
+      if (e) cudaEventDestroy(e);
     for (auto e : events) cudaEventDestroy(e);
     for (auto e : xcev) cudaEventDestroy(e);
     if (ev_screen0) cudaEventDestroy(ev_screen0);
@@ -728,14 +758,30 @@ int screen_and_plan(snk_ctx* c) {
     return oz_operand_bytes(b.nB, b.q, S5) +
            (int64_t)nd * (oz_operand_bytes(hiS, b.q, S5) + oz_operand_bytes(loS, b.q, S5));
   };
+  // lists side by side: few tiles, and everything with kLanes copies of G in one chunk
+  int lanes = 1;
+  {
+    int64_t tiles = 0, x = 0, f = 0, af = 0, ak = 0;
+    for (int t = 0; t < nb; ++t) {
+      tiles += (bd[t].q + kPointTile - 1) / kPointTile;
+      x += (int64_t)bd[t].ldq * bd[t].nB;
+      f += (int64_t)nd * bd[t].ldq * bd[t].nS;
+      af += tc ? oz_bytes(bd[t], 0) : 0;
+      ak += tc ? oz_bytes(bd[t], 1) : 0;
+    }
+    if (tiles <= (int64_t)kLaneTiles * c->num_sms &&
+        (x + (1 + kLanes) * f) * 8 + (mixed ? f * 4 : 0) + std::max(af, ak) <= c->ws_budget)
+      lanes = kLanes;
+  }
   while (j < nb) {
     snk_ctx::Chunk ch;
     ch.b0 = j;
+    ch.copies = lanes;
     int64_t xo = 0, fo = 0, af = 0, ak = 0;
     while (j < nb) {
       // F and G of density d at foff / goff + d ldq nS
       int64_t xs = (int64_t)bd[j].ldq * bd[j].nB, fs = (int64_t)nd * bd[j].ldq * bd[j].nS;
-      int64_t bytes = (xo + xs + 2 * (fo + fs)) * 8 + (mixed ? (fo + fs) * 4 : 0);
+      int64_t bytes = (xo + xs + (1 + lanes) * (fo + fs)) * 8 + (mixed ? (fo + fs) * 4 : 0);
       const int64_t ozf = tc ? oz_bytes(bd[j], 0) : 0, ozk = tc ? oz_bytes(bd[j], 1) : 0;
       bytes += std::max(af + ozf, ak + ozk);
       if (j > ch.b0 && bytes > c->ws_budget) break;
@@ -751,7 +797,7 @@ int screen_and_plan(snk_ctx* c) {
     int64_t xcur = 0, fcur = xo, gcur = xo + fo, f32cur = 0, scur = 0;
     ch.xn = xo;
     ch.goff = gcur;
-    ch.gbytes = fo * 8;
+    ch.gn = fo;
     for (int t = ch.b0; t < ch.b1; ++t) {
       const int64_t fs = (int64_t)nd * bd[t].ldq * bd[t].nS;
       bd[t].xoff = xcur;
@@ -770,8 +816,8 @@ int screen_and_plan(snk_ctx* c) {
       ch.max_nB = std::max(ch.max_nB, bd[t].nB);
       ch.max_nBshell = std::max(ch.max_nBshell, bd[t].nBshell);
     }
-    ch.bytes = (xo + 2 * fo) * 8;
-    need = std::max(need, xo + 2 * fo);
+    ch.bytes = (xo + (1 + lanes) * fo) * 8;
+    need = std::max(need, xo + (1 + lanes) * fo);
     need_tsum = std::max(need_tsum, scur);
     if (mixed) need32 = std::max(need32, fo);
     c->chunks.push_back(ch);
@@ -794,6 +840,13 @@ int screen_and_plan(snk_ctx* c) {
   SNK_CK(c, c->Khat.ensure((size_t)std::max<int64_t>(2 * c->n_dens * s.packed, 2)));
   if (mixed && c->opt.gemm != SNK_GEMM_FP64)
     SNK_CK(c, c->P2.ensure((size_t)std::max<int64_t>(c->n_dens * s.packed, 1)));
+  if (lanes > 1 && !c->ev_fork) {
+    for (int l = 0; l < kLanes - 1; ++l) {
+      if (!c->lane[l]) SNK_CK(c, cudaStreamCreateWithFlags(&c->lane[l], cudaStreamNonBlocking));
+      if (!c->ev_lane[l]) SNK_CK(c, cudaEventCreateWithFlags(&c->ev_lane[l], cudaEventDisableTiming));
+    }
+    SNK_CK(c, cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming));
+  }
   SNK_CK(c, cudaEventRecord(c->ev_screen1, st));
   SNK_CK(c, cudaStreamSynchronize(st));
 
@@ -875,6 +928,7 @@ IntegralArgs integral_args(snk_ctx* c, size_t ci, int k) {
   a.shell_xyz = c->center.p;
   a.eps_tile = (k >= kNumClasses && tile_screen(c)) ? (float)c->opt.eps_tile : 0.f;
   a.exec = c->exec.p + 2 * k;
+  a.gshift = 0;
   a.n_dens = c->n_dens;
   a.run = c->run[k];
   a.err = c->ozerr.p;
@@ -963,23 +1017,46 @@ int enqueue_build(snk_ctx* c, cudaStream_t st, double* dK, bool timed) {
       SNK_CK(c, launch_tile_sums(st, db, nbc, ch.max_tiles, c->ws.p, c->ws32.p, c->xyz.p, nd, c->tsum.p));
       ++c->launches_build;
     }
-    SNK_CK(c, cudaMemsetAsync(c->ws.p + ch.goff, 0, ch.gbytes, st));
+    SNK_CK(c, cudaMemsetAsync(c->ws.p + ch.goff, 0, sizeof(double) * ch.gn * ch.copies, st));
     SNK_CK(c, mark());
     // G_j, Eq. (gmat) with the 3c-CP integrals of App. A, list by list
-    for (int k = 0; k < kNumLists; ++k) {
+    auto integrals = [&](int k, int lane) -> cudaError_t {
       IntegralArgs a = integral_args(c, ci, k);
-      if (a.n_tiles > 0) {
-        int grid = (int)std::min<int64_t>(c->max_ctas[k], a.n_tiles);
-        SNK_CK(c, launch_integrals(st, k, a, grid));
-        ++c->launches_build;
+      if (a.n_tiles == 0) return cudaSuccess;
+      a.gshift = lane * ch.gn;
+      ++c->launches_build;
+      return launch_integrals(lane ? c->lane[lane - 1] : st, k, a, (int)std::min<int64_t>(c->max_ctas[k], a.n_tiles));
+    };
+    if (ch.copies > 1) {
+      // side by side: the lanes start after everything before and join before G is used
+      auto lanes = [&]() -> cudaError_t {
+        cudaError_t e = cudaEventRecord(c->ev_fork, st);
+        for (int l = 0; l < kLanes - 1 && e == cudaSuccess; ++l) e = cudaStreamWaitEvent(c->lane[l], c->ev_fork, 0);
+        for (int tier = 0; tier < 2; ++tier)
+          for (int o = 0; o < kNumClasses && e == cudaSuccess; ++o)
+            e = integrals(tier * kNumClasses + kLaneOrder[o], kLaneOf[kLaneOrder[o]]);
+        for (int l = 0; l < kLanes - 1; ++l) {  // join whatever was launched
+          const cudaError_t r = cudaEventRecord(c->ev_lane[l], c->lane[l]);
+          const cudaError_t w = cudaStreamWaitEvent(st, c->ev_lane[l], 0);
+          if (e == cudaSuccess) e = r != cudaSuccess ? r : w;
+        }
+        return e;
+      };
+      SNK_CK(c, lanes());
+      SNK_CK(c, launch_sum_copies(st, c->ws.p + ch.goff, ch.gn, ch.copies));
+      ++c->launches_build;
+      for (int k = 0; k < kNumLists; ++k) SNK_CK(c, mark());
+    } else {
+      for (int k = 0; k < kNumLists; ++k) {
+        SNK_CK(c, integrals(k, 0));
+        SNK_CK(c, mark());
       }
-      SNK_CK(c, mark());
     }
     // the operands of Kt_d += G_dj^T X_j, Eq. (usym_k)
     if (tc) {
       SNK_CK(c, oz_split(ch, 1));
     } else if (df32) {
-      SNK_CK(c, launch_split_df32(st, c->ws.p + ch.goff, ch.gbytes / 8));
+      SNK_CK(c, launch_split_df32(st, c->ws.p + ch.goff, ch.gn));
       ++c->launches_build;
     }
     SNK_CK(c, mark());

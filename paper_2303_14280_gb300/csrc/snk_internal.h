@@ -276,6 +276,8 @@ cudaError_t launch_kgemm(cudaStream_t st, const BatchDesc* dbatch, int nbatch, i
 cudaError_t launch_split_df32(cudaStream_t st, double* buf, int64_t n);
 cudaError_t launch_split_df32_copy(cudaStream_t st, const double* src, int64_t n, float2* dst);
 // out = sum_d |P_d| over n_dens consecutive arrays of n doubles.
+// g[e] = (g[e] + g[e + n]) + g[e + 2n] ... over `copies` copies of n doubles (n even)
+cudaError_t launch_sum_copies(cudaStream_t st, double* g, int64_t n, int copies);
 cudaError_t launch_abs_sum(cudaStream_t st, const double* P, int n_dens, int64_t n, double* out);
 cudaError_t launch_finish(cudaStream_t st, const MolDesc* mols, int n_mol, int64_t packed,
                           const unsigned long long* Khat, const double* fcomp, double* K);
@@ -328,6 +330,7 @@ struct IntegralArgs {
   const float* prim_share;
   const float2* pair_a;    // 4 per shell pair: R_a as 3 (hi, lo) pairs, padding
   int hi_ds;
+  int64_t gshift;  // this launch's copy of G: + gshift doubles from goff
   int n_dens;      // densities: F and G of density d at foff / goff (F32: foff32) + d ldq nS
   // tile screen of the FP32 lists (eps_tile > 0): a pair is skipped on a
   // 128-point tile when bound_ab x max(sum over b's columns, sum over a's
