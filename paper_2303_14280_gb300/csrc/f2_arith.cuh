@@ -12,6 +12,9 @@
 
 namespace snk {
 
+// the f2 overload of fma below must not hide the FP64 / FP32 ones
+using ::fma;
+
 struct f2 {
   float2 v;
   f2() = default;
