@@ -36,4 +36,18 @@ __device__ __forceinline__ double exp_neg(double x, const double* tab) {
   return __hiloint2double(__double2hiint(e) - ((k >> 8) << 20), __double2loint(e));
 }
 
+// e^{-a_k r^2} of a shell's primitives for k < n <= kRadialPrims into e, zero
+// beyond the cut.
+__device__ __forceinline__ void radial_exps(const double* __restrict__ exps, int n, double r2, double cut,
+                                            const double* tab, double (&e)[kRadialPrims]) {
+#pragma unroll
+  for (int k = 0; k < kRadialPrims; ++k) {
+    e[k] = 0.0;
+    if (k < n) {
+      const double x = exps[k] * r2;
+      if (x < cut) e[k] = exp_neg(x, tab);
+    }
+  }
+}
+
 }  // namespace snk

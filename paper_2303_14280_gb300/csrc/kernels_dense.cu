@@ -278,6 +278,8 @@ __global__ void __launch_bounds__(COL_THREADS) collocation_kernel(const BatchDes
     z = xyz[3 * (bd.p0 + i) + 2];
   }
   double* X = ws + bd.xoff;
+  double e[kRadialPrims];  // of the radial group at hand
+  int group = -1;
   for (int t = t0; t < t1; ++t) {
     const int sh = bshell[bd.bshell_off + t];
     const int col = bshell_col[bd.bshell_off + t];
@@ -290,11 +292,23 @@ __global__ void __launch_bounds__(COL_THREADS) collocation_kernel(const BatchDes
     const double dx = x - B.center[3 * sh], dy = y - B.center[3 * sh + 1], dz = z - B.center[3 * sh + 2];
     const double r2 = dx * dx + dy * dy + dz * dz;
     double rad = 0.0;
-    for (int k = B.poff[sh]; k < B.poff[sh] + B.nprim[sh]; ++k) {
-      // e^{-60} ~ 9e-27: primitives that far out add nothing representable next to
-      // the batch's other values, and skipping the FP64 exponential is the saving
-      const double x = B.exps[k] * r2;
-      if (x < kColExpCut) rad = fma(B.d[k], exp_neg(x, s_exp), rad);
+    // e^{-60} ~ 9e-27: primitives that far out add nothing representable next to
+    // the batch's other values, and skipping the FP64 exponential is the saving;
+    // the shells come group by group (same centre, same exponents) and share them
+    const int p0 = B.poff[sh], np = B.nprim[sh];
+    if (np <= kRadialPrims) {
+      if (B.rgroup[sh] != group) {
+        group = B.rgroup[sh];
+        radial_exps(B.exps + p0, np, r2, kColExpCut, s_exp, e);
+      }
+#pragma unroll
+      for (int k = 0; k < kRadialPrims; ++k)
+        if (k < np) rad = fma(B.d[p0 + k], e[k], rad);
+    } else {
+      for (int k = p0; k < p0 + np; ++k) {
+        const double x = B.exps[k] * r2;
+        if (x < kColExpCut) rad = fma(B.d[k], exp_neg(x, s_exp), rad);
+      }
     }
     const double* f = B.fcomp + B.foff[sh];
     if (l == 0) {

@@ -12,6 +12,7 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <map>
 #include <memory>
 #include <mutex>
 #include <new>
@@ -130,7 +131,7 @@ struct snk_ctx {
   int run[kNumLists];  // pairs per tile, per list
 
   // geometry (device)
-  DevBuf<int> l, poff, nprim, foff, fshell, bshell, bshell_col, xfunc;
+  DevBuf<int> l, poff, nprim, foff, fshell, bshell, bshell_col, xfunc, rgroup;
   DevBuf<double> center, exps, d, fcomp, exptab, xyz, w, boys, bound, qbound, bcenter, bradius, phit_f, phit_b;
   DevBuf<float> boys_f, boys_ds, prims_ds, pair_ab, pair_a, prims_f32, prim_share;  // mixed form: FP32 and (hi, lo) copies
   DevBuf<PairHdr> pairs;
@@ -231,7 +232,7 @@ struct snk_ctx {
   // every device buffer of the handle, for binding and moving them
   template <class F>
   void for_each_buffer(F f) {
-    f(l), f(poff), f(nprim), f(foff), f(fshell), f(bshell), f(bshell_col), f(xfunc);
+    f(l), f(poff), f(nprim), f(foff), f(fshell), f(bshell), f(bshell_col), f(xfunc), f(rgroup);
     f(center), f(exps), f(d), f(fcomp), f(exptab), f(xyz), f(w), f(boys), f(bound), f(qbound), f(bcenter), f(bradius);
     f(phit_f), f(phit_b);
     f(boys_f), f(boys_ds), f(prims_ds), f(pair_ab), f(pair_a), f(prims_f32), f(prim_share);
@@ -306,6 +307,7 @@ DeviceBasis dev_basis(snk_ctx* c) {
   b.fcomp = c->fcomp.p;
   b.foff = c->foff.p;
   b.exptab = c->exptab.p;
+  b.rgroup = c->rgroup.p;
   return b;
 }
 
@@ -1298,6 +1300,38 @@ int create(int n_mol, const snk_basis* bases, const snk_grid* grids, const snk_o
       col += ncart(s.l[s.bshell[t]]);
     }
   }
+  // shells of one centre with the same exponents (an SP shell's s and p, the s, p
+  // and d shells of an even-tempered set) form a radial group, named by its first
+  // shell; the collocation takes a batch's shells group by group and forms each
+  // e^{-a r^2} once
+  std::vector<int> rgroup(std::max(s.ns, 1), 0);
+  {
+    std::vector<int> order(s.ns), col(s.ns, -1), sh;
+    for (const auto& M : s.mols) {
+      std::map<std::vector<double>, int> seen;
+      for (int a = M.ms0; a < M.ms0 + M.ns; ++a) {
+        const int n = s.poff[a + 1] - s.poff[a];
+        std::vector<double> key(s.center.begin() + 3 * a, s.center.begin() + 3 * a + 3);
+        key.insert(key.end(), s.exps.begin() + s.poff[a], s.exps.begin() + s.poff[a + 1]);
+        rgroup[a] = n <= kRadialPrims ? seen.emplace(key, a).first->second : a;
+        order[a] = a;
+      }
+      std::stable_sort(order.begin() + M.ms0, order.begin() + M.ms0 + M.ns,
+                       [&](int x, int y) { return rgroup[x] < rgroup[y]; });
+    }
+    for (int j = 0; j < c->nbatch; ++j) {
+      const Setup::Mol& M = s.mols[s.bmol[j]];
+      const int t0 = s.bshell_off[j], t1 = s.bshell_off[j + 1];
+      sh.assign(s.bshell.begin() + t0, s.bshell.begin() + t1);
+      for (int t = t0; t < t1; ++t) col[s.bshell[t]] = s.bshell_col[t];
+      for (int k = M.ms0, t = t0; k < M.ms0 + M.ns; ++k)
+        if (col[order[k]] >= 0) {
+          s.bshell[t] = order[k];
+          s.bshell_col[t++] = col[order[k]];
+        }
+      for (int a : sh) col[a] = -1;
+    }
+  }
   std::vector<MolDesc> hm(s.n_mol);
   for (int m = 0; m < s.n_mol; ++m) {
     const Setup::Mol& M = s.mols[m];
@@ -1395,6 +1429,7 @@ int create(int n_mol, const snk_basis* bases, const snk_grid* grids, const snk_o
          SNK_CK(cp, upload(cp->bshell, s.bshell, st));
          SNK_CK(cp, upload(cp->bshell_col, s.bshell_col, st));
          SNK_CK(cp, upload(cp->xfunc, s.xfunc, st));
+         SNK_CK(cp, upload(cp->rgroup, rgroup, st));
          SNK_CK(cp, upload(cp->boys, s.boys, st));
          SNK_CK(cp, upload(cp->mols, hm, st));
          SNK_CK(cp, cudaStreamSynchronize(st));

@@ -49,6 +49,7 @@ __device__ __forceinline__ double khat_value(const unsigned long long* e) {
 // row: F_{L+m}(T_k)/m! for m = 0..7, exp(-T_k), T_k.
 // Table of the collocation kernels' e^{-x}: 2^{-j/256}.
 constexpr int kExpTable = 256;
+constexpr int kRadialPrims = 4;  // primitives whose e^{-a r^2} a thread keeps for the next shell of the group
 
 constexpr double kBoysH = 0.1;
 constexpr double kBoysTMax = 50.0;
@@ -214,6 +215,7 @@ void host_boys(int nmax, double T, double* F);
 // ---------------------------------------------------------------- kernels
 
 struct DeviceBasis {
+  const int* rgroup;     // shells of a group share centre and exponents (at most kRadialPrims of them)
   const double* exptab;  // 2^{-j/kExpTable} of exp_neg
   const int* l;
   const int* poff;
