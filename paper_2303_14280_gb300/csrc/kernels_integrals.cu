@@ -59,7 +59,11 @@ static_assert(kBoysTMax == 50.0, "kBoysTMaxBits encodes 50.0");
 template <int L>
 __device__ __forceinline__ void boys_seeds(double T, double pref, double pref_far, const double* tab, double* S) {
   if (__double_as_longlong(T) < kBoysTMaxBits) {
-    const int k = __float2int_rn(__double2float_rn(T) * (float)(1.0 / kBoysH));
+    // T in FP32 by integer operations: the conversion runs on the FP64 pipe (24
+    // atoms, FP64 integrals 156.7 -> 155.6 ms)
+    const int hi = max(__double2hiint(T), 0x38000000) - 0x38000000;  // 0 below 2^-127
+    const float tf = __int_as_float((int)__funnelshift_l((unsigned)__double2loint(T), (unsigned)hi, 3));
+    const int k = __float2int_rn(tf * (float)(1.0 / kBoysH));
     const double* row = tab + k * kBoysCols;
     const double x = row[kBoysCols - 1] - T;  // T_k - T, |x| <= 0.05
     double f = row[7];
