@@ -276,11 +276,11 @@ __device__ __forceinline__ void boys_seeds_f32(f2 nT, f2 pref, f2 pref_far, uint
 
 // The FP64 value of v by integer operations: the conversion instruction runs on
 // the FP64 pipe (2 lanes per clock and SM), which the G updates kept 20-35 %
-// busy.  Below 2^-126 gives zero; infinities and NaN become numbers of 2^128
-// and more, outside the range the K accumulator accepts.
+// busy.  Magnitudes below 2^-126 give zero; infinities and NaN stay what they are.
 __device__ __forceinline__ double f32_to_f64_bits(float v) {
   const uint32_t b = __float_as_uint(v), m = b & 0x7fffffffu;
-  const uint32_t hi = (b & 0x80000000u) | ((m >> 3) + 0x38000000u);
+  uint32_t hi = (b & 0x80000000u) | ((m >> 3) + 0x38000000u);
+  if (m >= 0x7f800000u) hi |= 0x7ff00000u;
   return m < 0x00800000u ? 0.0 : __hiloint2double((int)hi, (int)(b << 29));
 }
 
