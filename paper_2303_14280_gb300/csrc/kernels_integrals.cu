@@ -119,6 +119,18 @@ __device__ __forceinline__ void pair_xi(const PairHdr& h, const PrimPair* __rest
   C::hrr(acc, h.ABx, h.ABy, h.ABz, xi);
 }
 
+// Work item t of the FP64 / ds lists: tile t mod n_tiles, range t / n_tiles of its
+// list.
+__device__ __forceinline__ Tile tile_part(const IntegralArgs& a, int t) {
+  Tile tile = a.tiles[t % a.n_tiles];
+  if (a.parts > 1) {
+    const int64_t n = tile.k1 - tile.k0, part = t / a.n_tiles;
+    tile.k1 = tile.k0 + (int)(n * (part + 1) / a.parts);
+    tile.k0 += (int)(n * part / a.parts);
+  }
+  return tile;
+}
+
 // ND densities share every Xi block: F and G of density d sit d ldq nS
 // doubles after the batch's first block.
 template <int LA, int LB, int ND>
@@ -135,15 +147,15 @@ __global__ void __launch_bounds__(kIntThreads) integral_kernel(IntegralArgs a) {
     __syncthreads();
     const int t = s_tile;
     __syncthreads();
-    if (t >= a.n_tiles) break;
-    const Tile tile = a.tiles[t];
+    if (t >= a.n_tiles * a.parts) break;
+    const Tile tile = tile_part(a, t);
     const BatchDesc bd = a.batches[tile.batch];
     const int i = tile.i0 + threadIdx.x;
     if (i >= bd.q) continue;
     const int64_t ldq = bd.ldq, dstr = (int64_t)bd.ldq * bd.nS;
     const double cx = a.xyz[3 * (bd.p0 + i)], cy = a.xyz[3 * (bd.p0 + i) + 1], cz = a.xyz[3 * (bd.p0 + i) + 2];
     const double* F = a.ws + bd.foff + i;
-    double* G = a.ws + bd.goff + a.gshift + i;
+    double* G = a.ws + bd.goff + a.gshift + (t / a.n_tiles) * a.gpart + i;
     const int* cmap = a.colmap + bd.cm_off - bd.ms0;  // indexed by global shell id
     double ga[ND][NA], fa[ND][NA];
     int cur = -1, cola = 0;
@@ -867,8 +879,8 @@ __global__ void __launch_bounds__(kIntThreads) integral_kernel_ds(IntegralArgs a
     __syncthreads();
     const int t = s_tile;
     __syncthreads();
-    if (t >= a.n_tiles) break;
-    const Tile tile = a.tiles[t];
+    if (t >= a.n_tiles * a.parts) break;
+    const Tile tile = tile_part(a, t);
     const BatchDesc bd = a.batches[tile.batch];
     int i = tile.i0 + threadIdx.x;
     const bool act = i < bd.q;
@@ -878,7 +890,7 @@ __global__ void __launch_bounds__(kIntThreads) integral_kernel_ds(IntegralArgs a
     const ds cx = ds_from(a.xyz[3 * (bd.p0 + i)]), cy = ds_from(a.xyz[3 * (bd.p0 + i) + 1]),
              cz = ds_from(a.xyz[3 * (bd.p0 + i) + 2]);
     const double* F = a.ws + bd.foff + i;
-    double* G = a.ws + bd.goff + a.gshift + i;
+    double* G = a.ws + bd.goff + a.gshift + (t / a.n_tiles) * a.gpart + i;
     const int* cmap = a.colmap + bd.cm_off - bd.ms0;
     ds ga[ND][NA], fa[ND][NA];
     int cur = -1, cola = 0;

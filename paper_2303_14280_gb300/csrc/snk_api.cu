@@ -111,6 +111,11 @@ constexpr int kDefaultStep = kMaxPairsPerStep;  // pairs staged per step of the 
 // 28.9, 12 atoms 7.7, 16 atoms with two densities 14.5 against 15.0).
 constexpr int kLanes = 3;
 constexpr int kLaneTiles = 16;  // 128-point tiles per SM
+// With less than three tiles per SM the FP64 / double-FP32 lists are also cut into
+// ranges, up to kMaxParts, until there are about three work items per SM: a warp's
+// time is the latency of its range (an FP64 multiply-add takes about 60 clocks).  4
+// atoms (94 tiles), FP64: lists 0.69 -> 0.45 ms.
+constexpr int kMaxParts = 4;
 constexpr int kLaneOf[kNumClasses] = {0, 1, 2, 2, 1, 0};     // ss ps pp ds dp dd: about equal work per lane
 constexpr int kLaneOrder[kNumClasses] = {5, 4, 3, 0, 1, 2};  // heavier list of every lane first
 constexpr int kRunCandidates[] = {2, 4, 8, 16, 32, 64};
@@ -178,7 +183,8 @@ struct snk_ctx {
   struct Chunk {
     int b0 = 0, b1 = 0;
     int64_t bytes = 0, xn = 0, goff = 0, gn = 0;  // gn: doubles of one copy of G
-    int copies = 1;  // copies of G: kLanes when the lists run side by side
+    int parts = 1;   // ranges of every FP64 / ds list that add into copies of G of their own
+    int copies = 1;  // copies of G: kLanes x parts when the lists run side by side
     int max_ldq = 0, max_nS = 0, max_nB = 0, max_nBshell = 0;
     int64_t tile_off[kNumLists] = {0}, tile_n[kNumLists] = {0};
     // SNK_GEMM_SPLIT: split jobs of the F and K phases, product jobs of F hi, F lo, K hi, K lo
@@ -761,7 +767,7 @@ int screen_and_plan(snk_ctx* c) {
            (int64_t)nd * (oz_operand_bytes(hiS, b.q, S5) + oz_operand_bytes(loS, b.q, S5));
   };
   // lists side by side: few tiles, and everything with kLanes copies of G in one chunk
-  int lanes = 1;
+  int lanes = 1, parts = 1;
   {
     int64_t tiles = 0, x = 0, f = 0, af = 0, ak = 0;
     for (int t = 0; t < nb; ++t) {
@@ -771,19 +777,22 @@ int screen_and_plan(snk_ctx* c) {
       af += tc ? oz_bytes(bd[t], 0) : 0;
       ak += tc ? oz_bytes(bd[t], 1) : 0;
     }
+    const int most =
+        (int)std::max<int64_t>(1, std::min<int64_t>(kMaxParts, 3 * (int64_t)c->num_sms / std::max<int64_t>(tiles, 1)));
     if (tiles <= (int64_t)kLaneTiles * c->num_sms &&
-        (x + (1 + kLanes) * f) * 8 + (mixed ? f * 4 : 0) + std::max(af, ak) <= c->ws_budget)
-      lanes = kLanes;
+        (x + (1 + kLanes * most) * f) * 8 + (mixed ? f * 4 : 0) + std::max(af, ak) <= c->ws_budget)
+      lanes = kLanes, parts = most;
   }
   while (j < nb) {
     snk_ctx::Chunk ch;
     ch.b0 = j;
-    ch.copies = lanes;
+    ch.parts = parts;
+    ch.copies = lanes * parts;
     int64_t xo = 0, fo = 0, af = 0, ak = 0;
     while (j < nb) {
       // F and G of density d at foff / goff + d ldq nS
       int64_t xs = (int64_t)bd[j].ldq * bd[j].nB, fs = (int64_t)nd * bd[j].ldq * bd[j].nS;
-      int64_t bytes = (xo + xs + (1 + lanes) * (fo + fs)) * 8 + (mixed ? (fo + fs) * 4 : 0);
+      int64_t bytes = (xo + xs + (1 + lanes * parts) * (fo + fs)) * 8 + (mixed ? (fo + fs) * 4 : 0);
       const int64_t ozf = tc ? oz_bytes(bd[j], 0) : 0, ozk = tc ? oz_bytes(bd[j], 1) : 0;
       bytes += std::max(af + ozf, ak + ozk);
       if (j > ch.b0 && bytes > c->ws_budget) break;
@@ -818,8 +827,8 @@ int screen_and_plan(snk_ctx* c) {
       ch.max_nB = std::max(ch.max_nB, bd[t].nB);
       ch.max_nBshell = std::max(ch.max_nBshell, bd[t].nBshell);
     }
-    ch.bytes = (xo + (1 + lanes) * fo) * 8;
-    need = std::max(need, xo + (1 + lanes) * fo);
+    ch.bytes = (xo + (1 + lanes * parts) * fo) * 8;
+    need = std::max(need, xo + (1 + lanes * parts) * fo);
     need_tsum = std::max(need_tsum, scur);
     if (mixed) need32 = std::max(need32, fo);
     c->chunks.push_back(ch);
@@ -931,6 +940,8 @@ IntegralArgs integral_args(snk_ctx* c, size_t ci, int k) {
   a.eps_tile = (k >= kNumClasses && tile_screen(c)) ? (float)c->opt.eps_tile : 0.f;
   a.exec = c->exec.p + 2 * k;
   a.gshift = 0;
+  a.parts = k < kNumClasses ? ch.parts : 1;
+  a.gpart = ch.gn;
   a.n_dens = c->n_dens;
   a.run = c->run[k];
   a.err = c->ozerr.p;
@@ -1025,9 +1036,9 @@ int enqueue_build(snk_ctx* c, cudaStream_t st, double* dK, bool timed) {
     auto integrals = [&](int k, int lane) -> cudaError_t {
       IntegralArgs a = integral_args(c, ci, k);
       if (a.n_tiles == 0) return cudaSuccess;
-      a.gshift = lane * ch.gn;
+      a.gshift = (int64_t)lane * ch.parts * ch.gn;
       ++c->launches_build;
-      return launch_integrals(lane ? c->lane[lane - 1] : st, k, a, (int)std::min<int64_t>(c->max_ctas[k], a.n_tiles));
+      return launch_integrals(lane ? c->lane[lane - 1] : st, k, a, (int)std::min<int64_t>(c->max_ctas[k], (int64_t)a.n_tiles * a.parts));
     };
     if (ch.copies > 1) {
       // side by side: the lanes start after everything before and join before G is used

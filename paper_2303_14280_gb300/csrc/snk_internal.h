@@ -333,6 +333,10 @@ struct IntegralArgs {
   const float2* pair_a;    // 4 per shell pair: R_a as 3 (hi, lo) pairs, padding
   int hi_ds;
   int64_t gshift;  // this launch's copy of G: + gshift doubles from goff
+  // FP64 / ds lists: a tile's list is cut into `parts` ranges, each adding into a
+  // copy of G of its own, gpart doubles after the one before
+  int parts;
+  int64_t gpart;
   int n_dens;      // densities: F and G of density d at foff / goff (F32: foff32) + d ldq nS
   // tile screen of the FP32 lists (eps_tile > 0): a pair is skipped on a
   // 128-point tile when bound_ab x max(sum over b's columns, sum over a's
