@@ -752,7 +752,6 @@ int screen_and_plan(snk_ctx* c) {
 
   // chunks under the workspace budget (Alg. 1): X, F, G in doubles, plus the
   // FP32 copies of F and G in the mixed form
-  int j = 0;
   int64_t need = 1, need32 = 1, need_arena = 0, need_tsum = 1;
   const int nd = c->n_dens;
   // slice-arena bytes of one batch for the F phase (X_j and P[S_j, B_j] per
@@ -783,67 +782,86 @@ int screen_and_plan(snk_ctx* c) {
         (x + (1 + kLanes * most) * f) * 8 + (mixed ? f * 4 : 0) + std::max(af, ak) <= c->ws_budget)
       lanes = kLanes, parts = most;
   }
-  while (j < nb) {
-    snk_ctx::Chunk ch;
-    ch.b0 = j;
-    ch.parts = parts;
-    ch.copies = lanes * parts;
-    int64_t xo = 0, fo = 0, af = 0, ak = 0;
+  auto plan_chunks = [&]() {
+    c->chunks.clear();
+    need = need32 = need_tsum = 1;
+    need_arena = 0;
+    int j = 0;
     while (j < nb) {
-      // F and G of density d at foff / goff + d ldq nS
-      int64_t xs = (int64_t)bd[j].ldq * bd[j].nB, fs = (int64_t)nd * bd[j].ldq * bd[j].nS;
-      int64_t bytes = (xo + xs + (1 + lanes * parts) * (fo + fs)) * 8 + (mixed ? (fo + fs) * 4 : 0);
-      const int64_t ozf = tc ? oz_bytes(bd[j], 0) : 0, ozk = tc ? oz_bytes(bd[j], 1) : 0;
-      bytes += std::max(af + ozf, ak + ozk);
-      if (j > ch.b0 && bytes > c->ws_budget) break;
-      xo += xs;
-      fo += fs;
-      af += ozf;
-      ak += ozk;
-      ++j;
+      snk_ctx::Chunk ch;
+      ch.b0 = j;
+      ch.parts = parts;
+      ch.copies = lanes * parts;
+      int64_t xo = 0, fo = 0, af = 0, ak = 0;
+      while (j < nb) {
+        // F and G of density d at foff / goff + d ldq nS
+        int64_t xs = (int64_t)bd[j].ldq * bd[j].nB, fs = (int64_t)nd * bd[j].ldq * bd[j].nS;
+        int64_t bytes = (xo + xs + (1 + lanes * parts) * (fo + fs)) * 8 + (mixed ? (fo + fs) * 4 : 0);
+        const int64_t ozf = tc ? oz_bytes(bd[j], 0) : 0, ozk = tc ? oz_bytes(bd[j], 1) : 0;
+        bytes += std::max(af + ozf, ak + ozk);
+        if (j > ch.b0 && bytes > c->ws_budget) break;
+        xo += xs;
+        fo += fs;
+        af += ozf;
+        ak += ozk;
+        ++j;
+      }
+      ch.arena_bytes = std::max(af, ak);
+      need_arena = std::max(need_arena, ch.arena_bytes);
+      ch.b1 = j;
+      int64_t xcur = 0, fcur = xo, gcur = xo + fo, f32cur = 0, scur = 0;
+      ch.xn = xo;
+      ch.goff = gcur;
+      ch.gn = fo;
+      for (int t = ch.b0; t < ch.b1; ++t) {
+        const int64_t fs = (int64_t)nd * bd[t].ldq * bd[t].nS;
+        bd[t].xoff = xcur;
+        xcur += (int64_t)bd[t].ldq * bd[t].nB;
+        bd[t].foff = fcur;
+        bd[t].goff = gcur;
+        bd[t].foff32 = f32cur;
+        bd[t].ssoff = scur;
+        scur += (int64_t)(bd[t].ldq / kPointTile) * (bd[t].nS + 4);
+        ch.max_tiles = std::max(ch.max_tiles, bd[t].ldq / kPointTile);
+        fcur += fs;
+        gcur += fs;
+        f32cur += fs;
+        ch.max_ldq = std::max(ch.max_ldq, bd[t].ldq);
+        ch.max_nS = std::max(ch.max_nS, bd[t].nS);
+        ch.max_nB = std::max(ch.max_nB, bd[t].nB);
+        ch.max_nBshell = std::max(ch.max_nBshell, bd[t].nBshell);
+      }
+      ch.bytes = (xo + (1 + lanes * parts) * fo) * 8;
+      need = std::max(need, xo + (1 + lanes * parts) * fo);
+      need_tsum = std::max(need_tsum, scur);
+      if (mixed) need32 = std::max(need32, fo);
+      c->chunks.push_back(ch);
     }
-    ch.arena_bytes = std::max(af, ak);
-    need_arena = std::max(need_arena, ch.arena_bytes);
-    ch.b1 = j;
-    int64_t xcur = 0, fcur = xo, gcur = xo + fo, f32cur = 0, scur = 0;
-    ch.xn = xo;
-    ch.goff = gcur;
-    ch.gn = fo;
-    for (int t = ch.b0; t < ch.b1; ++t) {
-      const int64_t fs = (int64_t)nd * bd[t].ldq * bd[t].nS;
-      bd[t].xoff = xcur;
-      xcur += (int64_t)bd[t].ldq * bd[t].nB;
-      bd[t].foff = fcur;
-      bd[t].goff = gcur;
-      bd[t].foff32 = f32cur;
-      bd[t].ssoff = scur;
-      scur += (int64_t)(bd[t].ldq / kPointTile) * (bd[t].nS + 4);
-      ch.max_tiles = std::max(ch.max_tiles, bd[t].ldq / kPointTile);
-      fcur += fs;
-      gcur += fs;
-      f32cur += fs;
-      ch.max_ldq = std::max(ch.max_ldq, bd[t].ldq);
-      ch.max_nS = std::max(ch.max_nS, bd[t].nS);
-      ch.max_nB = std::max(ch.max_nB, bd[t].nB);
-      ch.max_nBshell = std::max(ch.max_nBshell, bd[t].nBshell);
-    }
-    ch.bytes = (xo + (1 + lanes * parts) * fo) * 8;
-    need = std::max(need, xo + (1 + lanes * parts) * fo);
-    need_tsum = std::max(need_tsum, scur);
-    if (mixed) need32 = std::max(need32, fo);
-    c->chunks.push_back(ch);
+  };
+  auto reserve = [&]() -> cudaError_t {
+    cudaError_t e = c->ws.ensure((size_t)need);
+    if (e == cudaSuccess && mixed) e = c->ws32.ensure((size_t)need32);
+    if (e == cudaSuccess && tile_screen(c)) e = c->tsum.ensure((size_t)need_tsum);
+    if (e == cudaSuccess && tc) e = c->arena.ensure((size_t)std::max<int64_t>(need_arena, 16));
+    return e;
+  };
+  plan_chunks();
+  cudaError_t res = reserve();
+  if (res == cudaErrorMemoryAllocation && lanes > 1) {  // no room for the copies of G: one list after another
+    cudaGetLastError();
+    c->ws.release();
+    lanes = parts = 1;
+    plan_chunks();
+    res = reserve();
   }
-  SNK_CK(c, c->ws.ensure((size_t)need));
-  if (mixed) SNK_CK(c, c->ws32.ensure((size_t)need32));
+  SNK_CK(c, res);
   SNK_CK(c, upload(c->batch, bd, st));
-  if (tile_screen(c)) SNK_CK(c, c->tsum.ensure((size_t)need_tsum));
   SNK_CK(c, c->exec.ensure(2 * kNumLists));
   SNK_CK(c, c->ozerr.ensure(1));  // device error flag of the products and the K accumulator
   SNK_CK(c, cudaMemsetAsync(c->ozerr.p, 0, sizeof(int), st));
   double tc_flops = 0.0;
   if (tc) {
     if (int rc = plan_tc(c, &tc_flops)) return rc;
-    SNK_CK(c, c->arena.ensure((size_t)std::max<int64_t>(need_arena, 16)));
   }
 
   if (int rc = make_tiles(c, st)) return rc;

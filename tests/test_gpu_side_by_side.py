@@ -50,3 +50,34 @@ def test_lists_side_by_side_match_lists_in_turn(form, n_atoms, n_r):
     K2, _ = build(dens=2)
     # two densities share one screen (sum of |P|): more pairs kept, below the screen's threshold
     assert np.max(np.abs(K2[0] - K)) <= tol + 1e-8 and np.max(np.abs(K2[1] - 0.5 * K)) <= tol + 1e-8
+
+
+def test_no_room_for_the_copies_falls_back_to_lists_in_turn():
+    """An allocator that refuses the workspace with copies of G: the build runs
+    its lists one after another in the smaller one, with the same K."""
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_2303_14280_gb300 as snk
+    p = synth.cluster(7, 47, n_r=20, n_theta=4, n_phi=9, n_occ=4)
+    eng = snk.Engine(p.basis, p.grid, batch_max=200)
+    eng.set_density(p.P)
+    K = eng.build_K()
+    with_copies = eng.stats()["workspace_bytes"]
+    eng.close()
+    eng = snk.Engine(p.basis, p.grid, batch_max=200)
+    blocks = {}
+
+    def alloc(nbytes):
+        if nbytes >= with_copies:
+            return 0
+        t = torch.empty(nbytes, dtype=torch.uint8, device="cuda")
+        blocks[t.data_ptr()] = t
+        return t.data_ptr()
+
+    eng.set_allocator(alloc, lambda ptr: blocks.pop(ptr, None))
+    eng.set_density(p.P)
+    K1 = eng.build_K()
+    assert eng.stats()["workspace_bytes"] < with_copies
+    eng.close()
+    assert np.max(np.abs(K1 - K)) <= 1e-12 * np.max(np.abs(K))
