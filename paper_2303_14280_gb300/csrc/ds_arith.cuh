@@ -91,6 +91,8 @@ __device__ __forceinline__ ds fma(ds x, ds y, ds z) {
 //   dot2(a, b, c, d)           a b + c d
 //   dot2_add<m>(a, b, c, d, x) a b + c d + m x, m = 1, 2, 3
 //   acc_add / acc_mac          running sums M += x, M += a b;  acc_get reads one
+//   acc_lead                   acc_add of a primitive pair's leading scalar; in double
+//                              acc_mac by the prefactor, which the FP64 seeds leave out
 //
 // In ds the products of a dot product stay unnormalised (p + e, 4 operations
 // each), the leading parts are added error-free and everything small is
@@ -112,6 +114,11 @@ template <class T>
 __device__ __forceinline__ void acc_add(T& s, T x) {
   s += x;
 }
+template <class A, class R>
+__device__ __forceinline__ void acc_lead(A& s, const R&, const R& x) {
+  acc_add(s, x);
+}
+__device__ __forceinline__ void acc_lead(double& s, double c, double x) { s = ::fma(c, x, s); }
 template <class T>
 __device__ __forceinline__ void acc_mac(T& s, T a, T b) {
   s = fma(a, b, s);

@@ -93,7 +93,7 @@ def scalars(la, lb):
 
 
 def gen_prim(la, lb):
-    """Seeds of one primitive pair into M; c(i, j) = sigma^i kappa^j are arguments."""
+    """Seeds of one primitive pair into M; c(i, j) = sigma^i kappa^j are arguments (FP64: times the prefactor)."""
     L = la + lb
     ms = scalars(la, lb)
     need = set()
@@ -117,7 +117,7 @@ def gen_prim(la, lb):
             c.add += 1
     for n, (i, j, s) in enumerate(ms):
         if i == 0 and j == 0:
-            lines.append(f"acc_add(M[{n}], w0_{s});")
+            lines.append(f"acc_lead(M[{n}], c.c00, w0_{s});")
             c.add += 1
         else:
             lines.append(f"acc_mac(M[{n}], c.c{i}{j}, w{i + j}_{s});")
@@ -296,8 +296,10 @@ def main(out=sys.stdout):
     w("// (App. A, Eq. vrr) with the primitive pairs contracted into scalars first (the\n")
     w("// derivation is in gen_os.py), and the HRR (Eq. hrr), with the operation counts.\n")
     w("#pragma once\n\nnamespace snk {\n\n")
-    w("// sigma^i kappa^j of one primitive pair, c<i><j>; a class reads those with i + 2j <= L\n")
-    w("template <typename R> struct OsCoef {\n  R c10, c20, c30, c40, c01, c11, c21, c02;\n};\n\n")
+    w("// sigma^i kappa^j of one primitive pair, c<i><j>; a class reads those with i + 2j <= L.\n")
+    w("// FP64: times the primitive pair's prefactor, c00 the prefactor itself; elsewhere the\n")
+    w("// seeds carry the prefactor and c00 is not read (acc_lead)\n")
+    w("template <typename R> struct OsCoef {\n  R c00, c10, c20, c30, c40, c01, c11, c21, c02;\n};\n\n")
     w("template <int LA, int LB> struct OsClass;\n\n")
     for (la, lb) in CLASSES:
         pl, pc, m_index = gen_prim(la, lb)

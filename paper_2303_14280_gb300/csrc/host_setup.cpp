@@ -465,18 +465,33 @@ int build_setup_one(const snk_basis* basis, const snk_grid* grid, const snk_opti
 
 // Boys interpolation tables of the FP64 and FP32 integral kernels.
 void build_boys_tables(Setup* s) {
-  // Boys table per L: F_{L+m}(T_k)/m!, exp(-T_k), T_k
+  // FP64 table per L: economised Taylor coefficients, exp(-T_k), T_k.  With y = x / h,
+  // y^7 = (112 y^5 - 56 y^3 + 7 y + T_7) / 64 and
+  // y^8 = (256 y^6 - 160 y^4 + 32 y^2 - 1 + T_8) / 128; T_7 and T_8 are dropped.
   s->boys.assign((size_t)(kBoysLMax + 1) * kBoysRows * kBoysCols, 0.0);
-  double F[kBoysLMax + kBoysTerms + 1];
-  double invfact[kBoysTerms];
+  constexpr int kTaylor = 9;
+  static_assert(kBoysTerms == 7 && kTaylor > kBoysTermsDs, "x^7 and x^8 are folded into x^0 .. x^6");
+  double F[kBoysLMax + kTaylor];
+  double invfact[kTaylor];
   invfact[0] = 1.0;
-  for (int m = 1; m < kBoysTerms; ++m) invfact[m] = invfact[m - 1] / m;
+  for (int m = 1; m < kTaylor; ++m) invfact[m] = invfact[m - 1] / m;
+  const double h2 = 0.25 * kBoysH * kBoysH, h4 = h2 * h2;
   for (int k = 0; k < kBoysRows; ++k) {
     double T = k * kBoysH;
-    host_boys(kBoysLMax + kBoysTerms, T, F);
+    host_boys(kBoysLMax + kTaylor - 1, T, F);
     for (int L = 0; L <= kBoysLMax; ++L) {
       double* row = &s->boys[((size_t)L * kBoysRows + k) * kBoysCols];
-      for (int m = 0; m < kBoysTerms; ++m) row[m] = F[L + m] * invfact[m];
+      double c[kTaylor];
+      for (int m = 0; m < kTaylor; ++m) c[m] = F[L + m] * invfact[m];
+      const double c7 = c[7] / 64.0, c8 = c[8] / 128.0;
+      c[0] -= c8 * h4 * h4;
+      c[1] += 7.0 * c7 * h4 * h2;
+      c[2] += 32.0 * c8 * h4 * h2;
+      c[3] -= 56.0 * c7 * h4;
+      c[4] -= 160.0 * c8 * h4;
+      c[5] += 112.0 * c7 * h2;
+      c[6] += 256.0 * c8 * h2;
+      for (int m = 0; m < kBoysTerms; ++m) row[m] = c[m];
       row[kBoysTerms] = std::exp(-T);
       row[kBoysTerms + 1] = T;
     }
@@ -484,24 +499,24 @@ void build_boys_tables(Setup* s) {
   // ds table of the mixed form: nodes T_k rounded to (hi, lo) float pairs and
   // the values at those nodes split the same way, so that T_k - T is exact in
   // ds arithmetic
-  s->boys_ds.assign((size_t)(kBoysLMax + 1) * kBoysRows * kBoysCols * 2, 0.0f);
-  for (int k = 0; k < kBoysRows; ++k) {
-    const double T0 = k * kBoysH;
+  s->boys_ds.assign((size_t)(kBoysLMax + 1) * kBoysRowsDs * kBoysColsDs * 2, 0.0f);
+  for (int k = 0; k < kBoysRowsDs; ++k) {
+    const double T0 = k * kBoysHDs;
     const float th = (float)T0;
     const float tl = (float)(T0 - (double)th);
     const double T = (double)th + (double)tl;
-    host_boys(kBoysLMax + kBoysTerms, T, F);
+    host_boys(kBoysLMax + kBoysTermsDs, T, F);
     for (int L = 0; L <= kBoysLMax; ++L) {
-      float* row = &s->boys_ds[(((size_t)L * kBoysRows + k) * kBoysCols) * 2];
-      double v[kBoysCols];
-      for (int m = 0; m < kBoysTerms; ++m) v[m] = F[L + m] * invfact[m];
-      v[kBoysTerms] = std::exp(-T);
-      for (int m = 0; m < kBoysTerms + 1; ++m) {
+      float* row = &s->boys_ds[(((size_t)L * kBoysRowsDs + k) * kBoysColsDs) * 2];
+      double v[kBoysColsDs];
+      for (int m = 0; m < kBoysTermsDs; ++m) v[m] = F[L + m] * invfact[m];
+      v[kBoysTermsDs] = std::exp(-T);
+      for (int m = 0; m < kBoysTermsDs + 1; ++m) {
         row[2 * m] = (float)v[m];
         row[2 * m + 1] = (float)(v[m] - (double)row[2 * m]);
       }
-      row[2 * (kBoysTerms + 1)] = th;
-      row[2 * (kBoysTerms + 1) + 1] = tl;
+      row[2 * (kBoysTermsDs + 1)] = th;
+      row[2 * (kBoysTermsDs + 1) + 1] = tl;
     }
   }
   // FP32 table of the mixed form: nodes at the float values fl32(k * 0.05f)

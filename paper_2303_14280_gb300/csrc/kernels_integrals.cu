@@ -52,12 +52,18 @@ constexpr unsigned long long kCopyWaitNs = 2000000000ull;  // 2 s per wait on a 
 constexpr long long kBoysTMaxBits = 0x4049000000000000LL;  // bit pattern of 50.0
 static_assert(kBoysTMax == 50.0, "kBoysTMaxBits encodes 50.0");
 
-// S_n = pref * F_n(T), n = 0..L (Eq. boys).  Below T = 50: an 8-term Taylor
-// expansion of F_L about the nearest table node (dF_n/dT = -F_{n+1}) and the
-// downward recursion F_n = (2T F_{n+1} + e^{-T}) / (2n+1); above: F_0 =
-// sqrt(pi/T)/2 and F_{n+1} = (2n+1) F_n / (2T) (e^{-T} < 2e-22 is dropped).
+// S_n = F_n(T), n = 0..L (Eq. boys).  Below T = 50: F_L by a polynomial of
+// degree 6 about the nearest table node (the Taylor series, dF_n/dT = -F_{n+1},
+// economised) and the downward recursion F_n = (2T F_{n+1} + e^{-T}) / (2n+1);
+// above: F_0 = sqrt(pi/T)/2 and F_{n+1} = (2n+1) F_n / (2T) (e^{-T} < 2e-22 is
+// dropped).  Every FP64 operation costs the whole SM 16 clocks per warp, so: the
+// primitive pair's prefactor is in its contraction coefficients, where it rides
+// on a multiply-add; 2T is one integer addition to T's exponent.  Against eight
+// Taylor terms on |x| <= 0.05 and seeds with the prefactor: 24 atoms 176.0 ->
+// 168.8 ms per build, 4 atoms 0.780 -> 0.743 ms; largest error of a seed times its
+// prefactor 1.4e-15 -> 6.8e-16 relative, rms at most 2.0e-16 -> 1.5e-16.
 template <int L>
-__device__ __forceinline__ void boys_seeds(double T, double pref, double pref_far, const double* tab, double* S) {
+__device__ __forceinline__ void boys_seeds(double T, const double* tab, double* S) {
   if (__double_as_longlong(T) < kBoysTMaxBits) {
     // T in FP32 by integer operations: the conversion runs on the FP64 pipe (24
     // atoms, FP64 integrals 156.7 -> 155.6 ms)
@@ -65,11 +71,11 @@ __device__ __forceinline__ void boys_seeds(double T, double pref, double pref_fa
     const float tf = __int_as_float((int)__funnelshift_l((unsigned)__double2loint(T), (unsigned)hi, 3));
     const int k = __float2int_rn(tf * (float)(1.0 / kBoysH));
     const double* row = tab + k * kBoysCols;
-    const double x = row[kBoysCols - 1] - T;  // T_k - T, |x| <= 0.05
-    double f = row[7];
+    const double x = row[kBoysCols - 1] - T;  // T_k - T, |x| <= 1/24
+    double f = row[kBoysTerms - 1];
 #pragma unroll
-    for (int m = 6; m >= 0; --m) f = fma(f, x, row[m]);
-    S[L] = pref * f;
+    for (int m = kBoysTerms - 2; m >= 0; --m) f = fma(f, x, row[m]);
+    S[L] = f;
     if (L > 0) {
       // e^{-T} = e^{-T_k} e^{x}, e^{x} by its 8-term Taylor polynomial
       double e = 1.0 / 5040.0;
@@ -80,14 +86,15 @@ __device__ __forceinline__ void boys_seeds(double T, double pref, double pref_fa
       e = fma(e, x, 0.5);
       e = fma(e, x, 1.0);
       e = fma(e, x, 1.0);
-      const double pe = (pref * row[kBoysTerms]) * e;
-      const double T2 = T + T;
+      const double pe = row[kBoysTerms] * e;
+      // below 2^-1022 the sum is not 2T but as small, and e^{-T} = 1 beside it
+      const double T2 = __hiloint2double(__double2hiint(T) + 0x00100000, __double2loint(T));
 #pragma unroll
       for (int n = L - 1; n >= 0; --n) S[n] = fma(T2, S[n + 1], pe) * (1.0 / (2 * n + 1));
     }
   } else {
     const double r = rsqrt(T);
-    S[0] = pref_far * r;
+    S[0] = 0.88622692545275801365 * r;  // sqrt(pi)/2
     if (L > 0) {
       const double o = 0.5 * (r * r);
 #pragma unroll
@@ -111,8 +118,8 @@ __device__ __forceinline__ void pair_xi(const PairHdr& h, const PrimPair* __rest
     const double PCx = pp.Px - cx, PCy = pp.Py - cy, PCz = pp.Pz - cz;
     const double T = pp.zeta * fma(PCx, PCx, fma(PCy, PCy, PCz * PCz));
     double S[C::L + 1];
-    boys_seeds<C::L>(T, pp.pref, pp.pref_far, tab, S);
-    C::prim(S, OsCoef<double>{pp.c10, pp.c20, pp.c30, pp.c40, pp.c01, pp.c11, pp.c21, pp.c02}, M);
+    boys_seeds<C::L>(T, tab, S);
+    C::prim(S, OsCoef<double>{pp.pref, pp.c10, pp.c20, pp.c30, pp.c40, pp.c01, pp.c11, pp.c21, pp.c02}, M);
   }
   double acc[C::NACC];
   C::build(M, -h.ABx, -h.ABy, -h.ABz, cx - A[0], cy - A[1], cz - A[2], acc);
@@ -739,7 +746,7 @@ __device__ __forceinline__ ds ds_ld(const float2* p) {
 
 __device__ __forceinline__ ds ds_c(const DsConst& c) { return ds_make(c.hi, c.lo); }
 
-// S_n = pref F_n(T), n = 0..L, in ds arithmetic: the FP64 method's 8-term
+// S_n = pref F_n(T), n = 0..L, in ds arithmetic: an 8-term
 // Taylor expansion about the nearest node of the 0.1-spaced table (nodes
 // rounded to ds-representable values, so T_k - T is exact to ds precision),
 // the downward recursion with e^{-T} = e^{-T_k} e^{x}, and the asymptotic
@@ -780,12 +787,12 @@ __device__ __forceinline__ ds ds_taylor(const Coef& c, ds x) {
 template <int L>
 __device__ __forceinline__ void boys_seeds_ds(ds T, ds pref, ds pref_far, const float2* tab, ds* S) {
   if (T.hi < (float)kBoysTMax) {
-    const int k = __float2int_rn(T.hi * (float)(1.0 / kBoysH));
-    const float2* row = tab + k * kBoysCols;
-    const ds x = ds_ld(row + kBoysCols - 1) - T;  // T_k - T, |x| <= 0.05
+    const int k = __float2int_rn(T.hi * (float)(1.0 / kBoysHDs));
+    const float2* row = tab + k * kBoysColsDs;
+    const ds x = ds_ld(row + kBoysColsDs - 1) - T;  // T_k - T, |x| <= 0.05
     S[L] = pref * ds_taylor(DsRow{row}, x);
     if (L > 0) {
-      const ds pe = (pref * ds_ld(row + kBoysTerms)) * ds_taylor(DsInvFact{}, x);
+      const ds pe = (pref * ds_ld(row + kBoysTermsDs)) * ds_taylor(DsInvFact{}, x);
       const ds T2 = ds_make(2.0f * T.hi, 2.0f * T.lo);
 #pragma unroll
       for (int n = L - 1; n >= 0; --n) {
@@ -870,8 +877,8 @@ __global__ void __launch_bounds__(kIntThreads) integral_kernel_ds(IntegralArgs a
   constexpr int NA = C::NA, NB = C::NB;
   constexpr bool kLockstep = C::L == 4;
   extern __shared__ float2 s_tab2[];
-  const float2* gtab = a.boys_ds + (size_t)C::L * kBoysRows * kBoysCols;
-  for (int e = threadIdx.x; e < kBoysRows * kBoysCols; e += blockDim.x) s_tab2[e] = gtab[e];
+  const float2* gtab = a.boys_ds + (size_t)C::L * kBoysRowsDs * kBoysColsDs;
+  for (int e = threadIdx.x; e < kBoysRowsDs * kBoysColsDs; e += blockDim.x) s_tab2[e] = gtab[e];
   __shared__ int s_tile;
   __syncthreads();
   for (;;) {
@@ -1053,8 +1060,10 @@ __global__ void debug_xi_kernel(const PairHdr* pair, const PrimPair* prims, cons
     const double PCx = pp.Px - cx, PCy = pp.Py - cy, PCz = pp.Pz - cz;
     const double T = pp.zeta * fma(PCx, PCx, fma(PCy, PCy, PCz * PCz));
     double S[C::L + 1];
-    boys_seeds<C::L>(T, pp.pref, pp.pref_far, tab, S);
-    C::vrr(S, pp.Px - A[0], pp.Py - A[1], pp.Pz - A[2], PCx, PCy, PCz, pp.c01, 2.0 * pp.c01, 3.0 * pp.c01, acc);
+    boys_seeds<C::L>(T, tab, S);
+    for (int m = 0; m <= C::L; ++m) S[m] *= pp.pref;
+    const double kappa = 0.5 / pp.zeta;
+    C::vrr(S, pp.Px - A[0], pp.Py - A[1], pp.Pz - A[2], PCx, PCy, PCz, kappa, 2.0 * kappa, 3.0 * kappa, acc);
   }
   double xi[C::NA * C::NB];
   C::hrr(acc, h.ABx, h.ABy, h.ABz, xi);
@@ -1064,7 +1073,7 @@ __global__ void debug_xi_kernel(const PairHdr* pair, const PrimPair* prims, cons
 template <int L>
 __device__ void boys_row(double T, const double* boys, double* out) {
   double S[L + 1];
-  boys_seeds<L>(T, 1.0, 0.88622692545275801365, boys + (size_t)L * kBoysRows * kBoysCols, S);
+  boys_seeds<L>(T, boys + (size_t)L * kBoysRows * kBoysCols, S);
   for (int n = 0; n <= L; ++n) out[n] = S[n];
 }
 
@@ -1082,6 +1091,7 @@ __global__ void debug_boys_kernel(const double* boys, int64_t n, const double* T
 }
 
 constexpr size_t kSmem64 = sizeof(double) * kBoysRows * kBoysCols;
+constexpr size_t kSmemDs = sizeof(float2) * kBoysRowsDs * kBoysColsDs;
 constexpr size_t kSmem32 = sizeof(float) * kBoysRowsF * kBoysColsF;
 
 // list < kNumClasses: FP64 kernel of that class; otherwise the FP32 kernel of
@@ -1098,7 +1108,7 @@ cudaError_t launch_kernel(K kernel, size_t smem, cudaStream_t st, const Integral
 template <int LA, int LB, int ND>
 cudaError_t launch_class_nd(cudaStream_t st, bool f32, const IntegralArgs& a, int grid) {
   if (f32) return launch_kernel(integral_kernel_f32<LA, LB, ND>, kSmem32, st, a, grid, kF32Threads);
-  if (a.hi_ds) return launch_kernel(integral_kernel_ds<LA, LB, ND>, kSmem64, st, a, grid);
+  if (a.hi_ds) return launch_kernel(integral_kernel_ds<LA, LB, ND>, kSmemDs, st, a, grid);
   return launch_kernel(integral_kernel<LA, LB, ND>, kSmem64, st, a, grid);
 }
 
@@ -1119,7 +1129,7 @@ int ctas_for(K kernel, size_t smem, int num_sms, int threads = kIntThreads) {
 template <int LA, int LB, int ND>
 int max_ctas_nd(bool f32, bool ds, int num_sms) {
   return f32  ? ctas_for(integral_kernel_f32<LA, LB, ND>, kSmem32, num_sms, kF32Threads)
-         : ds ? ctas_for(integral_kernel_ds<LA, LB, ND>, kSmem64, num_sms)
+         : ds ? ctas_for(integral_kernel_ds<LA, LB, ND>, kSmemDs, num_sms)
               : ctas_for(integral_kernel<LA, LB, ND>, kSmem64, num_sms);
 }
 

@@ -6,9 +6,11 @@
 
 namespace snk {
 
-// sigma^i kappa^j of one primitive pair, c<i><j>; a class reads those with i + 2j <= L
+// sigma^i kappa^j of one primitive pair, c<i><j>; a class reads those with i + 2j <= L.
+// FP64: times the primitive pair's prefactor, c00 the prefactor itself; elsewhere the
+// seeds carry the prefactor and c00 is not read (acc_lead)
 template <typename R> struct OsCoef {
-  R c10, c20, c30, c40, c01, c11, c21, c02;
+  R c00, c10, c20, c30, c40, c01, c11, c21, c02;
 };
 
 template <int LA, int LB> struct OsClass;
@@ -27,7 +29,7 @@ template <> struct OsClass<0, 0> {
   __device__ static __forceinline__ void prim(const R* S, const OsCoef<R>& c, A* M) {
     (void)c;
     const R w0_0 = S[0];
-    acc_add(M[0], w0_0);
+    acc_lead(M[0], c.c00, w0_0);
   }
   template <typename R, typename A>
   __device__ static __forceinline__ void build(const A* M, R nABx, R nABy, R nABz, R nACx, R nACy, R nACz,
@@ -67,7 +69,7 @@ template <> struct OsClass<1, 0> {
     const R w0_0 = S[0];
     const R w0_1 = S[1];
     const R w1_0 = w0_0 - w0_1;
-    acc_add(M[0], w0_1);
+    acc_lead(M[0], c.c00, w0_1);
     acc_mac(M[1], c.c10, w1_0);
   }
   template <typename R, typename A>
@@ -127,9 +129,9 @@ template <> struct OsClass<1, 1> {
     const R w1_0 = w0_0 - w0_1;
     const R w1_1 = w0_1 - w0_2;
     const R w2_0 = w1_0 - w1_1;
-    acc_add(M[0], w0_1);
+    acc_lead(M[0], c.c00, w0_1);
     acc_mac(M[1], c.c10, w1_0);
-    acc_add(M[2], w0_2);
+    acc_lead(M[2], c.c00, w0_2);
     acc_mac(M[3], c.c10, w1_1);
     acc_mac(M[4], c.c20, w2_0);
     acc_mac(M[5], c.c01, w1_0);
@@ -250,7 +252,7 @@ template <> struct OsClass<2, 0> {
     const R w1_0 = w0_0 - w0_1;
     const R w1_1 = w0_1 - w0_2;
     const R w2_0 = w1_0 - w1_1;
-    acc_add(M[0], w0_2);
+    acc_lead(M[0], c.c00, w0_2);
     acc_mac(M[1], c.c10, w1_1);
     acc_mac(M[2], c.c20, w2_0);
     acc_mac(M[3], c.c01, w1_0);
@@ -349,11 +351,11 @@ template <> struct OsClass<2, 1> {
     const R w2_0 = w1_0 - w1_1;
     const R w2_1 = w1_1 - w1_2;
     const R w3_0 = w2_0 - w2_1;
-    acc_add(M[0], w0_2);
+    acc_lead(M[0], c.c00, w0_2);
     acc_mac(M[1], c.c10, w1_1);
     acc_mac(M[2], c.c20, w2_0);
     acc_mac(M[3], c.c01, w1_0);
-    acc_add(M[4], w0_3);
+    acc_lead(M[4], c.c00, w0_3);
     acc_mac(M[5], c.c10, w1_2);
     acc_mac(M[6], c.c20, w2_1);
     acc_mac(M[7], c.c30, w3_0);
@@ -573,17 +575,17 @@ template <> struct OsClass<2, 2> {
     const R w3_0 = w2_0 - w2_1;
     const R w3_1 = w2_1 - w2_2;
     const R w4_0 = w3_0 - w3_1;
-    acc_add(M[0], w0_2);
+    acc_lead(M[0], c.c00, w0_2);
     acc_mac(M[1], c.c10, w1_1);
     acc_mac(M[2], c.c20, w2_0);
     acc_mac(M[3], c.c01, w1_0);
-    acc_add(M[4], w0_3);
+    acc_lead(M[4], c.c00, w0_3);
     acc_mac(M[5], c.c10, w1_2);
     acc_mac(M[6], c.c20, w2_1);
     acc_mac(M[7], c.c30, w3_0);
     acc_mac(M[8], c.c01, w1_1);
     acc_mac(M[9], c.c11, w2_0);
-    acc_add(M[10], w0_4);
+    acc_lead(M[10], c.c00, w0_4);
     acc_mac(M[11], c.c10, w1_3);
     acc_mac(M[12], c.c20, w2_2);
     acc_mac(M[13], c.c30, w3_1);

@@ -1407,7 +1407,11 @@ int create(int n_mol, const snk_basis* bases, const snk_grid* grids, const snk_o
          for (int e = 0; e < kExpTable; ++e) et[e] = std::exp2(-(double)e / kExpTable);
          SNK_CK(cp, upload(cp->exptab, et, st));
          SNK_CK(cp, upload(cp->pairs, s.pairs, st));
-         SNK_CK(cp, upload(cp->prims, s.prims, st));
+         // the FP64 kernels' copy: the prefactor in the contraction coefficients
+         std::vector<PrimPair> p64(s.prims);
+         for (PrimPair& P : p64)
+           for (double* v : {&P.c10, &P.c20, &P.c30, &P.c40, &P.c01, &P.c11, &P.c21, &P.c02}) *v *= P.pref;
+         SNK_CK(cp, upload(cp->prims, p64, st));
          SNK_CK(cp, upload(cp->bound, s.bound, st));
          SNK_CK(cp, upload(cp->qbound, s.qbound, st));
          SNK_CK(cp, upload(cp->bcenter, s.bcenter, st));

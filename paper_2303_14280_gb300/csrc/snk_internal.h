@@ -46,17 +46,27 @@ __device__ __forceinline__ double khat_value(const unsigned long long* e) {
 
 // Boys table: rows T_k = k * kBoysH, k = 0..kBoysRows-1; for T >= kBoysTMax the
 // asymptotic form is used.  One table per L = 0..4 with kBoysCols doubles per
-// row: F_{L+m}(T_k)/m! for m = 0..7, exp(-T_k), T_k.
+// row: seven coefficients, exp(-T_k), T_k.  The coefficients are the Taylor
+// series' F_{L+m}(T_k)/m!, m <= 8, with x^7 and x^8 replaced by their Chebyshev
+// approximations of degree 5 and 6 on |x| <= h = 1/24 (T_7 and T_8 dropped): the
+// error is F_{L+7} h^7 / (7! 64), below 3e-16 F_L, where eight Taylor terms on |x|
+// <= 0.05 have up to 3.5e-16 F_L.  43 KB: five CTAs fit an SM.
 // Table of the collocation kernels' e^{-x}: 2^{-j/256}.
 constexpr int kExpTable = 256;
 constexpr int kRadialPrims = 4;  // primitives whose e^{-a r^2} a thread keeps for the next shell of the group
 
-constexpr double kBoysH = 0.1;
+constexpr double kBoysH = 1.0 / 12.0;
 constexpr double kBoysTMax = 50.0;
-constexpr int kBoysRows = 502;
-constexpr int kBoysTerms = 8;
+constexpr int kBoysRows = 602;
+constexpr int kBoysTerms = 7;
 constexpr int kBoysCols = kBoysTerms + 2;
 constexpr int kBoysLMax = 2 * kLMax;
+
+// Double-FP32 table: F_{L+m}(T_k)/m! for m = 0..7, exp(-T_k), T_k.
+constexpr double kBoysHDs = 0.1;
+constexpr int kBoysRowsDs = 502;
+constexpr int kBoysTermsDs = 8;
+constexpr int kBoysColsDs = kBoysTermsDs + 2;
 
 // FP32 Boys table of the mixed form: nodes T_k = fl32(k * 0.05f) up to
 // kBoysTMaxF, rows of F_{L+m}(T_k)/m! for m = 0..3 (one float4).
@@ -93,6 +103,7 @@ struct PrimPair {
   double pref_far;      // pref * sqrt(pi) / 2  (large-T seed)
   double c10, c20, c30, c40;  // sigma^i, sigma = zeta_b / zeta (R_p - R_a = -sigma (R_a - R_b))
   double c01, c11, c21, c02;  // sigma^i kappa^j, kappa = 1 / (2 zeta)
+                              // (all eight times pref in the FP64 kernels' copy)
 };
 constexpr int kPrimWords = sizeof(PrimPair) / sizeof(double);
 constexpr int kPrimF32Words = 16;  // floats per primitive record of the FP32 tier
@@ -200,7 +211,7 @@ struct Setup {
 
   std::vector<double> boys;           // (kBoysLMax+1) x kBoysRows x kBoysCols
   std::vector<float> boys_f;          // (kBoysLMax+1) x kBoysRowsF x kBoysColsF
-  std::vector<float> boys_ds;         // (hi, lo) pairs: (kBoysLMax+1) x kBoysRows x kBoysCols x 2
+  std::vector<float> boys_ds;         // (hi, lo) pairs: (kBoysLMax+1) x kBoysRowsDs x kBoysColsDs x 2
 };
 
 // Validates and normalises the molecules' bases and grids; returns an
