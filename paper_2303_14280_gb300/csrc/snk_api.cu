@@ -111,11 +111,17 @@ constexpr int kDefaultStep = kMaxPairsPerStep;  // pairs staged per step of the 
 // 28.9, 12 atoms 7.7, 16 atoms with two densities 14.5 against 15.0).
 constexpr int kLanes = 3;
 constexpr int kLaneTiles = 16;  // 128-point tiles per SM
-// With less than three tiles per SM the FP64 / double-FP32 lists are also cut into
-// ranges, up to kMaxParts, until there are about three work items per SM: a warp's
-// time is the latency of its range (an FP64 multiply-add takes about 60 clocks).  4
-// atoms (94 tiles), FP64: lists 0.69 -> 0.45 ms.
-constexpr int kMaxParts = 4;
+// The FP64 / double-FP32 lists are also cut into ranges, up to kMaxParts, as long as
+// a lane then has at most kPartItems work items per SM: a warp's time is the latency
+// of its range (an FP64 multiply-add takes about 60 clocks), and a launch ends with
+// the SMs whose last items started late.  ms per build at 3 / 8 / 16 / 28 items (copies
+// of G kLanes x ranges): 4 atoms FP64 (0.6 tiles) 0.744 / 0.702 / 0.710 / 0.705, 12 atoms
+// mixed (3.2) 7.10 / 6.35 / 6.42 / 6.62, 17 atoms double-FP32 (5.4) 27.4 / 27.2 / 26.7 /
+// 26.4, 24 atoms FP64 (3.8) 165.2 / 160.8 / 158.8 / 158.0, 16 atoms with two densities
+// 14.9 / 14.9 / 14.7 / 15.3; beyond it the copies' clearing and sum cost what the shorter
+// ranges give.
+constexpr int kMaxParts = 8;
+constexpr int kPartItems = 12;
 constexpr int kLaneOf[kNumClasses] = {0, 1, 2, 2, 1, 0};     // ss ps pp ds dp dd: about equal work per lane
 constexpr int kLaneOrder[kNumClasses] = {5, 4, 3, 0, 1, 2};  // heavier list of every lane first
 constexpr int kRunCandidates[] = {2, 4, 8, 16, 32, 64};
@@ -776,11 +782,11 @@ int screen_and_plan(snk_ctx* c) {
       af += tc ? oz_bytes(bd[t], 0) : 0;
       ak += tc ? oz_bytes(bd[t], 1) : 0;
     }
-    const int most =
-        (int)std::max<int64_t>(1, std::min<int64_t>(kMaxParts, 3 * (int64_t)c->num_sms / std::max<int64_t>(tiles, 1)));
-    if (tiles <= (int64_t)kLaneTiles * c->num_sms &&
-        (x + (1 + kLanes * most) * f) * 8 + (mixed ? f * 4 : 0) + std::max(af, ak) <= c->ws_budget)
-      lanes = kLanes, parts = most;
+    int p = (int)std::min<int64_t>(kMaxParts, kPartItems * (int64_t)c->num_sms / std::max<int64_t>(tiles, 1));
+    if (tiles <= (int64_t)kLaneTiles * c->num_sms)
+      for (p = std::max(p, 1); p >= 1 && lanes == 1; --p)
+        if ((x + (1 + kLanes * p) * f) * 8 + (mixed ? f * 4 : 0) + std::max(af, ak) <= c->ws_budget)
+          lanes = kLanes, parts = p;
   }
   auto plan_chunks = [&]() {
     c->chunks.clear();
