@@ -19,6 +19,7 @@ BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(BUILD, "libsnk.so")
 SOURCES = ["host_setup.cpp", "kernels_dense.cu", "kernels_integrals.cu", "kernels_ozaki.cu", "kernels_xc.cu", "mlp.cu", "snk_api.cu"]
 HEADERS = ["snk_internal.h", "os_generated.cuh", "async_copy.cuh", "ds_arith.cuh", "f2_arith.cuh", "exp_neg.cuh",
+           "oz_digits.cuh",
            os.path.join("..", "..", "include", "snk.h")]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ARCH + ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", "-O2",

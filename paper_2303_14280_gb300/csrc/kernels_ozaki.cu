@@ -35,6 +35,7 @@
 #include <cstdint>
 
 #include "async_copy.cuh"
+#include "oz_digits.cuh"
 #include "snk_internal.h"
 
 namespace snk {
@@ -133,8 +134,7 @@ __device__ __forceinline__ void oz_emit8(const double* x, int e, uint8_t* dst) {
         d = (int)dl;
         r[q] = (int)r64[q];  // complete once s == k64 - 1
       } else if (k > 0) {
-        d = k == 24 ? (r[q] >> 24) + ((r[q] >> 23) & 1) : (r[q] + (1 << (k - 1))) >> k;
-        r[q] -= (int)((unsigned)d << k);
+        d = oz_take_digit(r[q], k);
       } else {
         d = r[q];
       }
