@@ -519,12 +519,13 @@ void build_boys_tables(Setup* s) {
       row[2 * (kBoysTermsDs + 1) + 1] = tl;
     }
   }
-  // FP32 table of the mixed form: nodes at the float values fl32(k * 0.05f)
-  // that the kernel forms itself, four Taylor coefficients per row
+  // FP32 table of the mixed form, four Taylor coefficients per row: the kernel's
+  // T_k - T is one multiply-add of k and the float 0.05, so the nodes are the exact
+  // products (a node rounded to FP32 is off by up to 9.5e-7 at T above 16, which
+  // moved F_L by up to 2.5e-7)
   s->boys_f.assign((size_t)(kBoysLMax + 1) * kBoysRowsF * kBoysColsF, 0.0f);
   for (int k = 0; k < kBoysRowsF; ++k) {
-    const float tk = (float)k * kBoysHF;
-    host_boys(kBoysLMax + kBoysTermsF, (double)tk, F);
+    host_boys(kBoysLMax + kBoysTermsF, (double)k * (double)kBoysHF, F);
     for (int L = 0; L <= kBoysLMax; ++L) {
       float* row = &s->boys_f[((size_t)L * kBoysRowsF + k) * kBoysColsF];
       for (int m = 0; m < kBoysTermsF; ++m) row[m] = (float)(F[L + m] * invfact[m]);

@@ -225,8 +225,8 @@ __global__ void __launch_bounds__(kIntThreads) integral_kernel(IntegralArgs a) {
 
 // FP32 seeds S_n = pref F_n(T) at two points: 4-term Taylor about the nearest
 // node of a 0.05-spaced float table below T = 30 (|T - T_k| <= 0.025:
-// truncation below 2e-8 relative; one 16-byte row per lookup, the node fl32(k *
-// 0.05f) formed in registers), the asymptotic form above (e^{-T} < 1e-13 is
+// truncation below 2e-8 relative; one 16-byte row per lookup, the distance to the
+// node k 0.05f formed by one multiply-add), the asymptotic form above (e^{-T} < 1e-13 is
 // below FP32 resolution).  e^{-T} of the downward recursion comes from the
 // hardware exponential (__expf, ~2^-21 relative).  The lookups and the
 // polynomial run per point (the two rows' coefficients sit in different

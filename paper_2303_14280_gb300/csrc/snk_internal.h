@@ -68,8 +68,8 @@ constexpr int kBoysRowsDs = 502;
 constexpr int kBoysTermsDs = 8;
 constexpr int kBoysColsDs = kBoysTermsDs + 2;
 
-// FP32 Boys table of the mixed form: nodes T_k = fl32(k * 0.05f) up to
-// kBoysTMaxF, rows of F_{L+m}(T_k)/m! for m = 0..3 (one float4).
+// FP32 Boys table of the mixed form: nodes T_k = k x (the float 0.05),
+// not rounded, up to kBoysTMaxF, rows of F_{L+m}(T_k)/m! for m = 0..3 (one float4).
 constexpr float kBoysTMaxF = 30.0f;
 constexpr float kBoysHF = 0.05f;
 constexpr int kBoysRowsF = 602;
