@@ -278,7 +278,7 @@ __global__ void __launch_bounds__(COL_THREADS) collocation_kernel(const BatchDes
   const int i = blockIdx.x * COL_THREADS + threadIdx.x;
   const int t0 = blockIdx.y * COL_SHELLS;
   if (blockIdx.x * COL_THREADS >= bd.ldq || t0 >= bd.nBshell) return;  // block-uniform
-  __shared__ double s_exp[kExpTable];
+  __shared__ double2 s_exp[kExpTable];
   exp_table_load(s_exp, B.exptab);
   if (i >= bd.ldq) return;
   const int t1 = min(t0 + COL_SHELLS, bd.nBshell);

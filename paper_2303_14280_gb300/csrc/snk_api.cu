@@ -21,6 +21,7 @@
 #include <utility>
 #include <vector>
 
+#include "exp_neg.cuh"
 #include "snk_internal.h"
 
 using namespace snk;
@@ -143,8 +144,9 @@ struct snk_ctx {
 
   // geometry (device)
   DevBuf<int> l, poff, nprim, foff, fshell, bshell, bshell_col, xfunc, rgroup;
-  DevBuf<double> center, exps, d, fcomp, exptab, xyz, w, boys, bound, qbound, bcenter, bradius, phit_f, phit_b;
+  DevBuf<double> center, exps, d, fcomp, xyz, w, boys, bound, qbound, bcenter, bradius, phit_f, phit_b;
   DevBuf<float> boys_f, boys_ds, prims_ds, pair_ab, pair_a, prims_f32, prim_share;  // mixed form: FP32 and (hi, lo) copies
+  DevBuf<double2> exptab;
   DevBuf<PairHdr> pairs;
   DevBuf<PrimPair> prims;
   DevBuf<MolDesc> mols;
@@ -1409,8 +1411,8 @@ int create(int n_mol, const snk_basis* bases, const snk_grid* grids, const snk_o
          SNK_CK(cp, upload(cp->exps, s.exps, st));
          SNK_CK(cp, upload(cp->d, s.d, st));
          SNK_CK(cp, upload(cp->fcomp, s.fcomp, st));
-         std::vector<double> et(kExpTable);
-         for (int e = 0; e < kExpTable; ++e) et[e] = std::exp2(-(double)e / kExpTable);
+         std::vector<double2> et(kExpTable);
+         exp_table_fill(et.data());
          SNK_CK(cp, upload(cp->exptab, et, st));
          SNK_CK(cp, upload(cp->pairs, s.pairs, st));
          // the FP64 kernels' copy: the prefactor in the contraction coefficients

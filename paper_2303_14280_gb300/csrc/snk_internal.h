@@ -44,6 +44,10 @@ __device__ __forceinline__ double khat_value(const unsigned long long* e) {
 }
 #endif
 
+// Table of the collocation kernels' e^{-x}: 2^{-j/256}.
+constexpr int kExpTable = 256;
+constexpr int kRadialPrims = 4;  // primitives whose e^{-a r^2} a thread keeps for the next shell of the group
+
 // Boys table: rows T_k = k * kBoysH, k = 0..kBoysRows-1; for T >= kBoysTMax the
 // asymptotic form is used.  One table per L = 0..4 with kBoysCols doubles per
 // row: seven coefficients, exp(-T_k), T_k.  The coefficients are the Taylor
@@ -51,10 +55,6 @@ __device__ __forceinline__ double khat_value(const unsigned long long* e) {
 // approximations of degree 5 and 6 on |x| <= h = 1/24 (T_7 and T_8 dropped): the
 // error is F_{L+7} h^7 / (7! 64), below 3e-16 F_L, where eight Taylor terms on |x|
 // <= 0.05 have up to 3.5e-16 F_L.  43 KB: five CTAs fit an SM.
-// Table of the collocation kernels' e^{-x}: 2^{-j/256}.
-constexpr int kExpTable = 256;
-constexpr int kRadialPrims = 4;  // primitives whose e^{-a r^2} a thread keeps for the next shell of the group
-
 constexpr double kBoysH = 1.0 / 12.0;
 constexpr double kBoysTMax = 50.0;
 constexpr int kBoysRows = 602;
@@ -227,7 +227,7 @@ void host_boys(int nmax, double T, double* F);
 
 struct DeviceBasis {
   const int* rgroup;     // shells of a group share centre and exponents (at most kRadialPrims of them)
-  const double* exptab;  // 2^{-j/kExpTable} of exp_neg
+  const double2* exptab;  // 2^{-j/kExpTable} of exp_neg, head and tail
   const int* l;
   const int* poff;
   const int* nprim;
