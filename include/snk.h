@@ -237,11 +237,17 @@ int snk_set_density_batch(snk_ctx *ctx, const double *const *P);
 
 /* Build K for the loaded density (Alg. 1 on one GPU).  K is host memory in the
  * packed layout of snk_set_density; the call returns when K is written.
- * Every form is reproducible bit for bit: each G entry of an integral launch
- * has a single writer whose additions come in pair-list order, and the
- * batches' contributions to K are summed as exact 64-bit fixed-point integers
+ * Every form is reproducible bit for bit, whatever the workspace size: each G
+ * entry of an integral launch has a single writer whose additions come in
+ * pair-list order, builds small enough to run their lists side by side add
+ * their copies of G in a fixed order (workspaces that do not hold all copies
+ * fill them group by group; only when the allocator refuses even one beside the
+ * sum do the lists run into one G, which rounds differently), and the batches'
+ * contributions to K are summed as exact 64-bit fixed-point integers
  * (resolution 2^-76, |contribution| < 2^30: a larger or non-finite one gives
- * SNK_ERR_UNSUPPORTED; at most 2^19 grid batches per handle). */
+ * SNK_ERR_UNSUPPORTED; at most 2^19 grid batches per handle).  A molecule in a
+ * handle of several agrees with the same molecule alone to rounding only: the
+ * cut of the work follows from all of the handle's points. */
 int snk_build_K(snk_ctx *ctx, double *K);
 /* Same, writing the packed blocks into device memory; returns once the work
  * is enqueued on the library stream (synchronise it before reading dK). */

@@ -921,20 +921,21 @@ cudaError_t launch_fgemm(cudaStream_t st, const BatchDesc* dbatch, int nbatch, i
 // 64 points each (a block's 4,096 fixed-point additions are then 1 % of its
 // FP64 work).  4 atoms, 21 functions, 4 batches of 3,000 points: 4 blocks took
 // 3.14 ms, 188 take 0.04; from about 900 (tile, batch) pairs on nothing is split.
-int point_split(int tiles, int max_q, int* klen) {
-  const int want = 152 * 6;
-  const int nsplit = std::max(1, std::min((want + tiles - 1) / std::max(tiles, 1), (max_q + 63) / 64));
-  *klen = std::max(TK, ((max_q + nsplit - 1) / nsplit + TK - 1) / TK * TK);
-  return (max_q + *klen - 1) / *klen;
+// All batches of the handle count, not a chunk's: the rounding of a block's sum, and
+// with it K, then does not depend on the workspace.
+int point_split(int nbatch, int max_q, int max_m, int max_n) {
+  constexpr int64_t want = 152 * 6;
+  const int64_t tiles = std::max<int64_t>(1, (int64_t)((max_m + TM - 1) / TM) * ((max_n + TN - 1) / TN) * nbatch);
+  const int nsplit = (int)std::max<int64_t>(1, std::min<int64_t>((want + tiles - 1) / tiles, (max_q + 63) / 64));
+  return std::max(TK, ((max_q + nsplit - 1) / nsplit + TK - 1) / TK * TK);
 }
 
 cudaError_t launch_kgemm(cudaStream_t st, const BatchDesc* dbatch, int nbatch, int max_ldq, int max_nS, int max_nB,
-                         const int* xfunc, const int* sfunc, const double* ws, unsigned long long* Khat, int mode,
-                         int dens, int* err) {
+                         int klen, const int* xfunc, const int* sfunc, const double* ws, unsigned long long* Khat,
+                         int mode, int dens, int* err) {
   if (nbatch == 0 || max_ldq == 0 || max_nS == 0 || max_nB == 0) return cudaSuccess;
   const int mt = (max_nS + TM - 1) / TM, nt = (max_nB + TN - 1) / TN;
-  int klen = 0;
-  const int nsplit = point_split(mt * nt * nbatch, max_ldq, &klen);
+  const int nsplit = (max_ldq + klen - 1) / klen;
   dim3 grid(mt * nsplit, nt, nbatch);
   if (mode == 2)
     kgemm_kernel<2><<<grid, GEMM_THREADS, 0, st>>>(dbatch, xfunc, sfunc, ws, Khat, dens, klen, mt, err);
@@ -1006,11 +1007,11 @@ cudaError_t launch_xc_fgemm(cudaStream_t st, const BatchDesc* dbatch, int nbatch
 }
 
 cudaError_t launch_xc_vgemm(cudaStream_t st, const BatchDesc* dbatch, int nbatch, int max_ldq, int max_nB,
-                            const int* xfunc, const double* ws, unsigned long long* Vhat, int mode, int* err) {
+                            int klen, const int* xfunc, const double* ws, unsigned long long* Vhat, int mode,
+                            int* err) {
   if (nbatch == 0 || max_ldq == 0 || max_nB == 0) return cudaSuccess;
   const int mt = (max_nB + TM - 1) / TM;
-  int klen = 0;
-  const int nsplit = point_split(mt * mt * nbatch, max_ldq, &klen);
+  const int nsplit = (max_ldq + klen - 1) / klen;
   dim3 grid(mt * nsplit, mt, nbatch);
   if (mode == 2)
     xc_vgemm_kernel<2><<<grid, GEMM_THREADS, 0, st>>>(dbatch, xfunc, ws, Vhat, klen, mt, err);

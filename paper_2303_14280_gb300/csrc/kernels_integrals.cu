@@ -126,12 +126,12 @@ __device__ __forceinline__ void pair_xi(const PairHdr& h, const PrimPair* __rest
   C::hrr(acc, h.ABx, h.ABy, h.ABz, xi);
 }
 
-// Work item t of the FP64 / ds lists: tile t mod n_tiles, range t / n_tiles of its
-// list.
+// Work item t of the FP64 / ds lists: tile t mod n_tiles, the launch's range t /
+// n_tiles of its list.
 __device__ __forceinline__ Tile tile_part(const IntegralArgs& a, int t) {
   Tile tile = a.tiles[t % a.n_tiles];
   if (a.parts > 1) {
-    const int64_t n = tile.k1 - tile.k0, part = t / a.n_tiles;
+    const int64_t n = tile.k1 - tile.k0, part = a.part0 + t / a.n_tiles;
     tile.k1 = tile.k0 + (int)(n * (part + 1) / a.parts);
     tile.k0 += (int)(n * part / a.parts);
   }
@@ -154,7 +154,7 @@ __global__ void __launch_bounds__(kIntThreads) integral_kernel(IntegralArgs a) {
     __syncthreads();
     const int t = s_tile;
     __syncthreads();
-    if (t >= a.n_tiles * a.parts) break;
+    if (t >= a.n_tiles * a.part_n) break;
     const Tile tile = tile_part(a, t);
     const BatchDesc bd = a.batches[tile.batch];
     const int i = tile.i0 + threadIdx.x;
@@ -894,7 +894,7 @@ __global__ void __launch_bounds__(kIntThreads) integral_kernel_ds(IntegralArgs a
     __syncthreads();
     const int t = s_tile;
     __syncthreads();
-    if (t >= a.n_tiles * a.parts) break;
+    if (t >= a.n_tiles * a.part_n) break;
     const Tile tile = tile_part(a, t);
     const BatchDesc bd = a.batches[tile.batch];
     int i = tile.i0 + threadIdx.x;

@@ -103,7 +103,10 @@ constexpr int kDefaultStep = kMaxPairsPerStep;  // pairs staged per step of the 
 // more than the others; one after another the twelve lists leave much of the
 // chip idle.  A lane's lists run in order, so every copy of G has one writer at a
 // time, and the copies are added in a fixed order: K stays the same bit for bit
-// from run to run.  Measured, lists one after another / side by side (tiles of
+// from run to run.  Which list range adds into which copy follows from the work
+// alone; with less memory fewer copies are held at a time (snk_ctx::group) and
+// filled group after group in the same order, so K does not depend on the
+// workspace.  Measured, lists one after another / side by side (tiles of
 // 128 points per SM in brackets): 17 atoms double-FP32 (5.4) 41.7 / 28.1 ms, 12
 // atoms mixed (3.2) 10.4 / 7.2, 24 atoms FP64 (3.8) 190 / 175, 4 atoms FP64 (0.6)
 // 1.23 / 1.13, 32 atoms mixed (13.5) 66.0 / 61.0; 24 molecules (30) 42.1 / 41.4 and 96
@@ -191,8 +194,6 @@ struct snk_ctx {
   struct Chunk {
     int b0 = 0, b1 = 0;
     int64_t bytes = 0, xn = 0, goff = 0, gn = 0;  // gn: doubles of one copy of G
-    int parts = 1;   // ranges of every FP64 / ds list that add into copies of G of their own
-    int copies = 1;  // copies of G: kLanes x parts when the lists run side by side
     int max_ldq = 0, max_nS = 0, max_nB = 0, max_nBshell = 0;
     int64_t tile_off[kNumLists] = {0}, tile_n[kNumLists] = {0};
     // SNK_GEMM_SPLIT: split jobs of the F and K phases, product jobs of F hi, F lo, K hi, K lo
@@ -203,6 +204,14 @@ struct snk_ctx {
   };
   std::vector<Chunk> chunks;
   int max_ctas[kNumLists] = {0};
+  // Lists side by side: the loaded density's kLanes x parts copies of G (copy c: lane
+  // c mod kLanes, range c / kLanes of the FP64 / ds lists) are filled `group` at a
+  // time; group 0: one list after another into one G.  group is kLanes x parts, or a
+  // smaller multiple of kLanes beside a G for the sum, or 1 (no two lists at a time).
+  int parts = 1, group = 0;
+  int group_limit = 1 << 30;  // largest group not refused by the allocator yet
+  int copies_held() const { return group == 0 ? 1 : group == kLanes * parts ? group : group + 1; }
+  int klen = 0;  // points per block of the K product's FP64 / double-FP32 tiles (point_split)
 
   // exchange-correlation potential (snk_build_Vxc): its own batch descriptors
   // (X, grad X and F / Z of each batch in xcws), chunks, fixed-point V-hat and
@@ -215,6 +224,7 @@ struct snk_ctx {
     int g_off[2] = {0, 0}, g_n[2] = {0, 0}, g_tiles[2] = {0, 0};
   };
   std::vector<XcChunk> xc_chunks;
+  int xc_klen = 0;  // points per block of the V-hat product (point_split)
   DevBuf<BatchDesc> xcbatch;
   DevBuf<double> xcws, xcE;
   DevBuf<unsigned long long> xchat;
@@ -773,24 +783,46 @@ int screen_and_plan(snk_ctx* c) {
     return oz_operand_bytes(b.nB, b.q, S5) +
            (int64_t)nd * (oz_operand_bytes(hiS, b.q, S5) + oz_operand_bytes(loS, b.q, S5));
   };
-  // lists side by side: few tiles, and everything with kLanes copies of G in one chunk
-  int lanes = 1, parts = 1;
+  // lists side by side: few tiles.  Lanes and ranges follow from the number of tiles;
+  // the memory decides how many of the copies of G are held at a time.
   {
-    int64_t tiles = 0, x = 0, f = 0, af = 0, ak = 0;
+    int64_t tiles = 0, x = 0, f = 0, af = 0, ak = 0, worst = 0;
+    int max_q = 0, max_nS = 0, max_nB = 0;
     for (int t = 0; t < nb; ++t) {
+      const int64_t xs = (int64_t)bd[t].ldq * bd[t].nB, fs = (int64_t)nd * bd[t].ldq * bd[t].nS;
+      const int64_t ozf = tc ? oz_bytes(bd[t], 0) : 0, ozk = tc ? oz_bytes(bd[t], 1) : 0;
       tiles += (bd[t].q + kPointTile - 1) / kPointTile;
-      x += (int64_t)bd[t].ldq * bd[t].nB;
-      f += (int64_t)nd * bd[t].ldq * bd[t].nS;
-      af += tc ? oz_bytes(bd[t], 0) : 0;
-      ak += tc ? oz_bytes(bd[t], 1) : 0;
+      x += xs;
+      f += fs;
+      af += ozf;
+      ak += ozk;
+      worst = std::max(worst, (xs + (2 + kLanes) * fs) * 8 + (mixed ? fs * 4 : 0) + std::max(ozf, ozk));
+      max_q = std::max(max_q, bd[t].ldq);
+      max_nS = std::max(max_nS, bd[t].nS);
+      max_nB = std::max(max_nB, bd[t].nB);
     }
-    int p = (int)std::min<int64_t>(kMaxParts, kPartItems * (int64_t)c->num_sms / std::max<int64_t>(tiles, 1));
-    if (tiles <= (int64_t)kLaneTiles * c->num_sms)
-      for (p = std::max(p, 1); p >= 1 && lanes == 1; --p)
-        if ((x + (1 + kLanes * p) * f) * 8 + (mixed ? f * 4 : 0) + std::max(af, ak) <= c->ws_budget)
-          lanes = kLanes, parts = p;
+    c->klen = point_split(nb, max_q, max_nS, max_nB);
+    c->parts = 1;
+    c->group = 0;
+    if (tiles <= (int64_t)kLaneTiles * c->num_sms) {
+      c->parts = (int)std::min<int64_t>(kMaxParts, kPartItems * (int64_t)c->num_sms / std::max<int64_t>(tiles, 1));
+      c->parts = std::max(c->parts, 1);
+      // the largest group that fits the workspace cap in one chunk; else groups of one
+      // range in smaller chunks, or single copies where even a batch is too large for that
+      c->group = worst <= c->ws_budget ? kLanes : 1;
+      for (int p = c->parts; p >= 1; --p) {
+        const int64_t copies = p == c->parts ? kLanes * p : kLanes * p + 1;
+        if (kLanes * p <= c->group_limit &&
+            (x + (1 + copies) * f) * 8 + (mixed ? f * 4 : 0) + std::max(af, ak) <= c->ws_budget) {
+          c->group = kLanes * p;
+          break;
+        }
+      }
+      if (c->group > c->group_limit) c->group = std::max(c->group_limit, 0);
+    }
   }
   auto plan_chunks = [&]() {
+    const int held = c->copies_held();
     c->chunks.clear();
     need = need32 = need_tsum = 1;
     need_arena = 0;
@@ -798,13 +830,11 @@ int screen_and_plan(snk_ctx* c) {
     while (j < nb) {
       snk_ctx::Chunk ch;
       ch.b0 = j;
-      ch.parts = parts;
-      ch.copies = lanes * parts;
       int64_t xo = 0, fo = 0, af = 0, ak = 0;
       while (j < nb) {
         // F and G of density d at foff / goff + d ldq nS
         int64_t xs = (int64_t)bd[j].ldq * bd[j].nB, fs = (int64_t)nd * bd[j].ldq * bd[j].nS;
-        int64_t bytes = (xo + xs + (1 + lanes * parts) * (fo + fs)) * 8 + (mixed ? (fo + fs) * 4 : 0);
+        int64_t bytes = (xo + xs + (1 + held) * (fo + fs)) * 8 + (mixed ? (fo + fs) * 4 : 0);
         const int64_t ozf = tc ? oz_bytes(bd[j], 0) : 0, ozk = tc ? oz_bytes(bd[j], 1) : 0;
         bytes += std::max(af + ozf, ak + ozk);
         if (j > ch.b0 && bytes > c->ws_budget) break;
@@ -839,8 +869,8 @@ int screen_and_plan(snk_ctx* c) {
         ch.max_nB = std::max(ch.max_nB, bd[t].nB);
         ch.max_nBshell = std::max(ch.max_nBshell, bd[t].nBshell);
       }
-      ch.bytes = (xo + (1 + lanes * parts) * fo) * 8;
-      need = std::max(need, xo + (1 + lanes * parts) * fo);
+      ch.bytes = (xo + (1 + held) * fo) * 8;
+      need = std::max(need, xo + (1 + held) * fo);
       need_tsum = std::max(need_tsum, scur);
       if (mixed) need32 = std::max(need32, fo);
       c->chunks.push_back(ch);
@@ -855,13 +885,17 @@ int screen_and_plan(snk_ctx* c) {
   };
   plan_chunks();
   cudaError_t res = reserve();
-  if (res == cudaErrorMemoryAllocation && lanes > 1) {  // no room for the copies of G: one list after another
+  const int limit = c->group_limit;
+  while (res == cudaErrorMemoryAllocation && c->group > 0) {  // no room for these copies of G: fewer at a time
     cudaGetLastError();
     c->ws.release();
-    lanes = parts = 1;
+    const int p = c->group / kLanes;
+    c->group = p > 1 ? kLanes * (p / 2) : p == 1 ? 1 : 0;
+    c->group_limit = c->group;  // later densities do not ask for more again
     plan_chunks();
     res = reserve();
   }
+  if (res != cudaSuccess) c->group_limit = limit;
   SNK_CK(c, res);
   SNK_CK(c, upload(c->batch, bd, st));
   SNK_CK(c, c->exec.ensure(2 * kNumLists));
@@ -877,7 +911,7 @@ int screen_and_plan(snk_ctx* c) {
   SNK_CK(c, c->Khat.ensure((size_t)std::max<int64_t>(2 * c->n_dens * s.packed, 2)));
   if (mixed && c->opt.gemm != SNK_GEMM_FP64)
     SNK_CK(c, c->P2.ensure((size_t)std::max<int64_t>(c->n_dens * s.packed, 1)));
-  if (lanes > 1 && !c->ev_fork) {
+  if (c->group > 1 && !c->ev_fork) {
     for (int l = 0; l < kLanes - 1; ++l) {
       if (!c->lane[l]) SNK_CK(c, cudaStreamCreateWithFlags(&c->lane[l], cudaStreamNonBlocking));
       if (!c->ev_lane[l]) SNK_CK(c, cudaEventCreateWithFlags(&c->ev_lane[l], cudaEventDisableTiming));
@@ -966,8 +1000,9 @@ IntegralArgs integral_args(snk_ctx* c, size_t ci, int k) {
   a.eps_tile = (k >= kNumClasses && tile_screen(c)) ? (float)c->opt.eps_tile : 0.f;
   a.exec = c->exec.p + 2 * k;
   a.gshift = 0;
-  a.parts = k < kNumClasses ? ch.parts : 1;
-  a.gpart = ch.gn;
+  a.parts = a.part_n = 1;
+  a.part0 = 0;
+  a.gpart = kLanes * ch.gn;
   a.n_dens = c->n_dens;
   a.run = c->run[k];
   a.err = c->ozerr.p;
@@ -1056,40 +1091,67 @@ int enqueue_build(snk_ctx* c, cudaStream_t st, double* dK, bool timed) {
       SNK_CK(c, launch_tile_sums(st, db, nbc, ch.max_tiles, c->ws.p, c->ws32.p, c->xyz.p, nd, c->tsum.p));
       ++c->launches_build;
     }
-    SNK_CK(c, cudaMemsetAsync(c->ws.p + ch.goff, 0, sizeof(double) * ch.gn * ch.copies, st));
+    const int first = std::max(c->group, 1);  // copies of G of the first group
+    SNK_CK(c, cudaMemsetAsync(c->ws.p + ch.goff, 0, sizeof(double) * ch.gn * first, st));
     SNK_CK(c, mark());
     // G_j, Eq. (gmat) with the 3c-CP integrals of App. A, list by list
-    auto integrals = [&](int k, int lane) -> cudaError_t {
-      IntegralArgs a = integral_args(c, ci, k);
+    auto integrals = [&](cudaStream_t sl, int k, const IntegralArgs& a) -> cudaError_t {
       if (a.n_tiles == 0) return cudaSuccess;
-      a.gshift = (int64_t)lane * ch.parts * ch.gn;
       ++c->launches_build;
-      return launch_integrals(lane ? c->lane[lane - 1] : st, k, a, (int)std::min<int64_t>(c->max_ctas[k], (int64_t)a.n_tiles * a.parts));
+      return launch_integrals(sl, k, a, (int)std::min<int64_t>(c->max_ctas[k], (int64_t)a.n_tiles * a.part_n));
     };
-    if (ch.copies > 1) {
-      // side by side: the lanes start after everything before and join before G is used
-      auto lanes = [&]() -> cudaError_t {
-        cudaError_t e = cudaEventRecord(c->ev_fork, st);
-        for (int l = 0; l < kLanes - 1 && e == cudaSuccess; ++l) e = cudaStreamWaitEvent(c->lane[l], c->ev_fork, 0);
-        for (int tier = 0; tier < 2; ++tier)
-          for (int o = 0; o < kNumClasses && e == cudaSuccess; ++o)
-            e = integrals(tier * kNumClasses + kLaneOrder[o], kLaneOf[kLaneOrder[o]]);
-        for (int l = 0; l < kLanes - 1; ++l) {  // join whatever was launched
-          const cudaError_t r = cudaEventRecord(c->ev_lane[l], c->lane[l]);
-          const cudaError_t w = cudaStreamWaitEvent(st, c->ev_lane[l], 0);
-          if (e == cudaSuccess) e = r != cudaSuccess ? r : w;
-        }
-        return e;
-      };
-      SNK_CK(c, lanes());
-      SNK_CK(c, launch_sum_copies(st, c->ws.p + ch.goff, ch.gn, ch.copies));
-      ++c->launches_build;
-      for (int k = 0; k < kNumLists; ++k) SNK_CK(c, mark());
-    } else {
+    if (c->group == 0) {
       for (int k = 0; k < kNumLists; ++k) {
-        SNK_CK(c, integrals(k, 0));
+        SNK_CK(c, integrals(st, k, integral_args(c, ci, k)));
         SNK_CK(c, mark());
       }
+    } else {
+      const int all = kLanes * c->parts;
+      // the lists of one lane over the copies [c0, c1) of the group, each list in order; the
+      // FP32 lists add into the lane's first copy
+      auto lane_lists = [&](int c0, int c1, int tier, int cls) -> cudaError_t {
+        const int lane = kLaneOf[cls], k = tier * kNumClasses + cls;
+        const int cl = c0 + (lane - c0 % kLanes + kLanes) % kLanes;  // the lane's first copy of the group
+        if (cl >= c1 || (tier == 1 && cl >= kLanes)) return cudaSuccess;
+        IntegralArgs a = integral_args(c, ci, k);
+        a.gshift = (int64_t)(cl - c0 + (c0 > 0)) * ch.gn;
+        if (tier == 0) {
+          a.parts = c->parts;
+          a.part0 = cl / kLanes;
+          a.part_n = (c1 - cl + kLanes - 1) / kLanes;
+        }
+        return integrals(c->group > 1 && lane ? c->lane[lane - 1] : st, k, a);
+      };
+      for (int c0 = 0; c0 < all; c0 += c->group) {
+        const int c1 = std::min(c0 + c->group, all);
+        if (c0 > 0) {  // the copies after the sum, and the tickets of the lists' next ranges
+          SNK_CK(c, cudaMemsetAsync(c->ws.p + ch.goff + ch.gn, 0, sizeof(double) * ch.gn * (c1 - c0), st));
+          SNK_CK(c, cudaMemsetAsync(c->tickets.p + ci * kNumLists, 0, sizeof(int) * kNumClasses, st));
+        }
+        // side by side: the lanes start after everything before and join before G is used
+        auto lanes = [&]() -> cudaError_t {
+          const bool fork = c->group > 1;
+          cudaError_t e = fork ? cudaEventRecord(c->ev_fork, st) : cudaSuccess;
+          for (int l = 0; fork && l < kLanes - 1 && e == cudaSuccess; ++l)
+            e = cudaStreamWaitEvent(c->lane[l], c->ev_fork, 0);
+          for (int tier = 0; tier < 2; ++tier)
+            for (int o = 0; o < kNumClasses && e == cudaSuccess; ++o) e = lane_lists(c0, c1, tier, kLaneOrder[o]);
+          for (int l = 0; fork && l < kLanes - 1; ++l) {  // join whatever was launched
+            const cudaError_t r = cudaEventRecord(c->ev_lane[l], c->lane[l]);
+            const cudaError_t w = cudaStreamWaitEvent(st, c->ev_lane[l], 0);
+            if (e == cudaSuccess) e = r != cudaSuccess ? r : w;
+          }
+          return e;
+        };
+        SNK_CK(c, lanes());
+        // the first group's first copy becomes the sum, later copies follow it
+        const int add = c1 - c0 + (c0 > 0);
+        if (add > 1) {
+          SNK_CK(c, launch_sum_copies(st, c->ws.p + ch.goff, ch.gn, add));
+          ++c->launches_build;
+        }
+      }
+      for (int k = 0; k < kNumLists; ++k) SNK_CK(c, mark());
     }
     // the operands of Kt_d += G_dj^T X_j, Eq. (usym_k)
     if (tc) {
@@ -1103,8 +1165,8 @@ int enqueue_build(snk_ctx* c, cudaStream_t st, double* dK, bool timed) {
       SNK_CK(c, oz_gemm(ch, 2));
     } else {
       for (int d = 0; d < nd; ++d) {
-        SNK_CK(c, launch_kgemm(st, db, nbc, ch.max_ldq, ch.max_nS, ch.max_nB, c->xfunc.p, c->sfunc.p, c->ws.p,
-                               c->Khat.p + 2 * d * pk, gmode, d, c->ozerr.p));
+        SNK_CK(c, launch_kgemm(st, db, nbc, ch.max_ldq, ch.max_nS, ch.max_nB, c->klen, c->xfunc.p, c->sfunc.p,
+                               c->ws.p, c->Khat.p + 2 * d * pk, gmode, d, c->ozerr.p));
         ++c->launches_build;
       }
     }
@@ -1667,6 +1729,9 @@ int build_vxc(snk_ctx* c, int fn, double* dV, double* E_host) {
       return rc == SNK_OK ? SNK_ERR_CUDA : rc;
     }
     c->xc_chunks = chunks;
+    int max_q = 0, max_nB = 0;
+    for (const BatchDesc& b : bd) max_q = std::max(max_q, b.ldq), max_nB = std::max(max_nB, b.nB);
+    c->xc_klen = point_split(nb, max_q, max_nB, max_nB);
     c->xc_gemm_flops = flops;
     c->xc_colloc_bytes = bytes;
   }
@@ -1705,7 +1770,8 @@ int build_vxc(snk_ctx* c, int fn, double* dV, double* E_host) {
     if (tc) {
       if (int rc = xc_tc_product(c, ch, 1, Vhat)) return rc;
     } else {
-      SNK_CK(c, launch_xc_vgemm(st, db, n, ch.max_ldq, ch.max_nB, c->xfunc.p, c->xcws.p, Vhat, mode, c->ozerr.p));
+      SNK_CK(c, launch_xc_vgemm(st, db, n, ch.max_ldq, ch.max_nB, c->xc_klen, c->xfunc.p, c->xcws.p, Vhat, mode,
+                                c->ozerr.p));
     }
     if (&ch == &c->xc_chunks.back()) SNK_CK(c, launch_xc_finish(st, c->mols.p, nm, pk, Vhat, Ehat, dV, c->xcE.p));
     SNK_CK(c, cudaEventRecord(c->xcev[ev++], st));
@@ -1980,6 +2046,7 @@ int snk_set_allocator(snk_ctx* c, snk_alloc_fn alloc, snk_free_fn free_fn, void*
   }
   c->graph_valid = false;
   c->have_density = false;
+  c->group_limit = 1 << 30;
   c->built = false;
   if (err != cudaSuccess) return cuda_fail(c, err, "snk_set_allocator: copying the handle's buffers");
   return SNK_OK;

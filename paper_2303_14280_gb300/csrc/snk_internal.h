@@ -23,8 +23,10 @@ constexpr int kLdqAlign = 128;   // leading-dimension padding of batch matrices
 // associative, so the sum of the batches' contributions does not depend on
 // the order in which they arrive (K is the same bit for bit from run to run).
 // A contribution v is cut as hi = rint(v 2^32), lo = rint((v - hi 2^-32) 2^76):
-// |v| < 2^30, |lo| <= 2^43 (sums of up to 2^19 batches stay below 2^62), and
-// what is dropped is below 2^-77 ~ 7e-24 per contribution.
+// |v| < 2^30, |lo| <= 2^43, and what is dropped is below 2^-77 ~ 7e-24 per
+// contribution.  A batch adds to an entry once, or once per block of its points where
+// point_split cuts them, which keeps the number of contributions below the number
+// of batches + 912: with up to 2^19 batches the sums of lo stay below 2^63.
 constexpr int kKhatMaxBatches = 1 << 19;
 constexpr int kErrKhatRange = 3;  // device error flag: a contribution outside |v| < 2^30
 #ifdef __CUDACC__
@@ -282,8 +284,11 @@ cudaError_t launch_pair_write(cudaStream_t st, const ScreenArgs& a, int nbatch, 
 cudaError_t launch_fgemm(cudaStream_t st, const BatchDesc* dbatch, int nbatch, int max_ldq, int max_nS,
                          const double* P, const float2* P2, const int* xfunc, const int* sfunc,
                          const double* fcomp, const double* w, double* ws, float* ws32, int mode, int dens);
+// Points per block of the products over a batch's points (K += G^T X, V-hat += Z^T X)
+// for all batches of a handle.
+int point_split(int nbatch, int max_q, int max_m, int max_n);
 cudaError_t launch_kgemm(cudaStream_t st, const BatchDesc* dbatch, int nbatch, int max_ldq, int max_nS, int max_nB,
-                         const int* xfunc, const int* sfunc, const double* ws, unsigned long long* Khat, int mode,
+                         int klen, const int* xfunc, const int* sfunc, const double* ws, unsigned long long* Khat, int mode,
                          int dens, int* err);
 // In place, each double of buf[0, n) becomes the float pair (fl32(v), fl32(v - fl32(v))).
 cudaError_t launch_split_df32(cudaStream_t st, double* buf, int64_t n);
@@ -309,8 +314,8 @@ cudaError_t launch_xc_fgemm(cudaStream_t st, const BatchDesc* dbatch, int nbatch
                             const double* P, const int* xfunc, double* ws, int mode);
 cudaError_t launch_xc_point(cudaStream_t st, const BatchDesc* dbatch, int nbatch, int max_ldq, const double* w,
                             int functional, double* ws, unsigned long long* Ehat, int* err);
-cudaError_t launch_xc_vgemm(cudaStream_t st, const BatchDesc* dbatch, int nbatch, int max_ldq, int max_nB, const int* xfunc,
-                            const double* ws, unsigned long long* Vhat, int mode, int* err);
+cudaError_t launch_xc_vgemm(cudaStream_t st, const BatchDesc* dbatch, int nbatch, int max_ldq, int max_nB, int klen,
+                            const int* xfunc, const double* ws, unsigned long long* Vhat, int mode, int* err);
 // V = V-hat + V-hat^T in every molecule block of the packed matrices, and
 // E[m] = E-hat of molecule m (two words per molecule).
 cudaError_t launch_xc_finish(cudaStream_t st, const MolDesc* mols, int n_mol, int64_t packed,
@@ -345,8 +350,9 @@ struct IntegralArgs {
   int hi_ds;
   int64_t gshift;  // this launch's copy of G: + gshift doubles from goff
   // FP64 / ds lists: a tile's list is cut into `parts` ranges, each adding into a
-  // copy of G of its own, gpart doubles after the one before
-  int parts;
+  // copy of G of its own; the launch runs the ranges [part0, part0 + part_n), their
+  // copies gpart doubles apart
+  int parts, part0, part_n;
   int64_t gpart;
   int n_dens;      // densities: F and G of density d at foff / goff (F32: foff32) + d ldq nS
   // tile screen of the FP32 lists (eps_tile > 0): a pair is skipped on a
