@@ -170,9 +170,11 @@ typedef struct {
   double ms_screen;            /* last set_density: upload, F-tilde, pair screen    */
   double ms_collocation, ms_fgemm, ms_integrals, ms_kgemm, ms_finish; /* last build  */
   double ms_build;             /* last build, first to last event                   */
-  double ms_integrals_class[6];/* per class ss ps pp ds dp dd (FP64 lists); builds small
-                                  enough to run all lists side by side report their
-                                  whole time in the first entry                      */
+  double ms_integrals_class[6];/* per class ss ps pp ds dp dd (FP64 lists).  Builds small
+                                  enough to run all lists side by side share the time
+                                  of the whole phase out to the lists of both tiers
+                                  (and ms_integrals, ms_integrals_fp32) by the time
+                                  each list ran on its own stream                   */
   double integrals_class[6];
   double flops_class[6];
   int64_t pairs_kept_fp32;     /* mixed form: kept (batch, pair) entries run in FP32 */

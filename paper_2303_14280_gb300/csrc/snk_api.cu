@@ -248,6 +248,12 @@ struct snk_ctx {
 
   // timing
   std::vector<cudaEvent_t> events;
+  // lists side by side: one list's launch ran between two events of its lane
+  struct LaneMark {
+    int chunk, list, from, to;
+  };
+  std::vector<cudaEvent_t> lane_events;
+  std::vector<LaneMark> lane_marks;
   cudaEvent_t ev_screen0 = nullptr, ev_screen1 = nullptr;
   int64_t launches_density = 0, launches_build = 0;
   bool built = false, built_graph = false;
@@ -283,6 +289,7 @@ struct snk_ctx {
     for (auto e : ev_lane)
       if (e) cudaEventDestroy(e);
     for (auto e : events) cudaEventDestroy(e);
+    for (auto e : lane_events) cudaEventDestroy(e);
     for (auto e : xcev) cudaEventDestroy(e);
     if (ev_screen0) cudaEventDestroy(ev_screen0);
     if (ev_screen1) cudaEventDestroy(ev_screen1);
@@ -396,11 +403,11 @@ int geometry_screen(snk_ctx* c) {
   return SNK_OK;
 }
 
-int ensure_events(snk_ctx* c, size_t n) {
-  while (c->events.size() < n) {
+int ensure_events(snk_ctx* c, std::vector<cudaEvent_t>& events, size_t n) {
+  while (events.size() < n) {
     cudaEvent_t e;
     SNK_CK(c, cudaEventCreate(&e));
-    c->events.push_back(e);
+    events.push_back(e);
   }
   return SNK_OK;
 }
@@ -1019,8 +1026,9 @@ int enqueue_build(snk_ctx* c, cudaStream_t st, double* dK, bool timed) {
   const int gmode = df32 ? 2 : 0;
   const int nd = c->n_dens;
   const int64_t pk = s.packed;
-  int ev = 0;
+  int ev = 0, lane_ev = 0;
   c->launches_build = 0;
+  c->lane_marks.clear();
   auto mark = [&]() -> cudaError_t { return timed ? cudaEventRecord(c->events[ev++], st) : cudaSuccess; };
   // one tensor-core product launch over a chunk's jobs of kind k (F hi, F lo, K hi, K lo)
   auto oz_gemm = [&](const snk_ctx::Chunk& ch, int k) -> cudaError_t {
@@ -1109,6 +1117,10 @@ int enqueue_build(snk_ctx* c, cudaStream_t st, double* dK, bool timed) {
       const int all = kLanes * c->parts;
       // the lists of one lane over the copies [c0, c1) of the group, each list in order; the
       // FP32 lists add into the lane's first copy
+      int last[kLanes];  // the event after which a lane's next list starts
+      auto lane_mark = [&](cudaStream_t sl) -> cudaError_t {
+        return timed ? cudaEventRecord(c->lane_events[lane_ev++], sl) : cudaSuccess;
+      };
       auto lane_lists = [&](int c0, int c1, int tier, int cls) -> cudaError_t {
         const int lane = kLaneOf[cls], k = tier * kNumClasses + cls;
         const int cl = c0 + (lane - c0 % kLanes + kLanes) % kLanes;  // the lane's first copy of the group
@@ -1120,7 +1132,15 @@ int enqueue_build(snk_ctx* c, cudaStream_t st, double* dK, bool timed) {
           a.part0 = cl / kLanes;
           a.part_n = (c1 - cl + kLanes - 1) / kLanes;
         }
-        return integrals(c->group > 1 && lane ? c->lane[lane - 1] : st, k, a);
+        if (a.n_tiles == 0) return cudaSuccess;
+        const cudaStream_t sl = c->group > 1 && lane ? c->lane[lane - 1] : st;
+        cudaError_t e = integrals(sl, k, a);
+        if (e == cudaSuccess) e = lane_mark(sl);
+        if (timed) {
+          c->lane_marks.push_back({(int)ci, k, last[lane], lane_ev - 1});
+          last[lane] = lane_ev - 1;
+        }
+        return e;
       };
       for (int c0 = 0; c0 < all; c0 += c->group) {
         const int c1 = std::min(c0 + c->group, all);
@@ -1131,7 +1151,9 @@ int enqueue_build(snk_ctx* c, cudaStream_t st, double* dK, bool timed) {
         // side by side: the lanes start after everything before and join before G is used
         auto lanes = [&]() -> cudaError_t {
           const bool fork = c->group > 1;
-          cudaError_t e = fork ? cudaEventRecord(c->ev_fork, st) : cudaSuccess;
+          cudaError_t e = lane_mark(st);
+          for (int& l : last) l = lane_ev - 1;
+          if (fork && e == cudaSuccess) e = cudaEventRecord(c->ev_fork, st);
           for (int l = 0; fork && l < kLanes - 1 && e == cudaSuccess; ++l)
             e = cudaStreamWaitEvent(c->lane[l], c->ev_fork, 0);
           for (int tier = 0; tier < 2; ++tier)
@@ -1151,7 +1173,8 @@ int enqueue_build(snk_ctx* c, cudaStream_t st, double* dK, bool timed) {
           ++c->launches_build;
         }
       }
-      for (int k = 0; k < kNumLists; ++k) SNK_CK(c, mark());
+      if (timed) ev += kNumLists - 1;  // one mark for all lists: their own times are in lane_marks
+      SNK_CK(c, mark());
     }
     // the operands of Kt_d += G_dj^T X_j, Eq. (usym_k)
     if (tc) {
@@ -1186,7 +1209,9 @@ int enqueue_build(snk_ctx* c, cudaStream_t st, double* dK, bool timed) {
 int build(snk_ctx* c, double* dK) {
   if (!c->have_density) return fail(c, SNK_ERR_BAD_STATE, "snk_build_K called before snk_set_density");
   if (!c->opt.graph || c->n_dens > 1) {
-    if (int rc = ensure_events(c, c->chunks.size() * kPhaseEvents + 2)) return rc;
+    if (int rc = ensure_events(c, c->events, c->chunks.size() * kPhaseEvents + 2)) return rc;
+    const size_t groups = c->group ? (kLanes * c->parts + c->group - 1) / c->group : 0;
+    if (int rc = ensure_events(c, c->lane_events, c->chunks.size() * groups * (kNumLists + 1))) return rc;
     if (int rc = enqueue_build(c, c->stream, dK, true)) return rc;
     c->built = true;
     c->built_graph = false;
@@ -1194,7 +1219,7 @@ int build(snk_ctx* c, double* dK) {
   }
   // CUDA-graph form: capture the whole build once per plan and output buffer,
   // replay it afterwards; ordered after / before the caller's stream by events
-  if (int rc = ensure_events(c, 2)) return rc;
+  if (int rc = ensure_events(c, c->events, 2)) return rc;
   if (!c->gstream) SNK_CK(c, cudaStreamCreateWithFlags(&c->gstream, cudaStreamNonBlocking));
   if (!c->ev_in) SNK_CK(c, cudaEventCreateWithFlags(&c->ev_in, cudaEventDisableTiming));
   if (!c->ev_out) SNK_CK(c, cudaEventCreateWithFlags(&c->ev_out, cudaEventDisableTiming));
@@ -1257,8 +1282,28 @@ void collect_times(snk_ctx* c) {
     st.ms_collocation += el(e0, e0 + 1);
     const double fs = el(e0 + 1, e0 + 2), fh = el(e0 + 2, e0 + 3), fl = el(e0 + 3, e0 + 4);
     st.ms_fgemm += fs + fh + fl;
+    // lists side by side: the phase's time, shared out by the time that every list
+    // ran on its lane
+    double lt[kNumLists] = {0};
+    if (c->group) {
+      double sum = 0.0;
+      for (const auto& m : c->lane_marks)
+        if (m.chunk == (int)ci) {
+          float ms = 0.f;
+          cudaEventElapsedTime(&ms, c->lane_events[m.from], c->lane_events[m.to]);
+          lt[m.list] += ms;
+          sum += ms;
+        }
+      const double all = el(e0 + 4, e0 + 4 + kNumLists);
+      if (sum > 0.0)
+        for (double& t : lt) t *= all / sum;
+      else
+        lt[0] = all;
+    } else {
+      for (int k = 0; k < kNumLists; ++k) lt[k] = el(e0 + 4 + k, e0 + 5 + k);
+    }
     for (int k = 0; k < kNumLists; ++k) {
-      const double t = el(e0 + 4 + k, e0 + 5 + k);
+      const double t = lt[k];
       if (k < kNumClasses) {
         st.ms_integrals_class[k] += t;
         st.ms_integrals += t;
