@@ -29,8 +29,9 @@ For each class (l_a, l_b) with l_a >= l_b, l <= 2 this emits
   * ``prim``: one primitive pair's differences, added into the NM scalars M;
   * ``build``: the recursion from M to [e; 0, 0, 0] for l_a <= |e| <= L, L = l_a + l_b;
   * ``hrr``: the horizontal recursion (App. A, Eq. hrr) to the target block Xi_{ab};
-  * ``vrr``: the recursion for one primitive pair, as Eq. (vrr) states it, for the
-    exports of a single shell pair's block;
+  * ``vrr``: the recursion for one primitive pair, as Eq. (vrr) states it: the FP32
+    tier's pp, dp and dd, FP64 pairs of uncontracted shells, and the exports of a single
+    shell pair's block;
 
 as straight-line code on named registers, templated on the arithmetic type:
 double (FP64 path), float (FP32 pairs of the mixed form) and ds (double-FP32).
@@ -334,9 +335,9 @@ def main(out=sys.stdout):
         for s in bl:
             w("    " + s + "\n")
         w("  }\n")
-        w("  template <typename R>\n")
+        w("  template <typename R, typename A>\n")
         w("  __device__ static __forceinline__ void vrr(const R* S, R PAx, R PAy, R PAz, R PCx, R PCy, R PCz,\n")
-        w("                                             R k1, R k2, R k3, R* acc) {\n")
+        w("                                             R k1, R k2, R k3, A* acc) {\n")
         w("    (void)PAx; (void)PAy; (void)PAz; (void)PCx; (void)PCy; (void)PCz; (void)k1; (void)k2; (void)k3;\n")
         for s in gen_vrr(la, lb):
             w("    " + s + "\n")

@@ -62,8 +62,9 @@ static_assert(kBoysTMax == 50.0, "kBoysTMaxBits encodes 50.0");
 // Taylor terms on |x| <= 0.05 and seeds with the prefactor: 24 atoms 176.0 ->
 // 168.8 ms per build, 4 atoms 0.780 -> 0.743 ms; largest error of a seed times its
 // prefactor 1.4e-15 -> 6.8e-16 relative, rms at most 2.0e-16 -> 1.5e-16.
+// With a prefactor (the recursion of a single primitive pair) every seed has it.
 template <int L>
-__device__ __forceinline__ void boys_seeds(double T, const double* tab, double* S) {
+__device__ __forceinline__ void boys_seeds(double T, const double* tab, double* S, double pref = 1.0) {
   if (__double_as_longlong(T) < kBoysTMaxBits) {
     // T in FP32 by integer operations: the conversion runs on the FP64 pipe (24
     // atoms, FP64 integrals 156.7 -> 155.6 ms)
@@ -75,7 +76,7 @@ __device__ __forceinline__ void boys_seeds(double T, const double* tab, double* 
     double f = row[kBoysTerms - 1];
 #pragma unroll
     for (int m = kBoysTerms - 2; m >= 0; --m) f = fma(f, x, row[m]);
-    S[L] = f;
+    S[L] = pref * f;
     if (L > 0) {
       // e^{-T} = e^{-T_k} e^{x}, e^{x} by its 8-term Taylor polynomial
       double e = 1.0 / 5040.0;
@@ -86,7 +87,7 @@ __device__ __forceinline__ void boys_seeds(double T, const double* tab, double* 
       e = fma(e, x, 0.5);
       e = fma(e, x, 1.0);
       e = fma(e, x, 1.0);
-      const double pe = row[kBoysTerms] * e;
+      const double pe = pref * (row[kBoysTerms] * e);
       // below 2^-1022 the sum is not 2T but as small, and e^{-T} = 1 beside it
       const double T2 = __hiloint2double(__double2hiint(T) + 0x00100000, __double2loint(T));
 #pragma unroll
@@ -94,7 +95,7 @@ __device__ __forceinline__ void boys_seeds(double T, const double* tab, double* 
     }
   } else {
     const double r = rsqrt(T);
-    S[0] = 0.88622692545275801365 * r;  // sqrt(pi)/2
+    S[0] = pref * (0.88622692545275801365 * r);  // sqrt(pi)/2
     if (L > 0) {
       const double o = 0.5 * (r * r);
 #pragma unroll
@@ -103,6 +104,22 @@ __device__ __forceinline__ void boys_seeds(double T, const double* tab, double* 
   }
 }
 
+// Classes where a pair of uncontracted shells runs the recursion for its one
+// primitive pair (the pair is the same for the whole block): contracting one pair
+// first costs dd 342 operations instead of 259, dp 134 instead of 110, pp 51 instead
+// of 46; from two primitive pairs on it is the cheaper form.  Uncontracted shells,
+// 36 atoms, 288,000 points, ms per build without / with: d alone 246.2 / 200.4, p
+// alone 50.5 / 47.1, p and d 312.8 / 272.5, s, p and d 349.8 / 324.2; contracted s
+// and p with one d primitive 221.6 / 218.2.
+template <int LA, int LB>
+constexpr bool kOneByRecursion = LA + LB >= 2 && LB > 0;
+
+// The sum of one term (0 + x is an addition to the compiler).
+struct OnlyTerm {
+  double v;
+  __device__ __forceinline__ void operator+=(double x) { v = x; }
+};
+
 // Contracted Xi_ab (no component factors) of one pair at the point (cx, cy, cz);
 // A is the centre of shell a.
 template <int LA, int LB>
@@ -110,6 +127,20 @@ __device__ __forceinline__ void pair_xi(const PairHdr& h, const PrimPair* __rest
                                         const double* __restrict__ A, const double* tab, double cx, double cy,
                                         double cz, double* xi) {
   using C = OsClass<LA, LB>;
+  if (kOneByRecursion<LA, LB> && h.pp_n == 1) {
+    const PrimPair pp = prims[h.pp_off];
+    const double PCx = pp.Px - cx, PCy = pp.Py - cy, PCz = pp.Pz - cz;
+    const double T = pp.zeta * fma(PCx, PCx, fma(PCy, PCy, PCz * PCz));
+    double S[C::L + 1], acc[C::NACC];
+    boys_seeds<C::L>(T, tab, S, pp.pref);
+    OnlyTerm one[C::NACC];
+    const double kappa = pp.pref_far;
+    C::vrr(S, pp.Px - A[0], pp.Py - A[1], pp.Pz - A[2], PCx, PCy, PCz, kappa, 2.0 * kappa, 3.0 * kappa, one);
+#pragma unroll
+    for (int k = 0; k < C::NACC; ++k) acc[k] = one[k].v;
+    C::hrr(acc, h.ABx, h.ABy, h.ABz, xi);
+    return;
+  }
   double M[C::NM];
 #pragma unroll
   for (int k = 0; k < C::NM; ++k) M[k] = 0.0;

@@ -38,9 +38,9 @@ template <> struct OsClass<0, 0> {
     const R v000_000 = acc_get(M[0]);
     acc[0] = v000_000;
   }
-  template <typename R>
+  template <typename R, typename A>
   __device__ static __forceinline__ void vrr(const R* S, R PAx, R PAy, R PAz, R PCx, R PCy, R PCz,
-                                             R k1, R k2, R k3, R* acc) {
+                                             R k1, R k2, R k3, A* acc) {
     (void)PAx; (void)PAy; (void)PAz; (void)PCx; (void)PCy; (void)PCz; (void)k1; (void)k2; (void)k3;
     const R t000_0 = S[0];
     acc[0] += t000_0;
@@ -85,9 +85,9 @@ template <> struct OsClass<1, 0> {
     acc[1] = v010_000;
     acc[2] = v001_000;
   }
-  template <typename R>
+  template <typename R, typename A>
   __device__ static __forceinline__ void vrr(const R* S, R PAx, R PAy, R PAz, R PCx, R PCy, R PCz,
-                                             R k1, R k2, R k3, R* acc) {
+                                             R k1, R k2, R k3, A* acc) {
     (void)PAx; (void)PAy; (void)PAz; (void)PCx; (void)PCy; (void)PCz; (void)k1; (void)k2; (void)k3;
     const R t000_0 = S[0];
     const R t000_1 = S[1];
@@ -171,9 +171,9 @@ template <> struct OsClass<1, 1> {
     acc[7] = v011_000;
     acc[8] = v002_000;
   }
-  template <typename R>
+  template <typename R, typename A>
   __device__ static __forceinline__ void vrr(const R* S, R PAx, R PAy, R PAz, R PCx, R PCy, R PCz,
-                                             R k1, R k2, R k3, R* acc) {
+                                             R k1, R k2, R k3, A* acc) {
     (void)PAx; (void)PAy; (void)PAz; (void)PCx; (void)PCy; (void)PCz; (void)k1; (void)k2; (void)k3;
     const R t000_0 = S[0];
     const R t000_1 = S[1];
@@ -284,9 +284,9 @@ template <> struct OsClass<2, 0> {
     acc[4] = v011_000;
     acc[5] = v002_000;
   }
-  template <typename R>
+  template <typename R, typename A>
   __device__ static __forceinline__ void vrr(const R* S, R PAx, R PAy, R PAz, R PCx, R PCy, R PCz,
-                                             R k1, R k2, R k3, R* acc) {
+                                             R k1, R k2, R k3, A* acc) {
     (void)PAx; (void)PAy; (void)PAz; (void)PCx; (void)PCy; (void)PCz; (void)k1; (void)k2; (void)k3;
     const R t000_0 = S[0];
     const R t000_1 = S[1];
@@ -435,9 +435,9 @@ template <> struct OsClass<2, 1> {
     acc[14] = v012_000;
     acc[15] = v003_000;
   }
-  template <typename R>
+  template <typename R, typename A>
   __device__ static __forceinline__ void vrr(const R* S, R PAx, R PAy, R PAz, R PCx, R PCy, R PCz,
-                                             R k1, R k2, R k3, R* acc) {
+                                             R k1, R k2, R k3, A* acc) {
     (void)PAx; (void)PAy; (void)PAz; (void)PCx; (void)PCy; (void)PCz; (void)k1; (void)k2; (void)k3;
     const R t000_0 = S[0];
     const R t000_1 = S[1];
@@ -749,9 +749,9 @@ template <> struct OsClass<2, 2> {
     acc[29] = v013_000;
     acc[30] = v004_000;
   }
-  template <typename R>
+  template <typename R, typename A>
   __device__ static __forceinline__ void vrr(const R* S, R PAx, R PAy, R PAz, R PCx, R PCy, R PCz,
-                                             R k1, R k2, R k3, R* acc) {
+                                             R k1, R k2, R k3, A* acc) {
     (void)PAx; (void)PAy; (void)PAz; (void)PCx; (void)PCy; (void)PCz; (void)k1; (void)k2; (void)k3;
     const R t000_0 = S[0];
     const R t000_1 = S[1];

@@ -1522,8 +1522,10 @@ int create(int n_mol, const snk_basis* bases, const snk_grid* grids, const snk_o
          exp_table_fill(et.data());
          SNK_CK(cp, upload(cp->exptab, et, st));
          SNK_CK(cp, upload(cp->pairs, s.pairs, st));
-         // the FP64 kernels' copy: the prefactor in the contraction coefficients
+         // the FP64 kernels' copy: the prefactor in the contraction coefficients, and in
+         // place of the large-T seed, which they form themselves, kappa alone
          std::vector<PrimPair> p64(s.prims);
+         for (PrimPair& P : p64) P.pref_far = P.c01;
          for (PrimPair& P : p64)
            for (double* v : {&P.c10, &P.c20, &P.c30, &P.c40, &P.c01, &P.c11, &P.c21, &P.c02}) *v *= P.pref;
          SNK_CK(cp, upload(cp->prims, p64, st));

@@ -102,7 +102,7 @@ struct PrimPair {
   double zeta;          // zeta_a + zeta_b
   double Px, Py, Pz;    // Gaussian product centre R_p
   double pref;          // 2 pi / zeta * exp(-zeta_a zeta_b |AB|^2 / zeta) * d_a d_b
-  double pref_far;      // pref * sqrt(pi) / 2  (large-T seed)
+  double pref_far;      // pref * sqrt(pi) / 2  (large-T seed); the FP64 kernels' copy: kappa
   double c10, c20, c30, c40;  // sigma^i, sigma = zeta_b / zeta (R_p - R_a = -sigma (R_a - R_b))
   double c01, c11, c21, c02;  // sigma^i kappa^j, kappa = 1 / (2 zeta)
                               // (all eight times pref in the FP64 kernels' copy)
