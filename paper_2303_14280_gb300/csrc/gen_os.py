@@ -148,6 +148,7 @@ def gen_vrr(la, lb):
         stack += [(m, n), (m, n + 1)]
         if m[q] > 0:
             stack += [(minus(m, q), n), (minus(m, q), n + 1)]
+    c = Counter()
     lines = []
     for (e, n) in sorted(need, key=lambda x: (sum(x[0]), -x[0][0], -x[0][1], x[1])):
         v = f"t{name_e(e)}_{n}"
@@ -158,13 +159,18 @@ def gen_vrr(la, lb):
         Q = "xyz"[q]
         m = minus(e, q)
         base = f"fma(PA{Q}, t{name_e(m)}_{n}, -PC{Q} * t{name_e(m)}_{n + 1})"
+        c.fma += 1
+        c.mul += 1
         if m[q] > 0:
+            c.fma += 1
+            c.add += 1
             mm = name_e(minus(m, q))
             base = f"fma(k{m[q]}, t{mm}_{n} - t{mm}_{n + 1}, {base})"
         lines.append(f"const R {v} = {base};")
     for k, (e, _) in enumerate(targets):
         lines.append(f"acc[{k}] += t{name_e(e)}_0;")
-    return lines
+        c.add += 1
+    return lines, c
 
 
 def build_nodes(la, lb, dirs):
@@ -311,6 +317,7 @@ def main(out=sys.stdout):
             if best is None or hc.ops < best[1].ops:
                 best = (hl, hc)
         hl, hc = best
+        vl, vc = gen_vrr(la, lb)
         L = la + lb
         w(f"// class ({la},{lb}): {pc.ops} operations ({pc.flops} flops) per primitive pair,\n")
         w(f"// {bc.ops + hc.ops} ({bc.flops + hc.flops} flops) per contracted pair\n")
@@ -322,6 +329,8 @@ def main(out=sys.stdout):
         w(f"  static constexpr int NB = {ncart(lb)};\n")
         w(f"  static constexpr int PRIM_FLOPS = {pc.flops};\n")
         w(f"  static constexpr int PAIR_FLOPS = {bc.flops + hc.flops};\n")
+        w(f"  static constexpr int VRR_FLOPS = {vc.flops};\n")
+        w(f"  static constexpr int HRR_FLOPS = {hc.flops};\n")
         w("  template <typename R, typename A>\n")
         w("  __device__ static __forceinline__ void prim(const R* S, const OsCoef<R>& c, A* M) {\n")
         w("    (void)c;\n")
@@ -339,7 +348,7 @@ def main(out=sys.stdout):
         w("  __device__ static __forceinline__ void vrr(const R* S, R PAx, R PAy, R PAz, R PCx, R PCy, R PCz,\n")
         w("                                             R k1, R k2, R k3, A* acc) {\n")
         w("    (void)PAx; (void)PAy; (void)PAz; (void)PCx; (void)PCy; (void)PCz; (void)k1; (void)k2; (void)k3;\n")
-        for s in gen_vrr(la, lb):
+        for s in vl:
             w("    " + s + "\n")
         w("  }\n")
         w("  template <typename R>\n")

@@ -1257,22 +1257,26 @@ cudaError_t launch_debug_boys(cudaStream_t st, const double* boys, int64_t n, co
   return cudaGetLastError();
 }
 
-// Algorithmic FP64 flops per (grid point, contracted shell pair), FMA = 2:
-// per primitive pair the T evaluation (8), the Boys seeds counted at the
-// cheaper large-T form (1 for L = 0, else 3 + 2L; the library rsqrt is not
-// counted) and the generated contraction into the scalars; per contracted pair
-// the generated VRR and HRR and the G_a contraction (2 NA NB).  The G_b half of off-diagonal pairs is not counted.
-void class_flops(int cls, double* per_prim, double* per_pair) {
+// Algorithmic flops per (grid point, contracted shell pair), FMA = 2: per primitive
+// pair the T evaluation (8), the Boys seeds counted at the cheaper large-T form (1
+// for L = 0, else 3 + 2L; the library rsqrt is not counted) and what the tier's form
+// does for it, the contraction into the scalars or (FP32 tier but for ps and ds) the
+// whole recursion; per contracted pair the rest, VRR and HRR or HRR alone, and the G_a
+// contraction (2 NA NB).  FP64 pairs of uncontracted shells count like the others.
+// The G_b half of off-diagonal pairs is not counted.
+void class_flops(int cls, bool f32, double* per_prim, double* per_pair) {
   int prim = 0, pair = 0, L = 0, na = 1, nb = 1;
   switch (cls) {
-#define SNK_CASE(c, A, B)          \
-  case c:                          \
-    prim = OsClass<A, B>::PRIM_FLOPS; \
-    pair = OsClass<A, B>::PAIR_FLOPS; \
-    L = OsClass<A, B>::L;           \
-    na = OsClass<A, B>::NA;         \
-    nb = OsClass<A, B>::NB;         \
-    break;
+#define SNK_CASE(c, A, B)                                                                   \
+  case c: {                                                                                 \
+    const bool first = !f32 || f32_early(A, B);                                             \
+    prim = first ? OsClass<A, B>::PRIM_FLOPS : OsClass<A, B>::VRR_FLOPS;                    \
+    pair = first ? OsClass<A, B>::PAIR_FLOPS : OsClass<A, B>::HRR_FLOPS;                    \
+    L = OsClass<A, B>::L;                                                                   \
+    na = OsClass<A, B>::NA;                                                                 \
+    nb = OsClass<A, B>::NB;                                                                 \
+    break;                                                                                  \
+  }
     SNK_CASE(0, 0, 0)
     SNK_CASE(1, 1, 0)
     SNK_CASE(2, 1, 1)

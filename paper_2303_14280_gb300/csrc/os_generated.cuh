@@ -25,6 +25,8 @@ template <> struct OsClass<0, 0> {
   static constexpr int NB = 1;
   static constexpr int PRIM_FLOPS = 1;
   static constexpr int PAIR_FLOPS = 0;
+  static constexpr int VRR_FLOPS = 1;
+  static constexpr int HRR_FLOPS = 0;
   template <typename R, typename A>
   __device__ static __forceinline__ void prim(const R* S, const OsCoef<R>& c, A* M) {
     (void)c;
@@ -63,6 +65,8 @@ template <> struct OsClass<1, 0> {
   static constexpr int NB = 1;
   static constexpr int PRIM_FLOPS = 4;
   static constexpr int PAIR_FLOPS = 9;
+  static constexpr int VRR_FLOPS = 12;
+  static constexpr int HRR_FLOPS = 0;
   template <typename R, typename A>
   __device__ static __forceinline__ void prim(const R* S, const OsCoef<R>& c, A* M) {
     (void)c;
@@ -120,6 +124,8 @@ template <> struct OsClass<1, 1> {
   static constexpr int NB = 3;
   static constexpr int PRIM_FLOPS = 13;
   static constexpr int PAIR_FLOPS = 66;
+  static constexpr int VRR_FLOPS = 54;
+  static constexpr int HRR_FLOPS = 18;
   template <typename R, typename A>
   __device__ static __forceinline__ void prim(const R* S, const OsCoef<R>& c, A* M) {
     (void)c;
@@ -243,6 +249,8 @@ template <> struct OsClass<2, 0> {
   static constexpr int NB = 1;
   static constexpr int PRIM_FLOPS = 10;
   static constexpr int PAIR_FLOPS = 39;
+  static constexpr int VRR_FLOPS = 51;
+  static constexpr int HRR_FLOPS = 0;
   template <typename R, typename A>
   __device__ static __forceinline__ void prim(const R* S, const OsCoef<R>& c, A* M) {
     (void)c;
@@ -338,6 +346,8 @@ template <> struct OsClass<2, 1> {
   static constexpr int NB = 3;
   static constexpr int PRIM_FLOPS = 24;
   static constexpr int PAIR_FLOPS = 177;
+  static constexpr int VRR_FLOPS = 130;
+  static constexpr int HRR_FLOPS = 36;
   template <typename R, typename A>
   __device__ static __forceinline__ void prim(const R* S, const OsCoef<R>& c, A* M) {
     (void)c;
@@ -557,6 +567,8 @@ template <> struct OsClass<2, 2> {
   static constexpr int NB = 6;
   static constexpr int PRIM_FLOPS = 45;
   static constexpr int PAIR_FLOPS = 503;
+  static constexpr int VRR_FLOPS = 268;
+  static constexpr int HRR_FLOPS = 158;
   template <typename R, typename A>
   __device__ static __forceinline__ void prim(const R* S, const OsCoef<R>& c, A* M) {
     (void)c;

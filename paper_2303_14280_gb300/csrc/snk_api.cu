@@ -751,8 +751,8 @@ int screen_and_plan(snk_ctx* c) {
     if (!split) b.nS_hi = col;
   }
   // counts for the statistics: integrals and algorithmic flops per list
-  double per_prim[kNumClasses], per_pair[kNumClasses];
-  for (int k = 0; k < kNumClasses; ++k) class_flops(k, &per_prim[k], &per_pair[k]);
+  double per_prim[kNumLists], per_pair[kNumLists];
+  for (int k = 0; k < kNumLists; ++k) class_flops(k % kNumClasses, k >= kNumClasses, &per_prim[k], &per_pair[k]);
   double lint[kNumLists] = {0}, lflops[kNumLists] = {0}, gflops = 0.0, gflops_hi = 0.0, xbytes = 0.0;
   int64_t kept[2] = {0, 0}, pair_points = 0;
   double listed32 = 0.0;
@@ -765,7 +765,7 @@ int screen_and_plan(snk_ctx* c) {
       const int la = cls >= 3 ? 2 : (cls >= 1 ? 1 : 0), lb = cls - la * (la + 1) / 2;
       const double n = c->hcounts[(size_t)j * kNumLists + k], npp = (double)c->hpp[(size_t)j * kNumLists + k];
       lint[k] += n * bd[j].q * ncart(la) * ncart(lb);
-      lflops[k] += (npp * per_prim[cls] + n * per_pair[cls]) * bd[j].q;
+      lflops[k] += (npp * per_prim[k] + n * per_pair[k]) * bd[j].q;
       kept[k >= kNumClasses] += (int64_t)n;
       pair_points += (int64_t)n * bd[j].q;
       if (k >= kNumClasses) listed32 += n * bd[j].q;
@@ -1329,7 +1329,7 @@ void collect_times(snk_ctx* c) {
     for (int k = kNumClasses; k < kNumLists; ++k) {
       double per_prim, per_pair;
       const int cls = k - kNumClasses;
-      class_flops(cls, &per_prim, &per_pair);
+      class_flops(cls, true, &per_prim, &per_pair);
       const int la = cls >= 3 ? 2 : (cls >= 1 ? 1 : 0), lb = cls - la * (la + 1) / 2;
       fl += (double)hx[2 * k] * per_prim + (double)hx[2 * k + 1] * per_pair;
       in += (double)hx[2 * k + 1] * ncart(la) * ncart(lb);

@@ -380,7 +380,7 @@ cudaError_t launch_debug_boys(cudaStream_t st, const double* boys, int64_t n, co
 
 // Algorithmic flops of the integral kernel per class and grid point: per
 // primitive pair and per contracted pair (from the generator's counts).
-void class_flops(int cls, double* per_prim, double* per_pair);
+void class_flops(int cls, bool f32, double* per_prim, double* per_pair);
 
 // Tiles of every (batch, list): ceil(count / run) runs x ceil(q / 128) slabs,
 // the (batch, list)'s tiles from tiles[tstart[batch * kNumLists + list]] on.
