@@ -812,8 +812,10 @@ int screen_and_plan(snk_ctx* c) {
     c->parts = 1;
     c->group = 0;
     if (tiles <= (int64_t)kLaneTiles * c->num_sms) {
-      c->parts = (int)std::min<int64_t>(kMaxParts, kPartItems * (int64_t)c->num_sms / std::max<int64_t>(tiles, 1));
-      c->parts = std::max(c->parts, 1);
+      // ranges only where there are FP64 / ds pairs: the FP32 lists are not cut
+      if (kept[0] > 0)
+        c->parts = std::max(1, (int)std::min<int64_t>(kMaxParts, kPartItems * (int64_t)c->num_sms /
+                                                                     std::max<int64_t>(tiles, 1)));
       // the largest group that fits the workspace cap in one chunk; else groups of one
       // range in smaller chunks, or single copies where even a batch is too large for that
       c->group = worst <= c->ws_budget ? kLanes : 1;

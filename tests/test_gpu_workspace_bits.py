@@ -92,3 +92,19 @@ def test_refused_plans_keep_the_bits_and_are_not_tried_again():
         eng.set_density(p.P)
         assert len(refused) == n and np.array_equal(np.asarray(eng.build_K()), K)
         eng.close()
+
+
+def test_no_copies_for_lists_without_pairs():
+    """With every pair in the FP32 tier the copies of G for ranges of the FP64 lists
+    would stay zero: the workspace holds one per lane (3), not up to 24 (about a fifth
+    of the FP64 form's doubles; half is allowed for X and the FP32 copy of F)."""
+    _, snk = _snk()
+    p = synth.cluster(4, 44, n_r=20, n_theta=4, n_phi=9, n_occ=4)
+    held = {}
+    for name, opts in (("fp64", dict()), ("fp32", dict(eps_E=0.0, eps_K=0.0, precision="mixed", fp32_bound=1e30))):
+        eng = snk.Engine(p.basis, p.grid, batch_max=200, **opts)
+        eng.set_density(p.P)
+        eng.build_K()
+        held[name] = eng.stats()["workspace_bytes"]
+        eng.close()
+    assert held["fp32"] < 0.5 * held["fp64"]
