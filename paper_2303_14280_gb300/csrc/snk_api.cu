@@ -2539,10 +2539,10 @@ int snk_mlp_grad(const float* weights, const float* features, const float* label
   if (launch_mlp_grad(0, dw, dx, dy, nullptr, n, under_weight, f32(3), f32(4),
                       reinterpret_cast<double*>(all.p + off[6]), dg, dg + kMlpWeights) != cudaSuccess)
     return SNK_ERR_CUDA;
-  std::vector<float> h(kMlpWeights + 1);
-  if (cudaMemcpy(h.data(), dg, sizes[5], cudaMemcpyDeviceToHost)) return SNK_ERR_CUDA;
-  std::copy(h.begin(), h.end() - 1, grad);
-  *loss = h.back();
+  float h[kMlpWeights + 1];  // 38 KB; nothing here allocates host memory, which could throw
+  if (cudaMemcpy(h, dg, sizes[5], cudaMemcpyDeviceToHost)) return SNK_ERR_CUDA;
+  std::copy(h, h + kMlpWeights, grad);
+  *loss = h[kMlpWeights];
   return SNK_OK;
 }
 
