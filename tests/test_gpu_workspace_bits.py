@@ -108,3 +108,31 @@ def test_no_copies_for_lists_without_pairs():
         held[name] = eng.stats()["workspace_bytes"]
         eng.close()
     assert held["fp32"] < 0.5 * held["fp64"]
+
+
+@pytest.mark.parametrize("kw", [dict(), dict(graph=1), dict(share=0.3), dict(share=0.05, graph=1)])
+def test_learned_screen_side_by_side(kw):
+    """The learned screen rewrites the lists before they are cut: the same bits with all
+    copies, in a graph, and group by group; two densities loaded one after another."""
+    _, snk = _snk()
+    p = synth.cluster(9, 49, n_r=20, n_theta=4, n_phi=9, n_occ=5)
+    w, skip, meta = snk.trained_screen()
+    opts = dict(FORMS["mixed_split"], screen="learned", learned_skip=skip, learned_fp32=meta["fp32_threshold"])
+
+    def build(**kw):
+        eng = snk.Engine(p.basis, p.grid, batch_max=200, **opts, **kw)
+        eng.screen_load(w)
+        K = []
+        for P in (p.P, 0.01 * p.P, p.P):
+            eng.set_density(P)
+            K.append(np.asarray(eng.build_K()).copy())
+        st = eng.stats()
+        eng.close()
+        return K, st
+
+    K, st = build()
+    assert st["pairs_learned_skipped"] > 0 and np.array_equal(K[0], K[2])
+    kw = dict(kw)
+    if "share" in kw:
+        kw["workspace_bytes"] = int(kw.pop("share") * st["workspace_bytes"])
+    assert all(np.array_equal(a, b) for a, b in zip(build(**kw)[0], K))
