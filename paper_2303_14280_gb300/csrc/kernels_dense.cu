@@ -145,16 +145,16 @@ __device__ __forceinline__ void gemm_tile(int m0, int n0, int mdim, int ndim, in
 // error-free TwoSum and everything else into the compensation c.  Twelve FP32
 // operations per multiply-add on the FP32 pipe (64x the FP64 issue rate on
 // GB300), relative error ~k 2^-46 for a length-k sum of same-sign terms.
-__device__ __forceinline__ float2 df32_split(double v) {
-  const float hi = __double2float_rn(v);
-  return make_float2(hi, __double2float_rn(v - (double)hi));
-}
-
 //
 // Two columns at once in packed arithmetic (half the issue slots; the scalar
 // form ran at 0.46 of the FP32 pipe's rate): products of a 17-atom build (102,000
 // points, 165 functions) 3.58 -> 2.83 ms.  nah = -ah: the product is formed as
 // m = -ah bh, so that its error is one packed fma and needs no negation.
+__device__ __forceinline__ float2 df32_split(double v) {
+  const float hi = __double2float_rn(v);
+  return make_float2(hi, __double2float_rn(v - (double)hi));
+}
+
 __device__ __forceinline__ void df32_mac(f2 ah, f2 nah, f2 al, f2 bh, f2 bl, f2& s, f2& c) {
   const f2 m = nah * bh;  // -p
   f2 e = fma(ah, bh, m);

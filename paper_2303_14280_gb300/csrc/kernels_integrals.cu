@@ -326,7 +326,8 @@ __device__ __forceinline__ void boys_seeds_f32(f2 nT, f2 pref, f2 pref_far, uint
 
 // The FP64 value of v by integer operations: the conversion instruction runs on
 // the FP64 pipe (2 lanes per clock and SM), which the G updates kept 20-35 %
-// busy.  Magnitudes below 2^-126 give zero; infinities and NaN stay what they are.
+// busy.  Magnitudes below 2^-126 give zero: such a term of G cannot reach K, whose
+// accumulator resolves 2^-76.  Infinities and NaN stay what they are.
 __device__ __forceinline__ double f32_to_f64_bits(float v) {
   const uint32_t b = __float_as_uint(v), m = b & 0x7fffffffu;
   uint32_t hi = (b & 0x80000000u) | ((m >> 3) + 0x38000000u);
@@ -373,7 +374,8 @@ __device__ __forceinline__ double f32_to_f64_bits(float v) {
 // bounds it now is latency (IPC 0.5 per scheduler, fixed-latency and shared-
 // memory waits): two points double the registers, so half as many warps fit.
 constexpr int kF32Threads = kPointTile / 2;
-// CTAs per SM asked of the compiler.  96 atoms and 768,000 points, ms per build
+// CTAs per SM asked of the compiler, chosen with one density (with two, dp spills 152
+// bytes, ps 64, pp 32 and ss 12 under it).  96 atoms and 768,000 points, ms per build
 // without / with: ss 30.5 / 29.1, ps 75.9 / 72.5, pp 65.8 / 60.1, dp 107 / 95; ds
 // and dd lose (47.3 / 48.8 in ds).
 constexpr int f32_min_ctas(int la, int lb) {

@@ -94,9 +94,8 @@ struct DevBuf {
   }
 };
 
-// pairs per integral tile for each class (cheap classes take longer runs);
-// the autotuner replaces these per list
-constexpr int kDefaultStep = kMaxPairsPerStep;  // pairs staged per step of the FP32 kernel, before autotuning
+// pairs the FP32 kernel stages per step; the autotuner replaces it per list
+constexpr int kDefaultStep = kMaxPairsPerStep;
 // Builds with few tiles run their pair lists side by side on three streams
 // ("lanes"), each adding into a G of its own.  A list's launch lasts at least the
 // latency of one warp walking the list, and ends with the SMs that got one tile
@@ -106,27 +105,30 @@ constexpr int kDefaultStep = kMaxPairsPerStep;  // pairs staged per step of the 
 // from run to run.  Which list range adds into which copy follows from the work
 // alone; with less memory fewer copies are held at a time (snk_ctx::group) and
 // filled group after group in the same order, so K does not depend on the
-// workspace.  Measured, lists one after another / side by side (tiles of
-// 128 points per SM in brackets): 17 atoms double-FP32 (5.4) 41.7 / 28.1 ms, 12
-// atoms mixed (3.2) 10.4 / 7.2, 24 atoms FP64 (3.8) 190 / 175, 4 atoms FP64 (0.6)
-// 1.23 / 1.13, 32 atoms mixed (13.5) 66.0 / 61.0; 24 molecules (30) 42.1 / 41.4 and 96
-// atoms mixed (39) 677 / 667 would pay two more copies of G (10 GB at 96 atoms) for
-// 1.5 %.  The line lies at kLaneTiles.  Six lanes are no better than three (17 atoms
-// 28.9, 12 atoms 7.7, 16 atoms with two densities 14.5 against 15.0).
+// workspace.  Measured, density load and build, lists one after another / side by
+// side in ranges (tiles of 128 points per SM in brackets): 4 atoms FP64 (0.6) 1.04 /
+// 0.673 ms, 12 atoms mixed (3.2) 9.87 / 6.15, 24 atoms FP64 (3.8) 177.4 / 158.8, 16
+// atoms with two densities (4.2) 22.4 / 16.1, 17 atoms double-FP32 (5.4) 41.9 / 26.9, 32
+// atoms mixed (13.5) 65.9 / 59.8; 24 molecules (30) 40.7 / 40.1 and 96 atoms mixed (39)
+// 624 / 613 would pay two more copies of G (10 GB at 96 atoms) for 1.5 %.  The line lies
+// at kLaneTiles.  Six lanes were no better than three when they were tried without
+// ranges (17 atoms 28.9 against 28.1, 12 atoms 7.7 / 7.2, two densities 14.5 / 15.0).
 constexpr int kLanes = 3;
 constexpr int kLaneTiles = 16;  // 128-point tiles per SM
 // The FP64 / double-FP32 lists are also cut into ranges, up to kMaxParts, as long as
 // a lane then has at most kPartItems work items per SM: a warp's time is the latency
 // of its range (an FP64 multiply-add takes about 60 clocks), and a launch ends with
-// the SMs whose last items started late.  ms per build at 3 / 8 / 16 / 28 items (copies
-// of G kLanes x ranges): 4 atoms FP64 (0.6 tiles) 0.744 / 0.702 / 0.710 / 0.705, 12 atoms
-// mixed (3.2) 7.10 / 6.35 / 6.42 / 6.62, 17 atoms double-FP32 (5.4) 27.4 / 27.2 / 26.7 /
-// 26.4, 24 atoms FP64 (3.8) 165.2 / 160.8 / 158.8 / 158.0, 16 atoms with two densities
-// 14.9 / 14.9 / 14.7 / 15.3; beyond it the copies' clearing and sum cost what the shorter
-// ranges give.
+// the SMs whose last items started late.  ms per build at 3 / 8 / 12 / 16 / 28 items
+// (copies of G kLanes x ranges): 4 atoms FP64 (0.6 tiles) 0.719 / 0.673 / 0.673 / 0.675 /
+// 0.672, 12 atoms mixed (3.2) 6.78 / 6.15 / 6.15 / 6.24 / 6.44, 24 atoms FP64 (3.8) 164.2 /
+// 160.0 / 158.8 / 157.7 / 156.6, 16 atoms with two densities (4.2) 16.8 / 16.8 / 16.1 /
+// 16.3 / 16.9, 17 atoms double-FP32 (5.4) 27.6 / 27.6 / 26.9 / 26.9 / 26.7.  12 is best or
+// within 1.4 % in all; beyond it the copies' clearing and sum cost the mixed forms what the
+// shorter ranges give.
 constexpr int kMaxParts = 8;
 constexpr int kPartItems = 12;
-constexpr int kLaneOf[kNumClasses] = {0, 1, 2, 2, 1, 0};     // ss ps pp ds dp dd: about equal work per lane
+constexpr int kLaneOf[kNumClasses] = {0, 1, 2, 2, 1, 0};     // ss ps pp ds dp dd: about equal work per
+                                                           // lane in the 24-atom cluster's basis
 constexpr int kLaneOrder[kNumClasses] = {5, 4, 3, 0, 1, 2};  // heavier list of every lane first
 constexpr int kRunCandidates[] = {2, 4, 8, 16, 32, 64};
 // per chunk: collocation, F operands, F high tier, F rest, integral lists, K operands, K high tier, K rest

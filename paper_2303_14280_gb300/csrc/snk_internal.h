@@ -293,9 +293,9 @@ cudaError_t launch_kgemm(cudaStream_t st, const BatchDesc* dbatch, int nbatch, i
 // In place, each double of buf[0, n) becomes the float pair (fl32(v), fl32(v - fl32(v))).
 cudaError_t launch_split_df32(cudaStream_t st, double* buf, int64_t n);
 cudaError_t launch_split_df32_copy(cudaStream_t st, const double* src, int64_t n, float2* dst);
-// out = sum_d |P_d| over n_dens consecutive arrays of n doubles.
 // g[e] = (g[e] + g[e + n]) + g[e + 2n] ... over `copies` copies of n doubles (n even)
 cudaError_t launch_sum_copies(cudaStream_t st, double* g, int64_t n, int copies);
+// out = sum_d |P_d| over n_dens consecutive arrays of n doubles.
 cudaError_t launch_abs_sum(cudaStream_t st, const double* P, int n_dens, int64_t n, double* out);
 cudaError_t launch_finish(cudaStream_t st, const MolDesc* mols, int n_mol, int64_t packed,
                           const unsigned long long* Khat, const double* fcomp, double* K);
