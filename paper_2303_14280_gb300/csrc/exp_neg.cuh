@@ -1,11 +1,12 @@
-// e^{-x} for 0 <= x < 700 in FP64 with ten FP64 operations, by the table-driven
+// e^{-x} for 0 <= x < 700 in FP64 with nine FP64 operations, by the table-driven
 // method (P. T. P. Tang, ACM Trans. Math. Softw. 15, 144, 1989): x = k ln2/256 +
 // r with |r| <= ln2/512, e^{-x} = 2^{-k/256} e^{-r}; 2^{-j/256}, j < 256, comes from a
-// table in shared memory as head and tail, the remaining power of two goes into
-// the exponent bits, and e^{-r} - 1 is its Taylor polynomial of degree 4 (the next
-// term is below 4e-17).  ln2/256 is split into a 32-bit head, so that k head is
-// exact, and a tail.  Relative error at most 1.5e-16: the last addition's rounding
-// and the polynomial's truncation (2.4e-16 without the table's tail).
+// table in shared memory as the double T and its relative error t, the remaining
+// power of two goes into the exponent bits, and e^{-r} - 1 is its Taylor polynomial
+// of degree 4 (the next term is below 4e-17), to which t is added by the multiply-add
+// that would be its last multiplication.  ln2/256 is split into a 32-bit head, so that
+// k head is exact, and a tail.  Relative error at most 1.5e-16: the last rounding and
+// the polynomial's truncation (2.4e-16 without t).
 //
 // FP64 issues at 2 lanes per clock and SM on GB300, so the number of FP64
 // operations is what the collocation kernels cost.
@@ -19,12 +20,12 @@
 
 namespace snk {
 
-// 2^{-j/256} = tab[j].x + tab[j].y
+// 2^{-j/256} = tab[j].x (1 + tab[j].y)
 inline void exp_table_fill(double2* tab) {
   for (int j = 0; j < kExpTable; ++j) {
     const long double v = exp2l(-(long double)j / kExpTable);
     tab[j].x = (double)v;
-    tab[j].y = (double)(v - (long double)tab[j].x);
+    tab[j].y = (double)((v - (long double)tab[j].x) / v);
   }
 }
 
@@ -44,7 +45,7 @@ __device__ __forceinline__ double exp_neg(double x, const double2* tab) {
   q = fma(q, r, 0.5);
   q = fma(q, r, -1.0);
   const double2 T = tab[k & (kExpTable - 1)];
-  const double e = T.x + fma(T.x, q * r, T.y);
+  const double e = fma(T.x, fma(q, r, T.y), T.x);
   return __hiloint2double(__double2hiint(e) - ((k >> 8) << 20), __double2loint(e));
 }
 

@@ -47,7 +47,7 @@ constexpr double kPi = 3.14159265358979323846;
 
 // X and its gradient on the batch's points, shell by shell of B_j.  Bound by
 // the FP64 pipe (32 bytes are written per FP64 operation's 16 clocks), so what
-// counts is the operations: e^{-x} in ten (exp_neg), and with u = q R0 and t =
+// counts is the operations: e^{-x} in nine (exp_neg), and with u = q R0 and t =
 // q R1 for the three directions a p shell takes 15 and a d shell 45 operations
 // for its functions and their gradients, where the general monomial took 22
 // per function.  The shells come group by group (same centre, same exponents), and

@@ -229,7 +229,7 @@ void host_boys(int nmax, double T, double* F);
 
 struct DeviceBasis {
   const int* rgroup;     // shells of a group share centre and exponents (at most kRadialPrims of them)
-  const double2* exptab;  // 2^{-j/kExpTable} of exp_neg, head and tail
+  const double2* exptab;  // 2^{-j/kExpTable} of exp_neg and their relative errors
   const int* l;
   const int* poff;
   const int* nprim;

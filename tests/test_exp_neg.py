@@ -1,6 +1,6 @@
 """e^{-x} of the collocation kernels, on the host, against long double.
 
-Tolerance: the table holds 2^{-j/256} as head and tail, so what is left is the
+Tolerance: the table holds 2^{-j/256} and its relative error, so what is left is the
 rounding of the last addition, at most 2^-53, the polynomial's truncation, 4e-17, and
 roundings 2^-9 times smaller: 1.6e-16 relative.  With the head alone its own rounding
 comes on top, 2.4e-16."""
