@@ -1215,7 +1215,10 @@ int build(snk_ctx* c, double* dK) {
   if (!c->opt.graph || c->n_dens > 1) {
     if (int rc = ensure_events(c, c->events, c->chunks.size() * kPhaseEvents + 2)) return rc;
     const size_t groups = c->group ? (kLanes * c->parts + c->group - 1) / c->group : 0;
-    if (int rc = ensure_events(c, c->lane_events, c->chunks.size() * groups * (kNumLists + 1))) return rc;
+    // a mark per group and per list launch: a group has the FP64 lists of its lanes, the first
+    // copies the FP32 lists too
+    const size_t lists = kNumClasses * groups / (c->group == 1 ? kLanes : 1) + kNumClasses;
+    if (int rc = ensure_events(c, c->lane_events, c->group ? c->chunks.size() * (groups + lists) : 0)) return rc;
     if (int rc = enqueue_build(c, c->stream, dK, true)) return rc;
     c->built = true;
     c->built_graph = false;
